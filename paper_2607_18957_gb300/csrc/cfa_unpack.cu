@@ -37,10 +37,17 @@ using cfa_dev::warp_sum;
 constexpr int kThreads = 256;
 constexpr int kWarps = kThreads / 32;
 constexpr int kUnroll = 4;
-constexpr int kMinBlocks = 4;     /* conversion classes: 64 registers per thread at most */
+constexpr int kMinBlocks = 4;     /* the other conversion classes: 64 registers per thread */
 constexpr int kCopyMinBlocks = 3; /* 2-8-byte copy classes: 80 registers, room for the
                                      realigning path; the 1-byte class keeps 4 CTAs (its byte-wise
                                      checksum wants the warps: 0.96 vs 0.92 of the roofline) */
+constexpr int unpack_min_blocks(int cls)
+{
+    /* fp16 -> bf16 is a 16-bit copy with arithmetic: the copy classes' depth and occupancy
+     * (1.9 GB: 580 us at three CTAs per SM, 610 at four) */
+    return (cls >= 1 && cls < 4) || cls == CFA_CLASS_OF_CONV(CFA_CONV_F16_BF16) ? kCopyMinBlocks
+                                                                               : kMinBlocks;
+}
 /* Rounds of 32-vector loads in flight per warp on the realigning path: four for slabs (with
  * three CTAs per SM the copy kernels hold them without spilling; two for the 1-byte class at
  * four CTAs), two for column-slice rows. */
@@ -92,13 +99,20 @@ __device__ __forceinline__ void st_stream(void *p, uint4 v)
                  : "memory");
 }
 
+/* The same for 32 bytes (32-byte aligned): whole sectors. */
+__device__ __forceinline__ void st_stream32(void *p, uint4 a, uint4 b)
+{
+    asm volatile("st.global.cs.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(p), "r"(a.x),
+                 "r"(a.y), "r"(a.z), "r"(a.w), "r"(b.x), "r"(b.y), "r"(b.z), "r"(b.w)
+                 : "memory");
+}
+
 template <int ES> struct Elem;
 template <> struct Elem<1> { typedef uint8_t T; };
 template <> struct Elem<2> { typedef uint16_t T; };
 template <> struct Elem<4> { typedef uint32_t T; };
 template <> struct Elem<8> { typedef unsigned long long T; };
 
-/* Sum of the ES-byte little-endian integers in a 16-byte vector. */
 /* Bytes k .. k+15 of the 32-byte concatenation a:b (little-endian), 0 < k < 16. */
 __device__ __forceinline__ uint4 funnel16(uint4 a, uint4 b, uint32_t k)
 {
@@ -168,6 +182,107 @@ template <int CONV> __device__ __forceinline__ uint32_t convert1(uint32_t x)
     else return f16_to_f32(x);
 }
 
+/* ---- conversion of eight elements at once ------------------------------------------------
+ * One or two instructions per pair of elements, on packed words, with the hardware's conversion
+ * instructions; the NaN results that the format fixes differently (convert1) are put right
+ * afterwards.  With convert1's integer forms on every element the 16-bit classes were bound by
+ * instructions and divergent branches: fp16 -> bf16, 1.9 GB: 1170 us, now 580 (0.49 and 0.99 of
+ * the copy rate); fp32 -> fp16, 1.0 GB: 583, now 460 (0.78, 0.99).  convert1 serves a run's ends. */
+
+/* fp32 pair -> bf16 pair, round to nearest even.  The instruction's only NaN result is 0x7FFF; the
+ * signed minimum with 0x7FC0 turns it into the quiet NaN that convert1 gives and changes nothing
+ * else (every other positive result is at most 0x7F80). */
+__device__ __forceinline__ uint32_t bf16x2_of(float lo, float hi)
+{
+    uint32_t r;
+    asm("cvt.rn.bf16x2.f32 %0, %2, %1;" : "=r"(r) : "f"(lo), "f"(hi));
+    asm("min.s16x2 %0, %0, %1;" : "+r"(r) : "r"(0x7FC07FC0u));
+    return r;
+}
+
+__device__ __forceinline__ uint32_t f16x2_of(float lo, float hi)
+{
+    uint32_t r;
+    asm("cvt.rn.f16x2.f32 %0, %2, %1;" : "=r"(r) : "f"(lo), "f"(hi));
+    return r;
+}
+
+__device__ __forceinline__ void f32x2_of_f16x2(uint32_t w, float &lo, float &hi)
+{
+    asm("{\n\t.reg .f16 l, h;\n\tmov.b32 {l, h}, %2;\n\t"
+        "cvt.f32.f16 %0, l;\n\tcvt.f32.f16 %1, h;\n\t}"
+        : "=f"(lo), "=f"(hi)
+        : "r"(w));
+}
+
+__device__ __forceinline__ uint32_t max_s16x2(uint32_t a, uint32_t b)
+{
+    uint32_t r;
+    asm("max.s16x2 %0, %1, %2;" : "=r"(r) : "r"(a), "r"(b));
+    return r;
+}
+
+/* x: eight source elements as packed words (eight of 32 bits, or four of two 16-bit elements);
+ * y: the converted elements, packed the same way. */
+template <int CONV> __device__ __forceinline__ void convert8(const uint32_t *x, uint32_t *y)
+{
+    if constexpr (CONV == CFA_CONV_F32_BF16) {
+        /* fp32 -> bf16 is bound by DRAM with the integer form as well; with the packed instruction
+         * its loads and stores came closer together and the launch was 1-2 % slower (1.8 GB of
+         * bf16: 1570 against 1542 us) */
+#pragma unroll
+        for (int q = 0; q < 4; ++q) y[q] = bf16_rne(x[2 * q]) | (bf16_rne(x[2 * q + 1]) << 16);
+    } else if constexpr (CONV == CFA_CONV_F32_F16) {
+#pragma unroll
+        for (int q = 0; q < 4; ++q)
+            y[q] = f16x2_of(__uint_as_float(x[2 * q]), __uint_as_float(x[2 * q + 1]));
+        /* the instruction's only NaN result is 0x7FFF, the largest signed half; convert1 keeps
+         * the sign of a NaN */
+        const uint32_t m = max_s16x2(max_s16x2(y[0], y[1]), max_s16x2(y[2], y[3]));
+        if ((m & 0xFFFFu) == 0x7FFFu || (m >> 16) == 0x7FFFu) {
+#pragma unroll
+            for (int q = 0; q < 8; ++q)
+                if ((x[q] & 0x7FFFFFFFu) > 0x7F800000u) {
+                    const uint32_t h = ((x[q] >> 16) & 0x8000u) | 0x7E00u;
+                    y[q / 2] = (q & 1) ? (y[q / 2] & 0xFFFFu) | (h << 16)
+                                       : (y[q / 2] & 0xFFFF0000u) | h;
+                }
+        }
+    } else if constexpr (CONV == CFA_CONV_F16_BF16) {
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            float lo, hi;
+            f32x2_of_f16x2(x[q], lo, hi);
+            y[q] = bf16x2_of(lo, hi);
+        }
+    } else if constexpr (CONV == CFA_CONV_BF16_F32) {
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            y[2 * q] = x[q] << 16;
+            y[2 * q + 1] = x[q] & 0xFFFF0000u;
+        }
+    } else {
+        uint32_t m = 0; /* magnitudes stay below 0x8000: signed and unsigned maxima agree */
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            float lo, hi;
+            f32x2_of_f16x2(x[q], lo, hi);
+            y[2 * q] = __float_as_uint(lo);
+            y[2 * q + 1] = __float_as_uint(hi);
+            m = max_s16x2(m, x[q] & 0x7FFF7FFFu);
+        }
+        /* convert1 keeps a NaN's payload as it is; the instruction makes it quiet */
+        if ((m & 0xFFFFu) > 0x7C00u || (m >> 16) > 0x7C00u) {
+#pragma unroll
+            for (int q = 0; q < 8; ++q) {
+                const uint32_t h = (x[q / 2] >> (16 * (q & 1))) & 0xFFFFu;
+                if ((h & 0x7FFFu) > 0x7C00u)
+                    y[q] = ((h & 0x8000u) << 16) | 0x7F800000u | ((h & 0x3FFu) << 13);
+            }
+        }
+    }
+}
+
 /* Source element size, destination element size and conversion of a work class. */
 template <int CLS> struct ClassOf {
     static constexpr int conv = CLS >= 4 ? CLS - 3 : 0;
@@ -193,6 +308,61 @@ __device__ __forceinline__ uint64_t copy_elems(const uint8_t *src, uint8_t *dst,
         acc += (uint64_t)v;
     }
     return acc;
+}
+
+/* The realigning loop: for every i < nvec, sink(i, bytes k .. k + 15 of the aligned source vectors
+ * s[i] and s[i + 1]), 0 < k < 16.  Both vectors hold needed bytes, so nothing outside the run is
+ * read.  A group of W lanes (a warp, W = 32, or an 8-lane segment of one on the sub-warp path for
+ * tiny pieces, W = 8) takes UR * W consecutive vectors at a time (lane l, round u: vector
+ * w0 + W u + l) and loads each once; s[i + 1] comes by shuffle from the next lane, or for the
+ * group's last lane from lane 0 of the next round.  The one vector per group that has no loaded
+ * neighbour (the last lane's last one, or the run's last vector) is loaded by its lane in the
+ * same round of loads.  Every shuffle stays inside the group. */
+template <int UR, int W, typename Sink>
+__device__ __forceinline__ void realign_run(const uint4 *__restrict__ s, uint32_t k,
+                                            uint32_t nvec, uint32_t tid, uint32_t nthr,
+                                            const Sink &sink)
+{
+    const uint32_t lane = tid & (W - 1u), wid = tid / W;
+    const uint32_t mask =
+        W == 32 ? 0xFFFFFFFFu : (((1u << W) - 1u) << (threadIdx.x & 31u & ~(W - 1u)));
+    const uint32_t step = nthr * UR;
+    for (uint32_t base = 0; base < nvec; base += step) {
+        const uint32_t w0 = base + wid * W * UR;
+        uint4 a[UR];
+        int own = -1; /* the round whose neighbour this lane loads itself */
+#pragma unroll
+        for (int u = 0; u < UR; ++u) {
+            const uint32_t i = w0 + W * u + lane;
+            a[u] = make_uint4(0u, 0u, 0u, 0u);
+            if (i < nvec) {
+                a[u] = ld_shared_line(s + i);
+                if (i + 1 == nvec || (lane == W - 1u && u == UR - 1)) own = u;
+            }
+        }
+        uint4 c = make_uint4(0u, 0u, 0u, 0u);
+        if (own >= 0) c = ld_shared_line(s + w0 + W * own + lane + 1);
+#pragma unroll
+        for (int u = 0; u < UR; ++u) {
+            const uint32_t i = w0 + W * u + lane;
+            uint4 b, n0;
+            b.x = __shfl_down_sync(mask, a[u].x, 1, W);
+            b.y = __shfl_down_sync(mask, a[u].y, 1, W);
+            b.z = __shfl_down_sync(mask, a[u].z, 1, W);
+            b.w = __shfl_down_sync(mask, a[u].w, 1, W);
+            if (u + 1 < UR) {
+                n0.x = __shfl_sync(mask, a[u + 1].x, 0, W);
+                n0.y = __shfl_sync(mask, a[u + 1].y, 0, W);
+                n0.z = __shfl_sync(mask, a[u + 1].z, 0, W);
+                n0.w = __shfl_sync(mask, a[u + 1].w, 0, W);
+                if (lane == W - 1u) b = n0;
+            }
+            if (i < nvec) {
+                if (own == u) b = c;
+                sink(i, funnel16(a[u], b, k));
+            }
+        }
+    }
 }
 
 /* Copies nbytes (a multiple of ES) from src to dst; thread tid of nthr.  Returns this thread's
@@ -234,58 +404,11 @@ __device__ uint64_t copy_run(const uint8_t *__restrict__ src, uint8_t *__restric
             }
         }
     } else {
-        /* source off by k bytes: every 16-byte store takes bytes k..k+15 of two aligned
-         * vectors s[i] and s[i + 1], both of which hold needed bytes, so nothing outside the
-         * run is read.  A group of W lanes (a warp, W = 32, or an 8-lane segment of one on the
-         * sub-warp path for tiny pieces, W = 8) takes UR * W consecutive vectors at a time
-         * (lane l, round u: vector w0 + W u + l) and loads each once; s[i + 1] comes by shuffle
-         * from the next lane, or for the group's last lane from lane 0 of the next round.  The
-         * one vector per group that has no loaded neighbour (the last lane's last one, or the
-         * run's last vector) is loaded by its lane in the same round of loads.  Every shuffle
-         * stays inside the group. */
-        const uint4 *s = reinterpret_cast<const uint4 *>(src - k);
-        const uint32_t lane = tid & (W - 1u), wid = tid / W;
-        const uint32_t mask =
-            W == 32 ? 0xFFFFFFFFu : (((1u << W) - 1u) << (threadIdx.x & 31u & ~(W - 1u)));
-        const uint32_t step = nthr * UR;
-        for (uint32_t base = 0; base < nvec; base += step) {
-            const uint32_t w0 = base + wid * W * UR;
-            uint4 a[UR];
-            int own = -1; /* the round whose neighbour this lane loads itself */
-#pragma unroll
-            for (int u = 0; u < UR; ++u) {
-                const uint32_t i = w0 + W * u + lane;
-                a[u] = make_uint4(0u, 0u, 0u, 0u);
-                if (i < nvec) {
-                    a[u] = ld_shared_line(s + i);
-                    if (i + 1 == nvec || (lane == W - 1u && u == UR - 1)) own = u;
-                }
-            }
-            uint4 c = make_uint4(0u, 0u, 0u, 0u);
-            if (own >= 0) c = ld_shared_line(s + w0 + W * own + lane + 1);
-#pragma unroll
-            for (int u = 0; u < UR; ++u) {
-                const uint32_t i = w0 + W * u + lane;
-                uint4 b, n0;
-                b.x = __shfl_down_sync(mask, a[u].x, 1, W);
-                b.y = __shfl_down_sync(mask, a[u].y, 1, W);
-                b.z = __shfl_down_sync(mask, a[u].z, 1, W);
-                b.w = __shfl_down_sync(mask, a[u].w, 1, W);
-                if (u + 1 < UR) {
-                    n0.x = __shfl_sync(mask, a[u + 1].x, 0, W);
-                    n0.y = __shfl_sync(mask, a[u + 1].y, 0, W);
-                    n0.z = __shfl_sync(mask, a[u + 1].z, 0, W);
-                    n0.w = __shfl_sync(mask, a[u + 1].w, 0, W);
-                    if (lane == W - 1u) b = n0;
-                }
-                if (i < nvec) {
-                    if (own == u) b = c;
-                    const uint4 o = funnel16(a[u], b, k);
-                    st_stream(d + i, o);
-                    acc += vsum<ES>(o);
-                }
-            }
-        }
+        realign_run<UR, W>(reinterpret_cast<const uint4 *>(src - k), k, nvec, tid, nthr,
+                           [&](uint32_t i, const uint4 &o) {
+                               st_stream(d + i, o);
+                               acc += vsum<ES>(o);
+                           });
     }
     /* tail */
     const uint64_t body = (uint64_t)nvec << 4;
@@ -293,17 +416,21 @@ __device__ uint64_t copy_run(const uint8_t *__restrict__ src, uint8_t *__restric
     return acc;
 }
 
-/* n elements of SES bytes at src -> n converted elements of DES bytes at dst.  Destination
- * stores are 16 bytes wide; eight elements form a group (32 or 16 source bytes, 16 or 32
- * destination bytes), loaded as 16-byte vectors when the source is aligned, else one by one. */
-template <int SES, int DES, int CONV, int U>
+/* n elements of SES bytes at src -> n converted elements of DES bytes at dst.  Eight elements
+ * form a group (32 or 16 source bytes, 16 or 32 destination bytes), U of them in flight per
+ * thread; a group is one 16-byte store, or one 32-byte store for 32-bit results: with
+ * two 16-byte stores, 32 bytes apart from lane to lane, each store wrote half of every 32-byte
+ * sector (fp16 -> fp32, 4.5 GB written: 1243 us, now 1044; bf16 -> fp32 at odd 2-byte offsets,
+ * whose elements were loaded one by one: 1236, now 1053). */
+template <int SES, int DES, int CONV, int U, int UR, int W>
 __device__ uint64_t convert_run(const uint8_t *__restrict__ src, uint8_t *__restrict__ dst,
                                 uint64_t n, uint32_t tid, uint32_t nthr)
 {
     typedef typename Elem<SES>::T ST;
     typedef typename Elem<DES>::T DT;
+    constexpr uint32_t kAlign = 8 * DES; /* of a group's store */
     uint64_t acc = 0;
-    uint32_t h = (uint32_t)(((16u - ((uintptr_t)dst & 15u)) & 15u) / DES);
+    uint32_t h = (uint32_t)(((kAlign - ((uintptr_t)dst & (kAlign - 1u))) & (kAlign - 1u)) / DES);
     if (h > n) h = (uint32_t)n;
     for (uint32_t e = tid; e < h; e += nthr) {
         const uint32_t y = convert1<CONV>(reinterpret_cast<const ST *>(src)[e]);
@@ -315,70 +442,71 @@ __device__ uint64_t convert_run(const uint8_t *__restrict__ src, uint8_t *__rest
     n -= h;
 
     const uint32_t ng = (uint32_t)(n >> 3);
-    uint4 *d = reinterpret_cast<uint4 *>(dst);
-    const bool vec = ((uintptr_t)src & 15u) == 0;
-    const uint32_t step = nthr * U;
-    for (uint32_t base = 0; base < ng; base += step) {
-        uint32_t x[U][8];
-#pragma unroll
-        for (int u = 0; u < U; ++u) {
-            const uint32_t g = base + u * nthr + tid;
-            if (g >= ng) continue;
-            if (vec && SES == 4) {
-                const uint4 a = ld_stream(src + 32ull * g), b = ld_stream(src + 32ull * g + 16);
-                x[u][0] = a.x; x[u][1] = a.y; x[u][2] = a.z; x[u][3] = a.w;
-                x[u][4] = b.x; x[u][5] = b.y; x[u][6] = b.z; x[u][7] = b.w;
-            } else if (vec && SES == 2) {
-                const uint4 a = ld_stream(src + 16ull * g);
-                x[u][0] = a.x & 0xFFFFu; x[u][1] = a.x >> 16; x[u][2] = a.y & 0xFFFFu;
-                x[u][3] = a.y >> 16; x[u][4] = a.z & 0xFFFFu; x[u][5] = a.z >> 16;
-                x[u][6] = a.w & 0xFFFFu; x[u][7] = a.w >> 16;
-            } else if (SES == 4 && ((uintptr_t)src & 7u) == 0) {
-                /* 8-byte aligned: four 8-byte loads instead of eight 4-byte ones */
-                const uint2 *s2 = reinterpret_cast<const uint2 *>(src + 32ull * g);
-#pragma unroll
-                for (int q = 0; q < 4; ++q) {
-                    const uint2 v = __ldg(s2 + q);
-                    x[u][2 * q] = v.x;
-                    x[u][2 * q + 1] = v.y;
-                }
-            } else if (SES == 4) {
-                /* 4 mod 8: the first and last elements alone, the six between as 8-byte pairs */
-                const uint32_t *s1 = reinterpret_cast<const uint32_t *>(src + 32ull * g);
-                const uint2 *s2 = reinterpret_cast<const uint2 *>(s1 + 1);
-                x[u][0] = __ldg(s1);
-#pragma unroll
-                for (int q = 0; q < 3; ++q) {
-                    const uint2 v = __ldg(s2 + q);
-                    x[u][1 + 2 * q] = v.x;
-                    x[u][2 + 2 * q] = v.y;
-                }
-                x[u][7] = __ldg(s1 + 7);
-            } else {
-#pragma unroll
-                for (int q = 0; q < 8; ++q)
-                    x[u][q] = reinterpret_cast<const ST *>(src)[8ull * g + q];
-            }
+    const uint32_t phase = (uint32_t)((uintptr_t)src & 15u);
+    auto put = [&](uint32_t g, const uint32_t *x) {
+        uint32_t y[2 * DES];
+        convert8<CONV>(x, y);
+        const uint4 lo = make_uint4(y[0], y[1], y[2], y[3]);
+        acc += vsum<DES>(lo);
+        if constexpr (DES == 2) {
+            st_stream(dst + 16ull * g, lo);
+        } else {
+            const uint4 hi = make_uint4(y[DES], y[DES + 1], y[DES + 2], y[DES + 3]);
+            acc += vsum<DES>(hi);
+            st_stream32(dst + 32ull * g, lo, hi);
         }
+    };
+    if (SES == 2 && phase != 0) {
+        /* a group of 16-bit elements is one vector: the copy path's realigning loop */
+        realign_run<UR, W>(reinterpret_cast<const uint4 *>(src - phase), phase, ng, tid, nthr,
+                           [&](uint32_t g, const uint4 &o) {
+                               const uint32_t x[8] = {o.x, o.y, o.z, o.w, 0u, 0u, 0u, 0u};
+                               put(g, x);
+                           });
+    } else {
+        const uint32_t step = nthr * U;
+        for (uint32_t base = 0; base < ng; base += step) {
+            uint32_t x[U][2 * SES];
 #pragma unroll
-        for (int u = 0; u < U; ++u) {
-            const uint32_t g = base + u * nthr + tid;
-            if (g >= ng) continue;
-            uint32_t r[8];
-            uint64_t sum = 0;
+            for (int u = 0; u < U; ++u) {
+                const uint32_t g = base + u * nthr + tid;
+                if (g >= ng) continue;
+                if constexpr (SES == 2) {
+                    const uint4 v = ld_stream(src + 16ull * g);
+                    x[u][0] = v.x; x[u][1] = v.y; x[u][2] = v.z; x[u][3] = v.w;
+                } else if (phase == 0) {
+                    const uint4 a = ld_stream(src + 32ull * g), b = ld_stream(src + 32ull * g + 16);
+                    x[u][0] = a.x; x[u][1] = a.y; x[u][2] = a.z; x[u][3] = a.w;
+                    x[u][4] = b.x; x[u][5] = b.y; x[u][6] = b.z; x[u][7] = b.w;
+                } else if ((phase & 7u) == 0) {
+                    /* 8-byte aligned: four 8-byte loads instead of eight 4-byte ones */
+                    const uint2 *s2 = reinterpret_cast<const uint2 *>(src + 32ull * g);
 #pragma unroll
-            for (int q = 0; q < 8; ++q) {
-                r[q] = convert1<CONV>(x[u][q]);
-                sum += r[q];
+                    for (int q = 0; q < 4; ++q) {
+                        const uint2 v = __ldg(s2 + q);
+                        x[u][2 * q] = v.x;
+                        x[u][2 * q + 1] = v.y;
+                    }
+                } else {
+                    /* 4 mod 8: the first and last elements alone, the six between as 8-byte
+                     * pairs */
+                    const uint32_t *s1 = reinterpret_cast<const uint32_t *>(src + 32ull * g);
+                    const uint2 *s2 = reinterpret_cast<const uint2 *>(s1 + 1);
+                    x[u][0] = __ldg(s1);
+#pragma unroll
+                    for (int q = 0; q < 3; ++q) {
+                        const uint2 v = __ldg(s2 + q);
+                        x[u][1 + 2 * q] = v.x;
+                        x[u][2 + 2 * q] = v.y;
+                    }
+                    x[u][7] = __ldg(s1 + 7);
+                }
             }
-            if constexpr (DES == 2) {
-                st_stream(d + g, make_uint4(r[0] | (r[1] << 16), r[2] | (r[3] << 16),
-                                            r[4] | (r[5] << 16), r[6] | (r[7] << 16)));
-            } else {
-                st_stream(d + 2ull * g, make_uint4(r[0], r[1], r[2], r[3]));
-                st_stream(d + 2ull * g + 1, make_uint4(r[4], r[5], r[6], r[7]));
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                const uint32_t g = base + u * nthr + tid;
+                if (g < ng) put(g, x[u]);
             }
-            acc += sum;
         }
     }
     const uint64_t body = (uint64_t)ng << 3;
@@ -403,6 +531,14 @@ __device__ __forceinline__ bool item_ok(const cfa_work &w, const UnpackArgs &a)
            (w.dst & ((1ull << dl) - 1)) == 0;
 }
 
+/* Groups in flight per thread (aligned sources) and rounds of the realigning loop of a conversion
+ * class: 64 source bytes a thread for 16-bit results; the classes that write twice what they read
+ * do better with less in flight (bf16 -> fp32, 8.8 GB written: two groups 2085 us, four 2155). */
+template <int CLS> struct ConvertDepth {
+    static constexpr int groups = ClassOf<CLS>::ses == 4 || ClassOf<CLS>::des == 4 ? 2 : 4;
+    static constexpr int rounds = ClassOf<CLS>::des == 4 ? 2 : kRealignRounds;
+};
+
 /* One work item: U 16-byte vectors per thread in flight on the aligned path, UR rounds of W
  * vectors per lane group on the realigning path (default: four for slabs of the 2-8-byte copy
  * classes, two for the 1-byte class). */
@@ -415,7 +551,8 @@ __device__ __forceinline__ uint64_t run_item(const cfa_work &w, const UnpackArgs
     uint8_t *dst = reinterpret_cast<uint8_t *>(w.dst);
     typedef ClassOf<CLS> C;
     if constexpr (C::conv != CFA_CONV_NONE)
-        return convert_run<C::ses, C::des, C::conv, (U > 2 ? 2 : U)>(src, dst, w.n, tid, nthr);
+        return convert_run<C::ses, C::des, C::conv, (U > 1 ? ConvertDepth<CLS>::groups : 1),
+                           (U > 1 ? ConvertDepth<CLS>::rounds : 1), W>(src, dst, w.n, tid, nthr);
     else
         return copy_run<(1 << CLS), U, UR, W>(src, dst, (uint64_t)w.n << CLS, tid, nthr);
 }
@@ -495,7 +632,7 @@ __device__ __forceinline__ void run_tiny(const UnpackArgs &a, uint32_t group, ui
 }
 
 template <int CLS>
-__global__ void __launch_bounds__(kThreads, (CLS >= 1 && CLS < 4 ? kCopyMinBlocks : kMinBlocks))
+__global__ void __launch_bounds__(kThreads, unpack_min_blocks(CLS))
     cfa_unpack_kernel(const UnpackArgs a)
 {
     __shared__ unsigned long long red[kWarps];
@@ -903,7 +1040,7 @@ __device__ __forceinline__ void tiny_staged(const UnpackArgs &a)
 }
 
 template <int CLS>
-__global__ void __launch_bounds__(kThreads, (CLS < 4 ? kCopyMinBlocks : kMinBlocks))
+__global__ void __launch_bounds__(kThreads, (CLS == 0 ? kCopyMinBlocks : unpack_min_blocks(CLS)))
     cfa_tiny_kernel(const UnpackArgs a)
 {
     if constexpr (CLS < 4) {
@@ -1013,7 +1150,9 @@ __device__ __forceinline__ bool sitem_ok(const cfa_swork &w, const StridedArgs &
  * like a contiguous run (16-byte vectors, realigned when source and destination disagree mod
  * 16, four vectors in flight per lane). */
 template <int CLS>
-__global__ void __launch_bounds__(kThreads, (CLS < 4 ? kCopyMinBlocks : kMinBlocks))
+__global__ void __launch_bounds__(kThreads, (CLS == 0 || ClassOf<CLS>::ses == 2
+                                                 ? kCopyMinBlocks
+                                                 : unpack_min_blocks(CLS)))
     cfa_strided_kernel(const StridedArgs a)
 {
     typedef ClassOf<CLS> C;
@@ -1041,7 +1180,8 @@ __global__ void __launch_bounds__(kThreads, (CLS < 4 ? kCopyMinBlocks : kMinBloc
             const uint8_t *s = src + (uint64_t)r * w.stride * SES;
             uint8_t *d = dst + (uint64_t)r * w.cols * DES;
             if constexpr (C::conv != CFA_CONV_NONE)
-                acc += convert_run<SES, DES, C::conv, 2>(s, d, w.cols, lane, 32u);
+                acc += convert_run<SES, DES, C::conv, ConvertDepth<CLS>::groups,
+                                   ConvertDepth<CLS>::rounds, 32>(s, d, w.cols, lane, 32u);
             else
                 acc += copy_run<DES, kUnroll, kRealignRoundsRows>(s, d, (uint64_t)w.cols * DES,
                                                                   lane, 32u);
