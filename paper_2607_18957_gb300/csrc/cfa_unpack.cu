@@ -60,6 +60,7 @@ struct UnpackArgs {
     const cfa_work *tiny;
     uint32_t n_slabs;
     uint32_t n_tiny;
+    uint32_t parts_log2; /* every block-level item is copied in 2^parts_log2 parts */
     uint64_t src_base;   /* device address of blob byte 0 for this launch */
     uint64_t src_period; /* 0, or P: blob byte o sits at src_base + (o mod P) */
     uint64_t src_lo;     /* blob bytes [src_lo, src_hi) are readable in this launch */
@@ -531,6 +532,30 @@ __device__ __forceinline__ bool item_ok(const cfa_work &w, const UnpackArgs &a)
            (w.dst & ((1ull << dl) - 1)) == 0;
 }
 
+/* Narrows a checked block-level item to part k of its 2^parts_log2 equal parts; false if that
+ * part is empty.  Parts hold at least CFA_MIN_PART_BYTES (of the wider side; a smaller item has
+ * fewer parts) and are cut where the destination is a multiple of CFA_PART_ALIGN, so only the
+ * item's own ends can be off the vector grid. */
+template <int SES, int DES>
+__device__ __forceinline__ bool take_part(cfa_work &w, uint32_t k, uint32_t parts_log2)
+{
+    if (parts_log2 == 0) return true;
+    constexpr uint32_t kAlignElems = CFA_PART_ALIGN / DES;
+    constexpr uint32_t kMinElems = CFA_MIN_PART_BYTES / (SES > DES ? SES : DES);
+    uint32_t per = (uint32_t)(((uint64_t)w.n + (1u << parts_log2) - 1u) >> parts_log2);
+    if (per < kMinElems) per = kMinElems;
+    const uint64_t step = ((uint64_t)per + kAlignElems - 1u) / kAlignElems * kAlignElems;
+    /* elements from the last aligned destination address to the item's first element */
+    const uint32_t lead = (uint32_t)(w.dst & (CFA_PART_ALIGN - 1u)) / DES;
+    const uint64_t a = k ? k * step - lead : 0;
+    const uint64_t b = (k + 1u) >> parts_log2 ? (uint64_t)w.n : (k + 1u) * step - lead;
+    if (a >= w.n) return false;
+    w.n = (uint32_t)((b < w.n ? b : w.n) - a);
+    w.src += a * SES;
+    w.dst += a * DES;
+    return true;
+}
+
 /* Groups in flight per thread (aligned sources) and rounds of the realigning loop of a conversion
  * class: 64 source bytes a thread for 16-bit results; the classes that write twice what they read
  * do better with less in flight (bf16 -> fp32, 8.8 GB written: two groups 2085 us, four 2155). */
@@ -637,8 +662,9 @@ __global__ void __launch_bounds__(kThreads, unpack_min_blocks(CLS))
 {
     __shared__ unsigned long long red[kWarps];
     const uint32_t n_groups = (a.n_tiny + kTinyPerGroup - 1) / kTinyPerGroup;
-    const uint32_t n_items = a.n_slabs + n_groups;
-    const uint32_t q = n_groups ? a.n_slabs / n_groups : 0;
+    const uint32_t n_slabs = a.n_slabs << a.parts_log2; /* parts of slabs */
+    const uint32_t n_items = n_slabs + n_groups;
+    const uint32_t q = n_groups ? n_slabs / n_groups : 0;
     const uint32_t mixed = n_groups * (q + 1); /* items in the interleaved prefix */
     const uint32_t lane = threadIdx.x & 31u, warp = threadIdx.x >> 5;
     uint64_t acc = 0;
@@ -658,11 +684,14 @@ __global__ void __launch_bounds__(kThreads, unpack_min_blocks(CLS))
             group = 0;
         }
         if (is_slab) {
-            const cfa_work w = a.slabs[slab]; /* the same 32 bytes for every thread */
+            cfa_work w = a.slabs[slab >> a.parts_log2]; /* the same 32 bytes for every thread */
             if (!item_ok<CLS>(w, a)) {
                 if (threadIdx.x == 0) atomicCAS(a.status, 0, 1);
                 continue;
             }
+            if (!take_part<ClassOf<CLS>::ses, ClassOf<CLS>::des>(
+                    w, slab & ((1u << a.parts_log2) - 1u), a.parts_log2))
+                continue;
             if (w.ck != acc_ck) {
                 if (acc_ck != CFA_NO_CK) block_flush(acc, acc_ck, a.ck, red);
                 acc = 0;
@@ -1243,16 +1272,24 @@ extern "C" cudaError_t cfa_launch_unpack(int cls, const cfa_work *slabs, uint32_
                                          uint64_t src_base, uint64_t src_period,
                                          uint64_t src_lo, uint64_t src_hi,
                                          unsigned long long *ck, int *status, int grid_cap,
-                                         int dev_src, cudaStream_t stream)
+                                         uint32_t item_bytes, int dev_src,
+                                         cudaStream_t stream)
 {
     if (cls < 0 || cls >= CFA_N_CLASSES || grid_cap <= 0) return cudaErrorInvalidValue;
-    const uint64_t items = (uint64_t)n_slabs + (n_tiny + kTinyPerGroup - 1) / kTinyPerGroup;
+    /* the fp32 -> 16-bit classes read twice what they write */
+    const bool narrows = cls == CFA_CLASS_OF_CONV(CFA_CONV_F32_BF16) ||
+                         cls == CFA_CLASS_OF_CONV(CFA_CONV_F32_F16);
+    const uint32_t parts_log2 =
+        cfa_parts_log2(n_slabs, (uint32_t)grid_cap, narrows ? 2 * item_bytes : item_bytes);
+    const uint64_t items =
+        ((uint64_t)n_slabs << parts_log2) + (n_tiny + kTinyPerGroup - 1) / kTinyPerGroup;
     if (items == 0) return cudaSuccess;
     UnpackArgs a;
     a.slabs = slabs;
     a.tiny = tiny;
     a.n_slabs = n_slabs;
     a.n_tiny = n_tiny;
+    a.parts_log2 = parts_log2;
     a.src_base = src_base;
     a.src_period = src_period;
     a.src_lo = src_lo;

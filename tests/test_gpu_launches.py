@@ -1,0 +1,89 @@
+"""How launches are cut: block-level items cut into parts where a launch has few of them (sizes
+around the parts, sources and destinations at odd phases).  Checked against slices of the blob."""
+import ctypes
+
+import numpy as np
+import pytest
+import torch
+
+import paper_2607_18957_gb300 as cfa
+from paper_2607_18957_gb300 import _lib
+
+pytestmark = pytest.mark.gpu
+
+ES = {"u8": 1, "bf16": 2, "f32": 4, "i64": 8}
+PART = 32768  # least bytes of a part
+
+
+@pytest.fixture(scope="module", autouse=True)
+def cuda_device():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    torch.cuda.set_device(0)
+
+
+class Copies:
+    """Plain copies: tensors of (dtype, bytes, source phase, destination phase) in one blob."""
+
+    def __init__(self, tensors, seed=3):
+        self.runs, at, to = [], 0, 0
+        for dtype, nbytes, sp, dp in tensors:
+            es = ES[dtype]
+            at, to = (at + 255) // 256 * 256 + sp * es, (to + 255) // 256 * 256 + 256 + dp * es
+            self.runs.append((dtype, at, to, nbytes // es * es))
+            at, to = at + nbytes, to + nbytes
+        self.blob_bytes = (at + 255) // 256 * 256
+        g = torch.Generator(device="cuda").manual_seed(seed)
+        self.blob = torch.randint(0, 256, (self.blob_bytes,), dtype=torch.uint8, device="cuda",
+                                  generator=g)
+        self.out = torch.full((to + 256,), 0xA5, dtype=torch.uint8, device="cuda")
+        self.want = self.out.clone()
+        for _, a, t, n in self.runs:
+            self.want[t:t + n] = self.blob[a:a + n]
+        shapes = [(n // ES[d],) for d, _, _, n in self.runs]
+        self.entries = cfa.make_entries(dtype=[r[0] for r in self.runs], shape=shapes,
+                                        offset=[r[1] for r in self.runs],
+                                        dst=list(range(len(self.runs))))
+        self.dsts = [(self.out.data_ptr() + r[2], r[0], s) for r, s in zip(self.runs, shapes)]
+
+    def checksums(self):
+        blob = self.blob.cpu().numpy()
+        u = {1: np.uint8, 2: np.uint16, 4: np.uint32, 8: np.uint64}
+        return np.array([blob[a:a + n].view(u[ES[d]]).astype(np.uint64).sum(dtype=np.uint64)
+                         for d, a, _, n in self.runs])
+
+
+def tensors(sizes, phases):
+    return [(d, n, p, q) for n in sizes for d in ES for p, q in phases]
+
+
+SIZES = [8192, PART - 16, PART, PART + 16, 2 * PART + 48, 7 * PART + 8, 300 * 1024, (2 << 20) + 24]
+
+
+@pytest.mark.parametrize("phases", [[(0, 0)], [(0, 0), (1, 0), (0, 1), (1, 3)]])
+@pytest.mark.parametrize("slab_kib", [0, 256, 4096])
+def test_planned_items_are_cut_into_parts(phases, slab_kib):
+    c = Copies(tensors(SIZES, phases))
+    with cfa.Plan(c.entries, c.dsts, c.blob_bytes, dev_slots=0, host_slots=0,
+                  slab_bytes=slab_kib << 10) as plan:
+        plan.load_async(cfa.Source.device(c.blob.data_ptr()))
+        plan.wait_layer()
+        ck = plan.checksums()
+    assert torch.equal(c.out, c.want)
+    assert np.array_equal(ck, c.checksums())
+
+
+def test_noalloc_items_are_cut_into_parts():
+    c = Copies(tensors(SIZES + [(4 << 20) + 8], [(0, 0), (1, 0), (1, 3)]))
+    ck = torch.full((len(c.runs),), -1, dtype=torch.int64, device="cuda")
+    status = torch.full((1,), -1, dtype=torch.int32, device="cuda")
+    dsts = cfa.make_dsts(c.dsts)
+    err = ctypes.create_string_buffer(256)
+    st = _lib.load().cfa_unpack_noalloc(
+        c.entries.arr.ctypes.data, len(c.entries), dsts.ctypes.data, len(dsts),
+        c.blob.data_ptr(), c.blob_bytes, ck.data_ptr(), status.data_ptr(),
+        torch.cuda.current_stream().cuda_stream, err, len(err))
+    assert st == 0, err.value
+    assert int(status.item()) == 0
+    assert torch.equal(c.out, c.want)
+    assert np.array_equal(ck.cpu().numpy().view(np.uint64), c.checksums())
