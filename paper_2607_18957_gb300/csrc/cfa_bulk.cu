@@ -13,6 +13,11 @@
  *     lanes), and one lane issues the bulk store; once the store of the previous sub-block has
  *     finished reading its stage (bulk_group read wait), that stage is released on its `empty`
  *     mbarrier.
+ * One launch takes the items of every element size (the consumer sums each stage by its item's
+ * size), cut into parts where there are too few for the grid (cfa_parts_log2).  With a launch per
+ * element size, forked and joined with events, and whole 256 KiB slabs, an 8-bit checkpoint with
+ * block scales unpacked in 64 MiB chunks (1.4 to 3 launches a chunk, 256 items for 456 CTAs) took
+ * 1630 us for 3.4 GB; one launch of parts 1370.
  * No block-wide barrier runs inside the loop.  Plain cp.async.bulk only: no tensor maps, no
  * multicast, one CTA's own shared memory.
  *
@@ -40,8 +45,10 @@ constexpr uint32_t kSpinLimit = 1u << 20;              /* try_wait polls before 
 constexpr uint32_t kLoseLoads = 1u << 31;              /* self-test: the loader issues nothing */
 
 struct BulkArgs {
-    const cfa_work *items;
-    uint32_t n_items;
+    cfa_bulk_range range[4]; /* item lists, one per element size present */
+    uint32_t n_ranges;
+    uint32_t n_items;    /* parts over all ranges */
+    uint32_t parts_log2; /* every item is copied in 2^parts_log2 parts */
     uint32_t spin_limit; /* try_wait polls before a wait gives up; the self-test sets a short one
                             and tells the loader to issue nothing (spin_limit | kLoseLoads) */
     uint64_t src_base;
@@ -127,15 +134,71 @@ __device__ __forceinline__ void mbar_arrive(uint64_t *bar)
     asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_addr(bar)) : "memory");
 }
 
-/* A bulk item is sound if its source lies inside the launch's readable range and source,
- * destination and length are multiples of 16 bytes. */
-template <int LOG2ES>
+/* A bulk item is sound if it is a plain copy, its source lies inside the launch's readable range
+ * and source, destination and length are multiples of 16 bytes. */
 __device__ __forceinline__ bool bulk_item_ok(const cfa_work &w, const BulkArgs &a)
 {
-    const uint64_t bytes = (uint64_t)w.n << LOG2ES;
-    return w.n != 0 && w.mode == CFA_MODE(LOG2ES, LOG2ES, 0) && w.src >= a.src_lo &&
+    const uint32_t log2es = w.mode & 3u;
+    const uint64_t bytes = (uint64_t)w.n << log2es;
+    return w.n != 0 && w.mode == CFA_MODE(log2es, log2es, 0) && w.src >= a.src_lo &&
            w.src <= a.src_hi && bytes <= a.src_hi - w.src && bytes < (1ull << 31) &&
            ((w.src | w.dst | bytes | a.src_base | a.src_period) & 15u) == 0;
+}
+
+/* Bytes [*at, *at + *len) of a checked item of `total` bytes at destination `dst` that are part k
+ * of its 2^parts_log2 equal parts (cut as in the vector kernel); false if the part is empty. */
+__device__ __forceinline__ bool bulk_part(uint64_t dst, uint32_t total, uint32_t k,
+                                          uint32_t parts_log2, uint32_t *at, uint32_t *len)
+{
+    *at = 0;
+    *len = total;
+    if (parts_log2 == 0) return true;
+    uint32_t step = (total + (1u << parts_log2) - 1u) >> parts_log2;
+    if (step < CFA_MIN_PART_BYTES) step = CFA_MIN_PART_BYTES;
+    step = (step + CFA_PART_ALIGN - 1u) & ~(CFA_PART_ALIGN - 1u);
+    const uint32_t lead = (uint32_t)(dst & (CFA_PART_ALIGN - 1u));
+    const uint64_t a = k ? (uint64_t)k * step - lead : 0;
+    const uint64_t b = (k + 1u) >> parts_log2 ? total : (uint64_t)(k + 1u) * step - lead;
+    if (a >= total) return false;
+    *at = (uint32_t)a;
+    *len = (uint32_t)((b < total ? b : total) - a);
+    return true;
+}
+
+/* Descriptor of part `v` of the launch. */
+__device__ __forceinline__ cfa_work bulk_fetch(const BulkArgs &a, uint32_t v)
+{
+    uint32_t i = v >> a.parts_log2;
+    int r = 0;
+#pragma unroll
+    for (int q = 0; q < 3; ++q)
+        if (r == q && i >= a.range[q].n && (uint32_t)q + 1u < a.n_ranges) {
+            i -= a.range[q].n;
+            r = q + 1;
+        }
+    const cfa_work *p = a.range[0].items;
+#pragma unroll
+    for (int q = 1; q < 4; ++q)
+        if (r == q) p = a.range[q].items;
+    return p[i];
+}
+
+/* Sum of a staged sub-block's elements over this lane's vectors: eight independent shared loads
+ * in flight, then the ragged rest. */
+template <int ES>
+__device__ __forceinline__ uint64_t stage_sum(const uint4 *v, uint32_t nv, uint32_t lane)
+{
+    uint64_t acc = 0;
+    uint32_t i = lane;
+    for (; i + 7 * 32 < nv; i += 8 * 32) {
+        uint4 x[8];
+#pragma unroll
+        for (int u = 0; u < 8; ++u) x[u] = v[i + u * 32];
+#pragma unroll
+        for (int u = 0; u < 8; ++u) acc += vsum<ES>(x[u]);
+    }
+    for (; i < nv; i += 32) acc += vsum<ES>(v[i]);
+    return acc;
 }
 
 /* What the consumer needs of a staged sub-block; written by the producer before the load is
@@ -144,9 +207,9 @@ struct StageMeta {
     uint64_t dst;
     uint32_t len;
     uint32_t ck;
+    uint32_t log2es;
 };
 
-template <int LOG2ES>
 __global__ void __launch_bounds__(kThreads) cfa_bulk_kernel(const BulkArgs a)
 {
     extern __shared__ __align__(128) uint8_t stage[];
@@ -175,26 +238,35 @@ __global__ void __launch_bounds__(kThreads) cfa_bulk_kernel(const BulkArgs a)
          * stage's previous tenant, has been released.  The next item's descriptor is fetched
          * while the current item's sub-blocks are issued. */
         if (lane == 0) {
-            /* item `it` is being issued from w; item it + gridDim.x is in flight into nxt */
-            uint32_t it = blockIdx.x, p = 0, off = 0;
+            /* part `it` is being issued from w, bytes [off, end) left; the descriptor of part
+             * it + gridDim.x is in flight into nxt */
+            uint32_t it = blockIdx.x, p = 0, off = 0, end = 0;
             bool have = it < a.n_items;
             cfa_work w{}, nxt{};
-            if (have) w = a.items[it];
+            if (have) w = bulk_fetch(a, it);
             uint32_t it_n = it + gridDim.x;
-            if (it_n < a.n_items) nxt = a.items[it_n];
-            auto step = [&]() { /* move to the next item of this CTA */
+            if (it_n < a.n_items) nxt = bulk_fetch(a, it_n);
+            auto step = [&]() { /* move to the next part of this CTA */
                 it = it_n;
                 have = it < a.n_items;
                 if (have) {
                     w = nxt;
                     it_n = it + gridDim.x;
-                    if (it_n < a.n_items) nxt = a.items[it_n];
+                    if (it_n < a.n_items) nxt = bulk_fetch(a, it_n);
                 }
             };
-            auto settle = [&]() { /* skip items that fail the checks */
-                while (have && !bulk_item_ok<LOG2ES>(w, a)) {
-                    atomicCAS(a.status, 0, 1);
-                    step();
+            auto settle = [&]() { /* skip items that fail the checks, and empty parts */
+                for (; have; step()) {
+                    if (!bulk_item_ok(w, a)) {
+                        atomicCAS(a.status, 0, 1);
+                        continue;
+                    }
+                    uint32_t len;
+                    if (bulk_part(w.dst, w.n << (w.mode & 3u),
+                                  it & ((1u << a.parts_log2) - 1u), a.parts_log2, &off, &len)) {
+                        end = off + len;
+                        break;
+                    }
                 }
             };
             settle();
@@ -210,11 +282,11 @@ __global__ void __launch_bounds__(kThreads) cfa_bulk_kernel(const BulkArgs a)
                     mbar_arrive(&full[s]);
                     break;
                 }
-                const uint32_t total = w.n << LOG2ES;
-                const uint32_t len = min(kStageBytes, total - off);
+                const uint32_t len = min(kStageBytes, end - off);
                 meta[s].dst = w.dst + off;
                 meta[s].len = len;
                 meta[s].ck = w.ck;
+                meta[s].log2es = w.mode & 3u;
                 mbar_expect_tx(&full[s], len);
                 const uint64_t so = a.src_period ? w.src % a.src_period : w.src;
                 bulk_load(stage + s * kStageBytes,
@@ -223,8 +295,7 @@ __global__ void __launch_bounds__(kThreads) cfa_bulk_kernel(const BulkArgs a)
                 ++p;
                 n_issued = p;
                 off += len;
-                if (off >= total) {
-                    off = 0;
+                if (off >= end) {
                     step();
                     settle();
                 }
@@ -249,18 +320,14 @@ __global__ void __launch_bounds__(kThreads) cfa_bulk_kernel(const BulkArgs a)
                 acc_ck = m.ck;
             }
             if (m.ck != CFA_NO_CK) {
-                /* eight independent shared loads per lane in flight, then the ragged rest */
                 const uint4 *v = reinterpret_cast<const uint4 *>(stage + s * kStageBytes);
                 const uint32_t nv = m.len >> 4;
-                uint32_t i = lane;
-                for (; i + 7 * 32 < nv; i += 8 * 32) {
-                    uint4 x[8];
-#pragma unroll
-                    for (int u = 0; u < 8; ++u) x[u] = v[i + u * 32];
-#pragma unroll
-                    for (int u = 0; u < 8; ++u) acc += vsum<1 << LOG2ES>(x[u]);
+                switch (m.log2es) {
+                case 0: acc += stage_sum<1>(v, nv, lane); break;
+                case 1: acc += stage_sum<2>(v, nv, lane); break;
+                case 2: acc += stage_sum<4>(v, nv, lane); break;
+                default: acc += stage_sum<8>(v, nv, lane); break;
                 }
-                for (; i < nv; i += 32) acc += vsum<1 << LOG2ES>(v[i]);
             }
             if (lane == 0) {
                 bulk_store(reinterpret_cast<uint8_t *>(m.dst), stage + s * kStageBytes, m.len);
@@ -292,39 +359,41 @@ __global__ void __launch_bounds__(kThreads) cfa_bulk_kernel(const BulkArgs a)
     }
 }
 
-typedef void (*bulk_fn)(const BulkArgs);
-const bulk_fn kBulk[4] = {cfa_bulk_kernel<0>, cfa_bulk_kernel<1>, cfa_bulk_kernel<2>,
-                          cfa_bulk_kernel<3>};
-
 } // namespace
 
-/* Resident CTAs per SM of the bulk kernel for element size 2^log2es (0 if it cannot run). */
-extern "C" int cfa_bulk_blocks_per_sm(int log2es)
+/* Resident CTAs per SM of the bulk kernel (0 if it cannot run). */
+extern "C" int cfa_bulk_blocks_per_sm(void)
 {
-    if (log2es < 0 || log2es > 3) return 0;
-    if (cudaFuncSetAttribute(kBulk[log2es], cudaFuncAttributeMaxDynamicSharedMemorySize,
+    if (cudaFuncSetAttribute(cfa_bulk_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              (int)kSmemBytes) != cudaSuccess)
         return 0;
     int n = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, kBulk[log2es], kThreads, kSmemBytes) !=
-        cudaSuccess)
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, cfa_bulk_kernel, kThreads,
+                                                      kSmemBytes) != cudaSuccess)
         return 0;
     return n;
 }
 
-/* Launches the bulk unpack over items whose source, destination and byte length are multiples
- * of 16; grid_cap bounds the persistent grid. */
-extern "C" cudaError_t cfa_launch_bulk(int log2es, const cfa_work *items, uint32_t n_items,
+/* Launches the bulk unpack over up to four lists of items whose source, destination and byte
+ * length are multiples of 16; grid_cap bounds the persistent grid. */
+extern "C" cudaError_t cfa_launch_bulk(const cfa_bulk_range *ranges, uint32_t n_ranges,
                                        uint64_t src_base, uint64_t src_period,
                                        uint64_t src_lo, uint64_t src_hi,
                                        unsigned long long *ck, int *status, int grid_cap,
-                                       cudaStream_t stream)
+                                       uint32_t item_bytes, cudaStream_t stream)
 {
-    if (log2es < 0 || log2es > 3 || grid_cap <= 0) return cudaErrorInvalidValue;
+    if (n_ranges > 4 || grid_cap <= 0) return cudaErrorInvalidValue;
+    BulkArgs a{};
+    uint64_t n_items = 0;
+    for (uint32_t r = 0; r < n_ranges; ++r) {
+        if (!ranges[r].n) continue;
+        a.range[a.n_ranges++] = ranges[r];
+        n_items += ranges[r].n;
+    }
     if (n_items == 0) return cudaSuccess;
-    BulkArgs a;
-    a.items = items;
-    a.n_items = n_items;
+    if (n_items >= (1ull << 31)) return cudaErrorInvalidValue;
+    a.parts_log2 = cfa_parts_log2((uint32_t)n_items, (uint32_t)grid_cap, item_bytes);
+    a.n_items = (uint32_t)n_items << a.parts_log2;
     a.spin_limit = kSpinLimit;
     a.src_base = src_base;
     a.src_period = src_period;
@@ -332,8 +401,8 @@ extern "C" cudaError_t cfa_launch_bulk(int log2es, const cfa_work *items, uint32
     a.src_hi = src_hi;
     a.ck = ck;
     a.status = status;
-    const uint32_t grid = n_items < (uint32_t)grid_cap ? n_items : (uint32_t)grid_cap;
-    kBulk[log2es]<<<grid, kThreads, kSmemBytes, stream>>>(a);
+    const uint32_t grid = a.n_items < (uint32_t)grid_cap ? a.n_items : (uint32_t)grid_cap;
+    cfa_bulk_kernel<<<grid, kThreads, kSmemBytes, stream>>>(a);
     return cudaGetLastError();
 }
 
@@ -349,7 +418,7 @@ extern "C" cudaError_t cfa_bulk_selftest_timeout(int *status_host)
     cudaError_t e = cudaSuccess;
     if (!status_host) return cudaErrorInvalidValue;
     *status_host = -1;
-    if ((e = cudaFuncSetAttribute(kBulk[1], cudaFuncAttributeMaxDynamicSharedMemorySize,
+    if ((e = cudaFuncSetAttribute(cfa_bulk_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                   (int)kSmemBytes)) != cudaSuccess)
         return e;
     if ((e = cudaMalloc(&d_item, sizeof(cfa_work))) != cudaSuccess) goto out;
@@ -366,8 +435,9 @@ extern "C" cudaError_t cfa_bulk_selftest_timeout(int *status_host)
         if ((e = cudaMemcpy(d_item, &w, sizeof w, cudaMemcpyHostToDevice)) != cudaSuccess) goto out;
         if ((e = cudaMemset(d_status, 0, sizeof(int))) != cudaSuccess) goto out;
         if ((e = cudaMemset(d_ck, 0, sizeof(unsigned long long))) != cudaSuccess) goto out;
-        BulkArgs a;
-        a.items = d_item;
+        BulkArgs a{};
+        a.range[0] = cfa_bulk_range{d_item, 1};
+        a.n_ranges = 1;
         a.n_items = 1;
         a.spin_limit = 256u | kLoseLoads;
         a.src_base = (uint64_t)(uintptr_t)d_buf;
@@ -376,7 +446,7 @@ extern "C" cudaError_t cfa_bulk_selftest_timeout(int *status_host)
         a.src_hi = 256;
         a.ck = d_ck;
         a.status = d_status;
-        kBulk[1]<<<1, kThreads, kSmemBytes>>>(a);
+        cfa_bulk_kernel<<<1, kThreads, kSmemBytes>>>(a);
         if ((e = cudaGetLastError()) != cudaSuccess) goto out;
         if ((e = cudaDeviceSynchronize()) != cudaSuccess) goto out;
         e = cudaMemcpy(status_host, d_status, sizeof(int), cudaMemcpyDeviceToHost);

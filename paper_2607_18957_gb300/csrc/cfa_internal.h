@@ -42,6 +42,12 @@ typedef struct cfa_work {
  * destination addresses that are multiples of it): one 8-lane warp segment copies one item. */
 #define CFA_TINY_SEG_BYTES 512u
 
+/* One of the item lists of a bulk launch (the items of one element size). */
+typedef struct cfa_bulk_range {
+    const cfa_work *items;
+    uint32_t n;
+} cfa_bulk_range;
+
 typedef struct cfa_swork {
     uint64_t src;
     uint64_t dst;

@@ -43,18 +43,18 @@
 #include "cfa_pool.h"
 
 extern "C" int cfa_unpack_blocks_per_sm(int cls);
-extern "C" int cfa_bulk_blocks_per_sm(int log2es);
+extern "C" int cfa_bulk_blocks_per_sm(void);
 extern "C" int cfa_strided_blocks_per_sm(int cls);
 extern "C" cudaError_t cfa_launch_strided(int cls, const cfa_swork *items, uint32_t n_items,
                                           uint64_t src_base, uint64_t src_period,
                                           uint64_t src_lo, uint64_t src_hi,
                                           unsigned long long *ck, int *status, int grid_cap,
                                           cudaStream_t stream);
-extern "C" cudaError_t cfa_launch_bulk(int log2es, const cfa_work *items, uint32_t n_items,
+extern "C" cudaError_t cfa_launch_bulk(const cfa_bulk_range *ranges, uint32_t n_ranges,
                                        uint64_t src_base, uint64_t src_period,
                                        uint64_t src_lo, uint64_t src_hi,
                                        unsigned long long *ck, int *status, int grid_cap,
-                                       cudaStream_t stream);
+                                       uint32_t item_bytes, cudaStream_t stream);
 extern "C" cudaError_t cfa_bulk_selftest_timeout(int *status_host);
 extern "C" cudaError_t cfa_launch_pull(const void *src, void *dst, uint64_t bytes, int grid,
                                        cudaStream_t stream);
@@ -118,7 +118,7 @@ struct cfa_plan {
     int device = 0;
     int pageable_access = 0; /* the device can read pageable host memory in place */
     int grid_cap[CFA_N_CLASSES] = {0};
-    int bulk_grid_cap[4] = {0};
+    int bulk_grid_cap = 0;
     int strided_grid_cap[CFA_N_CLASSES] = {0};
     cfa_work *d_slabs = nullptr, *d_tiny = nullptr, *d_bulk = nullptr;
     cfa_swork *d_strided = nullptr;
@@ -273,9 +273,9 @@ void CUDART_CB fill_host_fn(void *arg)
 }
 
 /* Unpacks chunks [c0, c1), whose blob byte o sits at device address src_base + o (or
- * src_base + (o mod period) for a periodic source): per work class present in those chunks
- * (normally one), a TMA bulk launch for its aligned cast-free slabs, a launch for its column
- * slices and a vector launch for everything else.  The kernels of one group write disjoint
+ * src_base + (o mod period) for a periodic source): one TMA bulk launch for the aligned cast-free
+ * slabs of every element size, and per work class present in those chunks (normally one) a launch
+ * for its column slices and a vector launch for everything else.  The kernels of one group write disjoint
  * destination bytes and add their checksums atomically, so they are independent: the first
  * runs on `s`, the others on side streams forked from `s` and joined back into it, so that
  * one kernel's last CTAs overlap the next kernel's first instead of the GPU draining between
@@ -300,10 +300,15 @@ cfa_status launch(cfa_plan *p, uint32_t c0, uint32_t c1, uint64_t src_base, uint
     };
     Job jobs[3 * CFA_N_CLASSES];
     int n = 0;
-    for (int k = 0; k < CFA_N_CLASSES && hp.n_bulk && (what & LAUNCH_CONTIG); ++k) {
+    cfa_bulk_range ranges[4]; /* bulk items are plain copies: classes 0 to 3 */
+    uint32_t n_ranges = 0;
+    for (int k = 0; k < 4 && hp.n_bulk && (what & LAUNCH_CONTIG); ++k) {
         const uint32_t b0 = hp.bulk_first[k * row + c0], b1 = hp.bulk_first[k * row + c1];
-        if (b1 != b0) jobs[n++] = Job{tma ? BULK : BULK_AS_VECTOR, k, b0, b1, 0, 0};
+        if (b1 == b0) continue;
+        if (!tma) jobs[n++] = Job{BULK_AS_VECTOR, k, b0, b1, 0, 0};
+        else ranges[n_ranges++] = cfa_bulk_range{p->d_bulk + b0, b1 - b0};
     }
+    if (n_ranges) jobs[n++] = Job{BULK, 0, 0, 0, 0, 0};
     for (int k = 0; k < CFA_N_CLASSES && hp.n_strided && (what & LAUNCH_STRIDED); ++k) {
         const uint32_t r0 = hp.strided_first[k * row + c0], r1 = hp.strided_first[k * row + c1];
         if (r1 != r0) jobs[n++] = Job{STRIDED, k, r0, r1, 0, 0};
@@ -329,8 +334,8 @@ cfa_status launch(cfa_plan *p, uint32_t c0, uint32_t c1, uint64_t src_base, uint
             p->t_k_c1[p->last_launches] = c1;
         }
         if (J.type == BULK)
-            CK(p, cfa_launch_bulk(k, p->d_bulk + J.a0, J.a1 - J.a0, src_base, period, lo, hi,
-                                  p->d_ck, p->d_status, cap(p->bulk_grid_cap[k]), ls));
+            CK(p, cfa_launch_bulk(ranges, n_ranges, src_base, period, lo, hi, p->d_ck,
+                                  p->d_status, cap(p->bulk_grid_cap), hp.opts.slab_bytes, ls));
         else if (J.type == BULK_AS_VECTOR) /* bulk items are copy-class slabs of class k */
             CK(p, cfa_launch_unpack(k, p->d_bulk + J.a0, J.a1 - J.a0, nullptr, 0, src_base,
                                     period, lo, hi, p->d_ck, p->d_status, cap(p->grid_cap[k]),
@@ -466,14 +471,12 @@ cfa_status setup_device(cfa_plan *p)
         p->strided_grid_cap[k] = sms * per_sm;
     }
     if (hp.n_bulk) {
-        for (int k = 0; k < 4; ++k) {
-            const int per_sm = cfa_bulk_blocks_per_sm(k);
-            if (per_sm <= 0) {
-                set_err(nullptr, "bulk kernel %d cannot run on device %d", k, p->device);
-                return CFA_ERR_CUDA;
-            }
-            p->bulk_grid_cap[k] = sms * per_sm;
+        const int per_sm = cfa_bulk_blocks_per_sm();
+        if (per_sm <= 0) {
+            set_err(nullptr, "the bulk kernel cannot run on device %d", p->device);
+            return CFA_ERR_CUDA;
         }
+        p->bulk_grid_cap = sms * per_sm;
     }
 
     auto upload = [&](cfa_work **d, const cfa_work *h, size_t n) -> cfa_status {
