@@ -34,6 +34,9 @@
 
 namespace {
 
+using cfa_dev::launch_begin;
+using cfa_dev::launch_ctl;
+using cfa_dev::launch_end;
 using cfa_dev::vsum;
 using cfa_dev::warp_sum;
 
@@ -56,6 +59,7 @@ struct BulkArgs {
     uint64_t src_lo, src_hi;
     unsigned long long *ck;
     int *status;
+    cfa_launch_ctl ctl;
 };
 
 __device__ __forceinline__ uint32_t smem_addr(const void *p)
@@ -229,6 +233,14 @@ __global__ void __launch_bounds__(kThreads) cfa_bulk_kernel(const BulkArgs a)
         n_issued = 0;
         n_consumed = 0;
     }
+    /* the loader's first two descriptors (the plan's own memory, written before any launch) are
+     * on their way while the launch waits for what is before it on the stream */
+    cfa_work w{}, nxt{};
+    if (threadIdx.x == 0) {
+        if (blockIdx.x < a.n_items) w = bulk_fetch(a, blockIdx.x);
+        if (blockIdx.x + gridDim.x < a.n_items) nxt = bulk_fetch(a, blockIdx.x + gridDim.x);
+    }
+    launch_begin(a.ctl);
     __syncthreads();
     const uint32_t lane = threadIdx.x & 31u;
     const uint32_t limit = a.spin_limit & ~kLoseLoads;
@@ -242,10 +254,7 @@ __global__ void __launch_bounds__(kThreads) cfa_bulk_kernel(const BulkArgs a)
              * it + gridDim.x is in flight into nxt */
             uint32_t it = blockIdx.x, p = 0, off = 0, end = 0;
             bool have = it < a.n_items;
-            cfa_work w{}, nxt{};
-            if (have) w = bulk_fetch(a, it);
             uint32_t it_n = it + gridDim.x;
-            if (it_n < a.n_items) nxt = bulk_fetch(a, it_n);
             auto step = [&]() { /* move to the next part of this CTA */
                 it = it_n;
                 have = it < a.n_items;
@@ -357,6 +366,7 @@ __global__ void __launch_bounds__(kThreads) cfa_bulk_kernel(const BulkArgs a)
         if (drained) atomicCAS(a.status, 0, 2);
         else atomicMax(a.status, 3);
     }
+    launch_end(a.ctl);
 }
 
 } // namespace
@@ -380,7 +390,7 @@ extern "C" cudaError_t cfa_launch_bulk(const cfa_bulk_range *ranges, uint32_t n_
                                        uint64_t src_base, uint64_t src_period,
                                        uint64_t src_lo, uint64_t src_hi,
                                        unsigned long long *ck, int *status, int grid_cap,
-                                       uint32_t item_bytes, cudaStream_t stream)
+                                       uint32_t item_bytes, const cfa_launch_ctl *ctl, cudaStream_t stream)
 {
     if (n_ranges > 4 || grid_cap <= 0) return cudaErrorInvalidValue;
     BulkArgs a{};
@@ -402,8 +412,8 @@ extern "C" cudaError_t cfa_launch_bulk(const cfa_bulk_range *ranges, uint32_t n_
     a.ck = ck;
     a.status = status;
     const uint32_t grid = a.n_items < (uint32_t)grid_cap ? a.n_items : (uint32_t)grid_cap;
-    cfa_bulk_kernel<<<grid, kThreads, kSmemBytes, stream>>>(a);
-    return cudaGetLastError();
+    a.ctl = ctl ? *ctl : cfa_launch_ctl{};
+    return launch_ctl(cfa_bulk_kernel, grid, kThreads, kSmemBytes, stream, a);
 }
 
 /* Self-test of the bounded waits: one CTA of the TMA kernel over one valid 16-byte item, with a

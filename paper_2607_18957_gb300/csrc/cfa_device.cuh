@@ -8,6 +8,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include "cfa_internal.h"
+
 namespace cfa_dev {
 
 /* Sum of the elements of one 16-byte vector of ES-byte unsigned elements. */
@@ -30,6 +32,49 @@ template <> __device__ __forceinline__ uint64_t vsum<4>(uint4 v)
 template <> __device__ __forceinline__ uint64_t vsum<8>(uint4 v)
 {
     return (((uint64_t)v.y << 32) | v.x) + (((uint64_t)v.w << 32) | v.z);
+}
+
+/* First thing of a kernel, every thread: the launch's place in its stream (cfa_launch_ctl).
+ * Dependents are released only after the wait, so that a later kernel of the group, which does
+ * not wait for the source itself, cannot start before the source is there. */
+__device__ __forceinline__ void launch_begin(const cfa_launch_ctl &c)
+{
+    if (c.flags & CFA_LAUNCH_WAIT_FIRST) asm volatile("griddepcontrol.wait;" ::: "memory");
+    if (c.flags & CFA_LAUNCH_RELEASE)
+        asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    if (c.clear) {
+        const uint64_t n = (uint64_t)gridDim.x * blockDim.x;
+        uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
+        for (; i < c.clear_words; i += n) c.clear[i] = 0;
+    }
+}
+
+/* Last thing of a kernel: one CTA that waits for the kernel before keeps the whole grid from
+ * ending first. */
+__device__ __forceinline__ void launch_end(const cfa_launch_ctl &c)
+{
+    if ((c.flags & CFA_LAUNCH_WAIT_LAST) && blockIdx.x == 0)
+        asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+
+/* Host side: launches fn(args) as the ctl in its arguments says. */
+template <typename Args>
+inline cudaError_t launch_ctl(void (*fn)(const Args), unsigned grid, unsigned threads, size_t smem,
+                              cudaStream_t stream, const Args &args)
+{
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = dim3(threads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = stream;
+    cudaLaunchAttribute attr = {};
+    if (args.ctl.flags & CFA_LAUNCH_EARLY) {
+        attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        attr.val.programmaticStreamSerializationAllowed = 1;
+        cfg.attrs = &attr;
+        cfg.numAttrs = 1;
+    }
+    return cudaLaunchKernelEx(&cfg, fn, args);
 }
 
 /* Sum over the 32 lanes of a warp; lane 0 holds the total. */

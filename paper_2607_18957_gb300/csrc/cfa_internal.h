@@ -159,6 +159,30 @@ static inline uint32_t cfa_parts_log2(uint32_t n_items, uint32_t grid_cap, uint3
     return k;
 }
 
+/*
+ * How a kernel launch follows the one before it on its stream (programmatic dependent launch),
+ * and what it clears before its work.
+ *   EARLY       may start once the kernel before it on the stream has released its dependents
+ *               (launch attribute) instead of after it has ended
+ *   WAIT_FIRST  the kernel waits for the end of everything before it on the stream before it reads
+ *               a source, writes, or releases its own dependents
+ *   WAIT_LAST   the kernel does not need the one before it (they write disjoint bytes and add
+ *               checksums atomically) but ends only after it, so that whatever follows on the
+ *               stream follows both
+ *   RELEASE     the kernel releases its dependents as soon as its CTAs run
+ * clear: words set to zero by this launch (the checksum half of the next load), or NULL.
+ */
+#define CFA_LAUNCH_EARLY 1u
+#define CFA_LAUNCH_WAIT_FIRST 2u
+#define CFA_LAUNCH_WAIT_LAST 4u
+#define CFA_LAUNCH_RELEASE 8u
+typedef struct cfa_launch_ctl {
+    unsigned long long *clear;
+    uint64_t clear_words;
+    uint32_t flags;
+    uint32_t pad;
+} cfa_launch_ctl;
+
 /* Sets the calling thread's detail string returned by cfa_last_error(NULL). */
 void cfa_internal_set_error(const char *msg);
 

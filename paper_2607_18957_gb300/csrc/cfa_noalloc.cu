@@ -41,7 +41,7 @@ extern "C" cudaError_t cfa_launch_unpack(int cls, const cfa_work *slabs, uint32_
                                          uint64_t src_lo, uint64_t src_hi,
                                          unsigned long long *ck, int *status, int grid_cap,
                                          uint32_t item_bytes, int dev_src,
-                                         cudaStream_t stream);
+                                         const cfa_launch_ctl *ctl, cudaStream_t stream);
 
 namespace {
 
@@ -330,7 +330,7 @@ extern "C" cfa_status cfa_unpack_noalloc(const cfa_tensor_entry *entries, size_t
                               scratch->items + base[k][1], count[k][1],
                               (uint64_t)(uintptr_t)blob_dev, 0, 0, blob_bytes,
                               reinterpret_cast<unsigned long long *>(cksum_dev), status,
-                              g_grid_cap[dev][k], (uint32_t)kSlabBytes, 1, stream);
+                              g_grid_cap[dev][k], (uint32_t)kSlabBytes, 1, nullptr, stream);
     }
     if (e != cudaSuccess) {
         say("cfa_unpack_noalloc: CUDA error %s", cudaGetErrorString(e));

@@ -49,12 +49,12 @@ extern "C" cudaError_t cfa_launch_strided(int cls, const cfa_swork *items, uint3
                                           uint64_t src_base, uint64_t src_period,
                                           uint64_t src_lo, uint64_t src_hi,
                                           unsigned long long *ck, int *status, int grid_cap,
-                                          cudaStream_t stream);
+                                          const cfa_launch_ctl *ctl, cudaStream_t stream);
 extern "C" cudaError_t cfa_launch_bulk(const cfa_bulk_range *ranges, uint32_t n_ranges,
                                        uint64_t src_base, uint64_t src_period,
                                        uint64_t src_lo, uint64_t src_hi,
                                        unsigned long long *ck, int *status, int grid_cap,
-                                       uint32_t item_bytes, cudaStream_t stream);
+                                       uint32_t item_bytes, const cfa_launch_ctl *ctl, cudaStream_t stream);
 extern "C" cudaError_t cfa_bulk_selftest_timeout(int *status_host);
 extern "C" cudaError_t cfa_launch_pull(const void *src, void *dst, uint64_t bytes, int grid,
                                        cudaStream_t stream);
@@ -64,7 +64,7 @@ extern "C" cudaError_t cfa_launch_unpack(int cls, const cfa_work *slabs, uint32_
                                          uint64_t src_lo, uint64_t src_hi,
                                          unsigned long long *ck, int *status, int grid_cap,
                                          uint32_t item_bytes, int dev_src,
-                                         cudaStream_t stream);
+                                         const cfa_launch_ctl *ctl, cudaStream_t stream);
 
 namespace {
 
@@ -109,9 +109,6 @@ inline size_t ck_clear_bytes(size_t n_entries)
 
 } // namespace
 
-/* Kernels of one launch group beyond the first run on up to this many side streams. */
-constexpr int kSideStreams = 2;
-
 struct cfa_plan {
     cfa_host_plan hp{};
     bool host_only = false;
@@ -123,16 +120,17 @@ struct cfa_plan {
     cfa_work *d_slabs = nullptr, *d_tiny = nullptr, *d_bulk = nullptr;
     cfa_swork *d_strided = nullptr;
     /* Two halves of checksums + status word: a load accumulates into the half cleared before
-     * it began and clears the other half, its predecessor's, on ck_stream beside its own work,
-     * so no clear sits between a load's start and its first kernel.  d_ck / d_status point into
-     * the half of the last load (or of cfa_unpack_chunks_async and cfa_reset_checksums). */
+     * it began, and its first kernel clears the other half, its predecessor's, so no clear and
+     * no second stream sits between a load's start and its first kernel.  d_ck / d_status point
+     * into the half of the last load (or of cfa_unpack_chunks_async and cfa_reset_checksums);
+     * ck_clear is the half still to be cleared by the load being enqueued. */
     unsigned long long *d_ck_mem = nullptr;
     size_t ck_half_words = 0;
     int ck_half = 0;
     unsigned long long *d_ck = nullptr;
     int *d_status = nullptr;
-    cudaStream_t ck_stream = nullptr;
-    cudaEvent_t ev_ck_clear = nullptr;
+    unsigned long long *ck_clear = nullptr;
+    uint64_t ck_clear_words = 0;
     uint8_t *d_slots = nullptr;
     bool own_slots = false;
     uint64_t slot_bytes = 0;
@@ -140,9 +138,6 @@ struct cfa_plan {
     uint8_t *h_slots = nullptr;
     int n_host_slots = 0;
     cudaStream_t fill_stream = nullptr, copy_stream = nullptr, aux_stream = nullptr;
-    /* side streams that run a launch group's other kernels beside the caller's stream */
-    cudaStream_t side_stream[kSideStreams] = {nullptr};
-    cudaEvent_t ev_fork = nullptr, ev_join[kSideStreams] = {nullptr};
     /* pinned sources: column slices read in place over the host link, beside the copy ring */
     cudaStream_t direct_stream = nullptr;
     cudaEvent_t ev_direct = nullptr;
@@ -166,6 +161,10 @@ struct cfa_plan {
      * experts unread, keeps its copy stream busy instead of cycling slots through them. */
     std::vector<uint8_t> chunk_busy;
     std::vector<uint32_t> layers_empty;
+    /* per layer: the event of the last load after which the layer is ready.  Layers that become
+     * ready at the same point of the stream share one event (ev_layer of the first of them, or
+     * ev_all), so a load records one event per such point and not one per layer. */
+    std::unique_ptr<std::atomic<cudaEvent_t>[]> layer_ready;
     std::unique_ptr<cfa::Pool> pool;
     std::vector<std::unique_ptr<LoadCtx>> loads;
     LoadCtx *last = nullptr;
@@ -275,17 +274,21 @@ void CUDART_CB fill_host_fn(void *arg)
 /* Unpacks chunks [c0, c1), whose blob byte o sits at device address src_base + o (or
  * src_base + (o mod period) for a periodic source): one TMA bulk launch for the aligned cast-free
  * slabs of every element size, and per work class present in those chunks (normally one) a launch
- * for its column slices and a vector launch for everything else.  The kernels of one group write disjoint
- * destination bytes and add their checksums atomically, so they are independent: the first
- * runs on `s`, the others on side streams forked from `s` and joined back into it, so that
- * one kernel's last CTAs overlap the next kernel's first instead of the GPU draining between
- * them.  With tma = false (a source in host memory, read over the host link) the aligned slabs
- * planned for the TMA kernel are copied by the vector kernel instead: bulk copies are for
- * device memory.  grid_div > 1 divides every kernel's grid cap by it. */
+ * for its column slices and a vector launch for everything else.  The kernels of one group write
+ * disjoint destination bytes and add their checksums atomically, so they are independent: each
+ * releases the next as soon as it runs, so that one kernel's last CTAs overlap the next kernel's
+ * first, and ends only after the one before it, so that what follows on `s` follows them all.
+ * (Side streams forked and joined with events did the same for 2-3 us more per extra kernel.)
+ * With early = true the group's first kernel too is launched while the kernel before it on `s`
+ * still runs, and waits for its end inside (consecutive chunks of a caller's own staging).  With
+ * tma = false (a source in host memory, read over the host link) the aligned slabs planned for the
+ * TMA kernel are copied by the vector kernel instead: bulk copies are for device memory.
+ * grid_div > 1 divides every kernel's grid cap by it. */
 enum { LAUNCH_CONTIG = 1, LAUNCH_STRIDED = 2, LAUNCH_ALL = 3 };
 
 cfa_status launch(cfa_plan *p, uint32_t c0, uint32_t c1, uint64_t src_base, uint64_t period,
-                  cudaStream_t s, bool tma = true, int what = LAUNCH_ALL, int grid_div = 1)
+                  cudaStream_t s, bool tma = true, int what = LAUNCH_ALL, int grid_div = 1,
+                  bool early = false)
 {
     auto cap = [grid_div](int c) { return std::max(1, c / grid_div); };
     const cfa_host_plan &hp = p->hp;
@@ -318,49 +321,61 @@ cfa_status launch(cfa_plan *p, uint32_t c0, uint32_t c1, uint64_t src_base, uint
         const uint32_t t0 = hp.tiny_first[k * row + c0], t1 = hp.tiny_first[k * row + c1];
         if (s1 != s0 || t1 != t0) jobs[n++] = Job{VECTOR, k, s0, s1, t0, t1};
     }
-    const int n_side = std::min(n - 1, kSideStreams);
-    if (n_side > 0) {
-        CK(p, cudaEventRecord(p->ev_fork, s));
-        for (int j = 0; j < n_side; ++j) CK(p, cudaStreamWaitEvent(p->side_stream[j], p->ev_fork, 0));
-    }
     for (int i = 0; i < n; ++i) {
         const Job &J = jobs[i];
         const int k = J.k;
-        cudaStream_t ls = i == 0 ? s : p->side_stream[(i - 1) % kSideStreams];
         const bool timing = timing_on && p->last_launches < p->t_k0.size();
+        /* timed launches run one after the other, so that each interval is that kernel's alone */
+        cfa_launch_ctl ctl{};
+        if (!timing) {
+            if (i > 0) ctl.flags |= CFA_LAUNCH_EARLY | CFA_LAUNCH_WAIT_LAST;
+            else if (early) ctl.flags |= CFA_LAUNCH_EARLY | CFA_LAUNCH_WAIT_FIRST;
+            if (i + 1 < n || early) ctl.flags |= CFA_LAUNCH_RELEASE;
+        }
+        ctl.clear = p->ck_clear;
+        ctl.clear_words = p->ck_clear_words;
         if (timing) {
-            CK(p, cudaEventRecord(p->t_k0[p->last_launches], ls));
+            CK(p, cudaEventRecord(p->t_k0[p->last_launches], s));
             p->t_k_c0[p->last_launches] = c0;
             p->t_k_c1[p->last_launches] = c1;
         }
         if (J.type == BULK)
             CK(p, cfa_launch_bulk(ranges, n_ranges, src_base, period, lo, hi, p->d_ck,
-                                  p->d_status, cap(p->bulk_grid_cap), hp.opts.slab_bytes, ls));
+                                  p->d_status, cap(p->bulk_grid_cap), hp.opts.slab_bytes, &ctl,
+                                  s));
         else if (J.type == BULK_AS_VECTOR) /* bulk items are copy-class slabs of class k */
             CK(p, cfa_launch_unpack(k, p->d_bulk + J.a0, J.a1 - J.a0, nullptr, 0, src_base,
                                     period, lo, hi, p->d_ck, p->d_status, cap(p->grid_cap[k]),
-                                    hp.opts.slab_bytes, tma, ls));
+                                    hp.opts.slab_bytes, tma, &ctl, s));
         else if (J.type == STRIDED)
             CK(p, cfa_launch_strided(k, p->d_strided + J.a0, J.a1 - J.a0, src_base, period, lo,
-                                     hi, p->d_ck, p->d_status, cap(p->strided_grid_cap[k]), ls));
+                                     hi, p->d_ck, p->d_status, cap(p->strided_grid_cap[k]),
+                                     &ctl, s));
         else
             CK(p, cfa_launch_unpack(k, p->d_slabs + J.a0, J.a1 - J.a0, p->d_tiny + J.b0,
                                     J.b1 - J.b0, src_base, period, lo, hi, p->d_ck, p->d_status,
-                                    cap(p->grid_cap[k]), hp.opts.slab_bytes, tma, ls));
-        if (timing) CK(p, cudaEventRecord(p->t_k1[p->last_launches], ls));
+                                    cap(p->grid_cap[k]), hp.opts.slab_bytes, tma, &ctl, s));
+        p->ck_clear = nullptr; /* this launch clears it */
+        p->ck_clear_words = 0;
+        if (timing) CK(p, cudaEventRecord(p->t_k1[p->last_launches], s));
         p->last_launches++;
-    }
-    for (int j = 0; j < n_side; ++j) {
-        CK(p, cudaEventRecord(p->ev_join[j], p->side_stream[j]));
-        CK(p, cudaStreamWaitEvent(s, p->ev_join[j], 0));
     }
     return CFA_OK;
 }
 
-cfa_status record_layers(cfa_plan *p, uint32_t c0, uint32_t c1, cudaStream_t s)
+/* Layers whose last chunk is in [c0, c1) are ready at this point of `s`: one event for them all,
+ * or none when the caller records `shared` here itself. */
+cfa_status record_layers(cfa_plan *p, uint32_t c0, uint32_t c1, cudaStream_t s,
+                         cudaEvent_t shared = nullptr)
 {
     for (uint32_t c = c0; c < c1; ++c)
-        for (uint32_t l : p->layers_ending[c]) CK(p, cudaEventRecord(p->ev_layer[l], s));
+        for (uint32_t l : p->layers_ending[c]) {
+            if (!shared) {
+                shared = p->ev_layer[l];
+                CK(p, cudaEventRecord(shared, s));
+            }
+            p->layer_ready[l].store(shared, std::memory_order_release);
+        }
     return CFA_OK;
 }
 
@@ -387,7 +402,6 @@ void release(cfa_plan *p)
         if (p->copy_stream) cudaStreamSynchronize(p->copy_stream);
         if (p->ev_all) cudaEventSynchronize(p->ev_all);
         if (p->aux_stream) cudaStreamSynchronize(p->aux_stream);
-        if (p->ck_stream) cudaStreamSynchronize(p->ck_stream);
         auto kill = [](std::vector<cudaEvent_t> &v) {
             for (cudaEvent_t e : v)
                 if (e) cudaEventDestroy(e);
@@ -408,17 +422,9 @@ void release(cfa_plan *p)
         kill(p->t_k1);
         if (p->ev_begin) cudaEventDestroy(p->ev_begin);
         if (p->ev_all) cudaEventDestroy(p->ev_all);
-        if (p->ev_fork) cudaEventDestroy(p->ev_fork);
-        if (p->ev_ck_clear) cudaEventDestroy(p->ev_ck_clear);
-        if (p->ck_stream) cudaStreamDestroy(p->ck_stream);
         if (p->direct_stream) cudaStreamSynchronize(p->direct_stream);
         if (p->ev_direct) cudaEventDestroy(p->ev_direct);
         if (p->direct_stream) cudaStreamDestroy(p->direct_stream);
-        for (int j = 0; j < kSideStreams; ++j) {
-            if (p->side_stream[j]) cudaStreamSynchronize(p->side_stream[j]);
-            if (p->ev_join[j]) cudaEventDestroy(p->ev_join[j]);
-            if (p->side_stream[j]) cudaStreamDestroy(p->side_stream[j]);
-        }
         if (p->fill_stream) cudaStreamDestroy(p->fill_stream);
         if (p->copy_stream) cudaStreamDestroy(p->copy_stream);
         if (p->gather_stream) cudaStreamDestroy(p->gather_stream);
@@ -538,13 +544,6 @@ cfa_status setup_device(cfa_plan *p)
     CK(nullptr, cudaStreamCreateWithFlags(&p->fill_stream, cudaStreamNonBlocking));
     CK(nullptr, cudaStreamCreateWithFlags(&p->copy_stream, cudaStreamNonBlocking));
     CK(nullptr, cudaStreamCreateWithFlags(&p->aux_stream, cudaStreamNonBlocking));
-    CK(nullptr, cudaStreamCreateWithFlags(&p->ck_stream, cudaStreamNonBlocking));
-    if ((st = make_event(nullptr, &p->ev_ck_clear, false))) return st;
-    for (int j = 0; j < kSideStreams; ++j) {
-        CK(nullptr, cudaStreamCreateWithFlags(&p->side_stream[j], cudaStreamNonBlocking));
-        if ((st = make_event(nullptr, &p->ev_join[j], false))) return st;
-    }
-    if ((st = make_event(nullptr, &p->ev_fork, false))) return st;
     CK(nullptr, cudaStreamCreateWithFlags(&p->direct_stream, cudaStreamNonBlocking));
     if ((st = make_event(nullptr, &p->ev_direct, false))) return st;
     const bool timing = (o.flags & CFA_OPT_TIMING) != 0;
@@ -569,6 +568,8 @@ cfa_status setup_device(cfa_plan *p)
     if ((st = events(p->ev_host_free, p->n_host_slots, false))) return st;
     if ((st = events(p->ev_filled, p->n_host_slots, false))) return st;
     if ((st = events(p->ev_layer, hp.n_layers, timing))) return st;
+    p->layer_ready.reset(new std::atomic<cudaEvent_t>[hp.n_layers]);
+    for (uint32_t l = 0; l < hp.n_layers; ++l) p->layer_ready[l].store(p->ev_layer[l]);
     if ((st = make_event(nullptr, &p->ev_begin, timing))) return st;
     if ((st = make_event(nullptr, &p->ev_all, timing))) return st;
     if (timing) {
@@ -815,27 +816,45 @@ cfa_status cfa_load_async(cfa_plan *p, const cfa_source *src, cfa_stream stream_
     p->last_h2d = 0;
     const bool timing = (hp.opts.flags & CFA_OPT_TIMING) != 0;
 
-    /* the load starts after the previous load of this plan, after prior work on cs and after
-     * the clear of the checksum half it takes; it clears the other half for the next load */
+    /* the load starts after the previous load of this plan and after prior work on cs.  A source
+     * read in place needs no other stream, so the event that starts them is recorded only for the
+     * staged kinds (and for timing). */
     CK(p, cudaStreamWaitEvent(cs, p->ev_all, 0));
-    CK(p, cudaStreamWaitEvent(cs, p->ev_ck_clear, 0));
-    CK(p, cudaEventRecord(p->ev_begin, cs));
-    CK(p, cudaStreamWaitEvent(p->fill_stream, p->ev_begin, 0));
-    CK(p, cudaStreamWaitEvent(p->copy_stream, p->ev_begin, 0));
-    {
-        /* the half the previous load used is cleared for the next load; this load switches to
-         * the other one only once that clear is enqueued, so a load that fails here leaves the
-         * clean half for the next */
-        unsigned long long *prev = p->d_ck;
-        CK(p, cudaStreamWaitEvent(p->ck_stream, p->ev_begin, 0));
-        if (hp.any_cksum)
-            CK(p, cudaMemsetAsync(prev, 0, ck_clear_bytes(hp.n_entries), p->ck_stream));
-        else
-            CK(p, cudaMemsetAsync(prev + (p->ck_half_words - 1), 0, sizeof(int), p->ck_stream));
-        CK(p, cudaEventRecord(p->ev_ck_clear, p->ck_stream));
-        use_ck_half(p, p->ck_half ^ 1);
+    if (!in_place || timing) CK(p, cudaEventRecord(p->ev_begin, cs));
+    if (!in_place) {
+        CK(p, cudaStreamWaitEvent(p->fill_stream, p->ev_begin, 0));
+        CK(p, cudaStreamWaitEvent(p->copy_stream, p->ev_begin, 0));
     }
-    for (uint32_t l : p->layers_empty) CK(p, cudaEventRecord(p->ev_layer[l], cs));
+    /* the half the previous load used is cleared for the next load by this load's first kernel;
+     * a load that fails before it has launched one leaves the clean half for the next */
+    struct CkSwitch {
+        cfa_plan *p;
+        int prev;
+        explicit CkSwitch(cfa_plan *p_) : p(p_), prev(p_->ck_half)
+        {
+            const bool all = p->hp.any_cksum != 0;
+            p->ck_clear = all ? p->d_ck : p->d_ck + (p->ck_half_words - 1);
+            p->ck_clear_words = all ? p->ck_half_words : 1;
+            use_ck_half(p, prev ^ 1);
+        }
+        ~CkSwitch()
+        {
+            if (!p->ck_clear) return;
+            p->ck_clear = nullptr;
+            p->ck_clear_words = 0;
+            use_ck_half(p, prev);
+        }
+    } ck_switch(p);
+    {
+        cudaEvent_t shared = nullptr; /* layers without bytes are ready where the load starts */
+        for (uint32_t l : p->layers_empty) {
+            if (!shared) {
+                shared = p->ev_layer[l];
+                CK(p, cudaEventRecord(shared, cs));
+            }
+            p->layer_ready[l].store(shared, std::memory_order_release);
+        }
+    }
 
     if (in_place) {
         /* the kernel reads the blob where it is: device memory (one launch over all chunks per
@@ -850,7 +869,9 @@ cfa_status cfa_load_async(cfa_plan *p, const cfa_source *src, cfa_stream stream_
             cfa_status st =
                 launch(p, c0, c1, base, src->period_bytes, cs, kind == CFA_SRC_DEVICE);
             if (st) return st;
-            if ((st = record_layers(p, c0, c1, cs))) return st;
+            /* the load's end follows the last run directly: its event serves the layers there */
+            if ((st = record_layers(p, c0, c1, cs, c1 == hp.n_chunks ? p->ev_all : nullptr)))
+                return st;
             c0 = c1;
         }
     } else {
@@ -1031,6 +1052,11 @@ cfa_status cfa_load_async(cfa_plan *p, const cfa_source *src, cfa_stream stream_
             if ((st = record_layers(p, c, c + 1, cs))) return st;
         }
     }
+    if (p->ck_clear) { /* no kernel was launched */
+        CK(p, cudaMemsetAsync(p->ck_clear, 0, p->ck_clear_words * sizeof(unsigned long long), cs));
+        p->ck_clear = nullptr;
+        p->ck_clear_words = 0;
+    }
     CK(p, cudaEventRecord(p->ev_all, cs));
     logf("load %llu enqueued: source kind %d, %llu kernel launches, %u staged chunks",
          (unsigned long long)p->n_loads, kind, (unsigned long long)p->last_launches, p->last_h2d);
@@ -1046,7 +1072,8 @@ cfa_status cfa_wait_layer(cfa_plan *p, int32_t layer, cfa_stream consumer, int64
     }
     cudaEvent_t ev;
     if (layer == CFA_ALL) ev = p->ev_all;
-    else if (layer >= 0 && (uint32_t)layer < p->hp.n_layers) ev = p->ev_layer[layer];
+    else if (layer >= 0 && (uint32_t)layer < p->hp.n_layers)
+        ev = p->layer_ready[layer].load(std::memory_order_acquire);
     else {
         set_err(p, "unknown readiness group %d", layer);
         return CFA_ERR_INVAL;
@@ -1138,7 +1165,7 @@ cfa_status cfa_get_layer_times(cfa_plan *p, float *ms_out, size_t n)
     DeviceGuard g(p->device);
     CK(p, cudaEventSynchronize(p->ev_all));
     for (size_t l = 0; l < n; ++l)
-        CK(p, cudaEventElapsedTime(&ms_out[l], p->ev_begin, p->ev_layer[l]));
+        CK(p, cudaEventElapsedTime(&ms_out[l], p->ev_begin, p->layer_ready[l].load()));
     return CFA_OK;
 }
 
@@ -1209,7 +1236,8 @@ cfa_status cfa_unpack_chunks_async(cfa_plan *p, uint32_t chunk_begin, uint32_t c
     const uint64_t saved = p->last_launches;
     p->last_launches = p->t_k0.size(); /* no timing events for direct launches */
     cfa_status st =
-        launch(p, chunk_begin, chunk_end, base, 0, reinterpret_cast<cudaStream_t>(stream));
+        launch(p, chunk_begin, chunk_end, base, 0, reinterpret_cast<cudaStream_t>(stream), true,
+               LAUNCH_ALL, 1, true);
     p->last_launches = saved;
     return st;
 }

@@ -31,6 +31,9 @@
 
 namespace {
 
+using cfa_dev::launch_begin;
+using cfa_dev::launch_ctl;
+using cfa_dev::launch_end;
 using cfa_dev::vsum;
 using cfa_dev::warp_sum;
 
@@ -68,6 +71,7 @@ struct UnpackArgs {
     unsigned long long *ck;
     int *status;
     uint32_t dev_src;    /* 1: the source is device memory (staging slots or a device blob) */
+    cfa_launch_ctl ctl;
 };
 
 /* ---- memory operations ------------------------------------------------------------------ */
@@ -661,6 +665,7 @@ __global__ void __launch_bounds__(kThreads, unpack_min_blocks(CLS))
     cfa_unpack_kernel(const UnpackArgs a)
 {
     __shared__ unsigned long long red[kWarps];
+    launch_begin(a.ctl);
     const uint32_t n_groups = (a.n_tiny + kTinyPerGroup - 1) / kTinyPerGroup;
     const uint32_t n_slabs = a.n_slabs << a.parts_log2; /* parts of slabs */
     const uint32_t n_items = n_slabs + n_groups;
@@ -705,6 +710,7 @@ __global__ void __launch_bounds__(kThreads, unpack_min_blocks(CLS))
         }
     }
     if (acc_ck != CFA_NO_CK) block_flush(acc, acc_ck, a.ck, red);
+    launch_end(a.ctl);
 }
 
 /* A launch of tiny pieces only (no block-level items).  A tiny piece is bound by latency, not
@@ -1072,11 +1078,13 @@ template <int CLS>
 __global__ void __launch_bounds__(kThreads, (CLS == 0 ? kCopyMinBlocks : unpack_min_blocks(CLS)))
     cfa_tiny_kernel(const UnpackArgs a)
 {
+    launch_begin(a.ctl);
     if constexpr (CLS < 4) {
         /* device-memory sources take the shared-memory pipeline; host memory read in place over
          * the link keeps plain loads */
         if (a.dev_src) {
             tiny_staged<CLS>(a);
+            launch_end(a.ctl);
             return;
         }
     }
@@ -1119,6 +1127,7 @@ __global__ void __launch_bounds__(kThreads, (CLS == 0 ? kCopyMinBlocks : unpack_
         w = wn;
         group = next;
     }
+    launch_end(a.ctl);
 }
 
 /* ---- host -> device pull over the host link --------------------------------------------- */
@@ -1162,6 +1171,7 @@ struct StridedArgs {
     uint64_t src_lo, src_hi;
     unsigned long long *ck;
     int *status;
+    cfa_launch_ctl ctl;
 };
 
 template <int CLS>
@@ -1189,6 +1199,7 @@ __global__ void __launch_bounds__(kThreads, (CLS == 0 || ClassOf<CLS>::ses == 2
     constexpr int DES = C::des;
     __shared__ unsigned long long red[kWarps];
     const uint32_t lane = threadIdx.x & 31u, warp = threadIdx.x >> 5;
+    launch_begin(a.ctl);
     uint64_t acc = 0;
     uint32_t acc_ck = CFA_NO_CK;
     for (uint32_t item = blockIdx.x; item < a.n_items; item += gridDim.x) {
@@ -1217,6 +1228,7 @@ __global__ void __launch_bounds__(kThreads, (CLS == 0 || ClassOf<CLS>::ses == 2
         }
     }
     if (acc_ck != CFA_NO_CK) block_flush(acc, acc_ck, a.ck, red);
+    launch_end(a.ctl);
 }
 
 typedef void (*strided_fn)(const StridedArgs);
@@ -1273,7 +1285,7 @@ extern "C" cudaError_t cfa_launch_unpack(int cls, const cfa_work *slabs, uint32_
                                          uint64_t src_lo, uint64_t src_hi,
                                          unsigned long long *ck, int *status, int grid_cap,
                                          uint32_t item_bytes, int dev_src,
-                                         cudaStream_t stream)
+                                         const cfa_launch_ctl *ctl, cudaStream_t stream)
 {
     if (cls < 0 || cls >= CFA_N_CLASSES || grid_cap <= 0) return cudaErrorInvalidValue;
     /* the fp32 -> 16-bit classes read twice what they write */
@@ -1297,6 +1309,7 @@ extern "C" cudaError_t cfa_launch_unpack(int cls, const cfa_work *slabs, uint32_
     a.ck = ck;
     a.status = status;
     a.dev_src = dev_src ? 1u : 0u;
+    a.ctl = ctl ? *ctl : cfa_launch_ctl{};
     const uint64_t grid = items < (uint64_t)grid_cap ? items : (uint64_t)grid_cap;
     /* tiny pieces alone take the tiny kernel (same occupancy class as the combined one, so the
      * same grid cap holds); its copy classes stage device-memory sources in dynamic shared
@@ -1307,11 +1320,10 @@ extern "C" cudaError_t cfa_launch_unpack(int cls, const cfa_work *slabs, uint32_
             cudaError_t e = tiny_smem_ready(cls);
             if (e != cudaSuccess) return e;
         }
-        kTiny[cls]<<<(unsigned)grid, kThreads, staged ? kStagedSmem : 0, stream>>>(a);
-    } else {
-        kKernels[cls]<<<(unsigned)grid, kThreads, 0, stream>>>(a);
+        return launch_ctl(kTiny[cls], (unsigned)grid, kThreads, staged ? kStagedSmem : 0, stream,
+                          a);
     }
-    return cudaGetLastError();
+    return launch_ctl(kKernels[cls], (unsigned)grid, kThreads, 0, stream, a);
 }
 
 /* Pulls `bytes` from host memory at src into device memory at dst (same offset within 16
@@ -1343,7 +1355,7 @@ extern "C" cudaError_t cfa_launch_strided(int cls, const cfa_swork *items, uint3
                                           uint64_t src_base, uint64_t src_period,
                                           uint64_t src_lo, uint64_t src_hi,
                                           unsigned long long *ck, int *status, int grid_cap,
-                                          cudaStream_t stream)
+                                          const cfa_launch_ctl *ctl, cudaStream_t stream)
 {
     if (cls < 0 || cls >= CFA_N_CLASSES || grid_cap <= 0) return cudaErrorInvalidValue;
     if (n_items == 0) return cudaSuccess;
@@ -1357,7 +1369,7 @@ extern "C" cudaError_t cfa_launch_strided(int cls, const cfa_swork *items, uint3
     a.src_hi = src_hi;
     a.ck = ck;
     a.status = status;
+    a.ctl = ctl ? *ctl : cfa_launch_ctl{};
     const uint32_t grid = n_items < (uint32_t)grid_cap ? n_items : (uint32_t)grid_cap;
-    kStrided[cls]<<<grid, kThreads, 0, stream>>>(a);
-    return cudaGetLastError();
+    return launch_ctl(kStrided[cls], grid, kThreads, 0, stream, a);
 }

@@ -1,5 +1,7 @@
-"""How launches are cut: block-level items cut into parts where a launch has few of them (sizes
-around the parts, sources and destinations at odd phases).  Checked against slices of the blob."""
+"""How launches are cut and chained: block-level items cut into parts where a launch has few of
+them (sizes around the parts, sources and destinations at odd phases), one TMA launch over several
+element sizes, and chunks unpacked one after the other from a staging slot that the caller
+overwrites in between, on a stream and in a CUDA graph.  Checked against slices of the blob."""
 import ctypes
 
 import numpy as np
@@ -87,3 +89,48 @@ def test_noalloc_items_are_cut_into_parts():
     assert int(status.item()) == 0
     assert torch.equal(c.out, c.want)
     assert np.array_equal(ck.cpu().numpy().view(np.uint64), c.checksums())
+
+
+def chunk_plan(c, chunk):
+    return cfa.Plan(c.entries, c.dsts, c.blob_bytes, chunk_bytes=chunk, dev_slots=0, host_slots=0)
+
+
+def unpack_through_one_slot(c, plan, chunk, slot):
+    for k in range(plan.info()["n_chunks"]):
+        part = c.blob[k * chunk:(k + 1) * chunk]
+        slot[:part.numel()].copy_(part)  # a kernel or a copy that the unpack has to wait for
+        slot[:part.numel()].bitwise_xor_(0xFF).bitwise_xor_(0xFF)
+        plan.unpack_chunks_async(k, k + 1, slot.data_ptr())
+
+
+@pytest.mark.parametrize("chunk", [1 << 20, 8 << 20])
+def test_chunks_through_one_slot_that_is_overwritten(chunk):
+    c = Copies(tensors(SIZES + [96, 5000], [(0, 0), (1, 3)]))
+    slot = torch.empty(chunk, dtype=torch.uint8, device="cuda")
+    with chunk_plan(c, chunk) as plan:
+        for _ in range(3):
+            c.out.fill_(0xA5)
+            plan.reset_checksums()
+            unpack_through_one_slot(c, plan, chunk, slot)
+            assert torch.equal(c.out, c.want)
+
+
+def test_consecutive_chunks_in_a_cuda_graph():
+    chunk = 4 << 20
+    c = Copies(tensors(SIZES + [96, 5000], [(0, 0), (1, 3)]))
+    slot = torch.empty(chunk, dtype=torch.uint8, device="cuda")
+    with chunk_plan(c, chunk) as plan:
+        unpack_through_one_slot(c, plan, chunk, slot)
+        torch.cuda.synchronize()
+        graph = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(graph):
+            plan.reset_checksums()
+            unpack_through_one_slot(c, plan, chunk, slot)
+            for k in range(plan.info()["n_chunks"]):  # and with nothing in between
+                plan.unpack_chunks_async(k, k + 1, c.blob.data_ptr() + k * chunk)
+        for _ in range(2):
+            c.out.fill_(0xA5)
+            graph.replay()
+            torch.cuda.synchronize()
+            assert torch.equal(c.out, c.want)
+        del graph
