@@ -13,6 +13,8 @@
  *     lanes), and one lane issues the bulk store; once the store of the previous sub-block has
  *     finished reading its stage (bulk_group read wait), that stage is released on its `empty`
  *     mbarrier.
+ * An item is a contiguous run, or a block of rows of a column slice: then one bulk load per row
+ * gathers the rows back to back in the stage and one bulk store writes them.
  * One launch takes the items of every element size (the consumer sums each stage by its item's
  * size), cut into parts where there are too few for the grid (cfa_parts_log2).  With a launch per
  * element size, forked and joined with events, and whole 256 KiB slabs, an 8-bit checkpoint with
@@ -48,8 +50,7 @@ constexpr uint32_t kSpinLimit = 1u << 20;              /* try_wait polls before 
 constexpr uint32_t kLoseLoads = 1u << 31;              /* self-test: the loader issues nothing */
 
 struct BulkArgs {
-    cfa_bulk_range range[4]; /* item lists, one per element size present */
-    uint32_t n_ranges;
+    cfa_bulk_range range[CFA_BULK_RANGES]; /* item lists that are not empty */
     uint32_t n_items;    /* parts over all ranges */
     uint32_t parts_log2; /* every item is copied in 2^parts_log2 parts */
     uint32_t spin_limit; /* try_wait polls before a wait gives up; the self-test sets a short one
@@ -138,15 +139,27 @@ __device__ __forceinline__ void mbar_arrive(uint64_t *bar)
     asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_addr(bar)) : "memory");
 }
 
+/* An item of either kind: `rows` rows of `cols` elements, `stride` apart in the source and back to
+ * back in the destination; a contiguous run is one row. */
+struct BulkItem {
+    uint64_t src, dst;
+    uint32_t rows, cols, stride, ck, mode;
+};
+
 /* A bulk item is sound if it is a plain copy, its source lies inside the launch's readable range
- * and source, destination and length are multiples of 16 bytes. */
-__device__ __forceinline__ bool bulk_item_ok(const cfa_work &w, const BulkArgs &a)
+ * and source, destination, rows and row distance are multiples of 16 bytes. */
+__device__ __forceinline__ bool bulk_item_ok(const BulkItem &w, const BulkArgs &a)
 {
-    const uint32_t log2es = w.mode & 3u;
-    const uint64_t bytes = (uint64_t)w.n << log2es;
-    return w.n != 0 && w.mode == CFA_MODE(log2es, log2es, 0) && w.src >= a.src_lo &&
-           w.src <= a.src_hi && bytes <= a.src_hi - w.src && bytes < (1ull << 31) &&
-           ((w.src | w.dst | bytes | a.src_base | a.src_period) & 15u) == 0;
+    const uint32_t l = w.mode & 3u;
+    const uint64_t row = (uint64_t)w.cols << l, pitch = (uint64_t)w.stride << l;
+    if (w.mode != CFA_MODE(l, l, 0) || w.rows == 0 || w.cols == 0 || pitch < row) return false;
+    /* no product overflows: rows and columns below 2^32, so bounded before it is taken */
+    if (row >= (1ull << 31) || w.rows > (1ull << 31) / row) return false;
+    const uint64_t extent = (w.rows - 1) * pitch + row;
+    return w.src >= a.src_lo && w.src <= a.src_hi && extent <= a.src_hi - w.src &&
+           row * w.rows < (1ull << 31) &&
+           ((w.src | w.dst | row | (w.rows > 1 ? pitch : 0) | a.src_base | a.src_period) & 15u) ==
+               0;
 }
 
 /* Bytes [*at, *at + *len) of a checked item of `total` bytes at destination `dst` that are part k
@@ -170,21 +183,31 @@ __device__ __forceinline__ bool bulk_part(uint64_t dst, uint32_t total, uint32_t
 }
 
 /* Descriptor of part `v` of the launch. */
-__device__ __forceinline__ cfa_work bulk_fetch(const BulkArgs &a, uint32_t v)
+__device__ __forceinline__ BulkItem bulk_fetch(const BulkArgs &a, uint32_t v)
 {
     uint32_t i = v >> a.parts_log2;
     int r = 0;
-#pragma unroll
-    for (int q = 0; q < 3; ++q)
-        if (r == q && i >= a.range[q].n && (uint32_t)q + 1u < a.n_ranges) {
-            i -= a.range[q].n;
-            r = q + 1;
-        }
-    const cfa_work *p = a.range[0].items;
-#pragma unroll
-    for (int q = 1; q < 4; ++q)
-        if (r == q) p = a.range[q].items;
-    return p[i];
+    while (i >= a.range[r].n) i -= a.range[r++].n;
+    BulkItem b;
+    if (a.range[r].rows) {
+        const cfa_swork w = static_cast<const cfa_swork *>(a.range[r].items)[i];
+        b.src = w.src;
+        b.dst = w.dst;
+        b.rows = w.rows;
+        b.cols = w.cols;
+        b.stride = w.stride;
+        b.ck = w.ck;
+        b.mode = w.mode;
+    } else {
+        const cfa_work w = static_cast<const cfa_work *>(a.range[r].items)[i];
+        b.src = w.src;
+        b.dst = w.dst;
+        b.rows = 1;
+        b.cols = b.stride = w.n;
+        b.ck = w.ck;
+        b.mode = w.mode;
+    }
+    return b;
 }
 
 /* Sum of a staged sub-block's elements over this lane's vectors: eight independent shared loads
@@ -235,7 +258,7 @@ __global__ void __launch_bounds__(kThreads) cfa_bulk_kernel(const BulkArgs a)
     }
     /* the loader's first two descriptors (the plan's own memory, written before any launch) are
      * on their way while the launch waits for what is before it on the stream */
-    cfa_work w{}, nxt{};
+    BulkItem w{}, nxt{};
     if (threadIdx.x == 0) {
         if (blockIdx.x < a.n_items) w = bulk_fetch(a, blockIdx.x);
         if (blockIdx.x + gridDim.x < a.n_items) nxt = bulk_fetch(a, blockIdx.x + gridDim.x);
@@ -271,7 +294,7 @@ __global__ void __launch_bounds__(kThreads) cfa_bulk_kernel(const BulkArgs a)
                         continue;
                     }
                     uint32_t len;
-                    if (bulk_part(w.dst, w.n << (w.mode & 3u),
+                    if (bulk_part(w.dst, (w.rows * w.cols) << (w.mode & 3u),
                                   it & ((1u << a.parts_log2) - 1u), a.parts_log2, &off, &len)) {
                         end = off + len;
                         break;
@@ -291,16 +314,34 @@ __global__ void __launch_bounds__(kThreads) cfa_bulk_kernel(const BulkArgs a)
                     mbar_arrive(&full[s]);
                     break;
                 }
-                const uint32_t len = min(kStageBytes, end - off);
+                /* of short rows, whole ones: a stage then holds no part of a row */
+                const uint32_t row = w.cols << (w.mode & 3u);
+                uint32_t len = kStageBytes;
+                if (w.rows > 1 && row <= kStageBytes) {
+                    const uint32_t in = off % row;
+                    len = (kStageBytes + in) / row * row - in;
+                }
+                len = min(len, end - off);
                 meta[s].dst = w.dst + off;
                 meta[s].len = len;
                 meta[s].ck = w.ck;
                 meta[s].log2es = w.mode & 3u;
                 mbar_expect_tx(&full[s], len);
                 const uint64_t so = a.src_period ? w.src % a.src_period : w.src;
-                bulk_load(stage + s * kStageBytes,
-                          reinterpret_cast<const uint8_t *>(a.src_base + so) + off, len,
-                          &full[s]);
+                const uint8_t *src = reinterpret_cast<const uint8_t *>(a.src_base + so);
+                if (w.rows == 1) {
+                    bulk_load(stage + s * kStageBytes, src + off, len, &full[s]);
+                } else {
+                    /* the rows, and parts of rows, under [off, off + len), back to back */
+                    uint32_t r = off / row, c = off - r * row;
+                    for (uint32_t at = 0; at < len; ++r, c = 0) {
+                        const uint32_t k = min(row - c, len - at);
+                        bulk_load(stage + s * kStageBytes + at,
+                                  src + ((uint64_t)r * w.stride << (w.mode & 3u)) + c, k,
+                                  &full[s]);
+                        at += k;
+                    }
+                }
                 ++p;
                 n_issued = p;
                 off += len;
@@ -384,20 +425,21 @@ extern "C" int cfa_bulk_blocks_per_sm(void)
     return n;
 }
 
-/* Launches the bulk unpack over up to four lists of items whose source, destination and byte
- * length are multiples of 16; grid_cap bounds the persistent grid. */
+/* Launches the bulk unpack over up to CFA_BULK_RANGES lists of items whose source, destination and
+ * byte length are multiples of 16; grid_cap bounds the persistent grid. */
 extern "C" cudaError_t cfa_launch_bulk(const cfa_bulk_range *ranges, uint32_t n_ranges,
                                        uint64_t src_base, uint64_t src_period,
                                        uint64_t src_lo, uint64_t src_hi,
                                        unsigned long long *ck, int *status, int grid_cap,
-                                       uint32_t item_bytes, const cfa_launch_ctl *ctl, cudaStream_t stream)
+                                       uint32_t item_bytes, const cfa_launch_ctl *ctl,
+                                       cudaStream_t stream)
 {
-    if (n_ranges > 4 || grid_cap <= 0) return cudaErrorInvalidValue;
+    if (n_ranges > CFA_BULK_RANGES || grid_cap <= 0) return cudaErrorInvalidValue;
     BulkArgs a{};
     uint64_t n_items = 0;
-    for (uint32_t r = 0; r < n_ranges; ++r) {
+    for (uint32_t r = 0, k = 0; r < n_ranges; ++r) {
         if (!ranges[r].n) continue;
-        a.range[a.n_ranges++] = ranges[r];
+        a.range[k++] = ranges[r];
         n_items += ranges[r].n;
     }
     if (n_items == 0) return cudaSuccess;
@@ -446,8 +488,7 @@ extern "C" cudaError_t cfa_bulk_selftest_timeout(int *status_host)
         if ((e = cudaMemset(d_status, 0, sizeof(int))) != cudaSuccess) goto out;
         if ((e = cudaMemset(d_ck, 0, sizeof(unsigned long long))) != cudaSuccess) goto out;
         BulkArgs a{};
-        a.range[0] = cfa_bulk_range{d_item, 1};
-        a.n_ranges = 1;
+        a.range[0] = cfa_bulk_range{d_item, 1, 0};
         a.n_items = 1;
         a.spin_limit = 256u | kLoseLoads;
         a.src_base = (uint64_t)(uintptr_t)d_buf;

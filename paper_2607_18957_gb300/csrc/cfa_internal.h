@@ -42,12 +42,6 @@ typedef struct cfa_work {
  * destination addresses that are multiples of it): one 8-lane warp segment copies one item. */
 #define CFA_TINY_SEG_BYTES 512u
 
-/* One of the item lists of a bulk launch (the items of one element size). */
-typedef struct cfa_bulk_range {
-    const cfa_work *items;
-    uint32_t n;
-} cfa_bulk_range;
-
 typedef struct cfa_swork {
     uint64_t src;
     uint64_t dst;
@@ -58,6 +52,22 @@ typedef struct cfa_swork {
     uint32_t mode;
     uint32_t cls;    /* work class, used while the plan is built */
 } cfa_swork;
+
+/* Column slices whose rows hold at least this many bytes, and start and lie at multiples of 16,
+ * go to the TMA kernel (one bulk load a row).  Shorter rows stay with the vector kernel's warps: a
+ * tensor-parallel rank whose attention slices have rows of 2 KiB took 540 us with those rows
+ * there and 556 with them loaded one by one; with rows of 14-28 KiB on the vector kernel another
+ * took 135, and with TMA loads 110. */
+#define CFA_BULK_ROW_BYTES 4096u
+
+/* One of the item lists of a bulk launch: the contiguous runs (cfa_work), or the row blocks
+ * (cfa_swork), of one element size. */
+typedef struct cfa_bulk_range {
+    const void *items;
+    uint32_t n;
+    uint32_t rows; /* 1: cfa_swork */
+} cfa_bulk_range;
+#define CFA_BULK_RANGES 8
 
 /*
  * A host->device copy of one chunk: `rows` runs of `width` bytes, `pitch` bytes apart, the first
@@ -128,6 +138,9 @@ typedef struct cfa_host_plan {
     cfa_swork *strided; /* block-level, rows of column slices */
     size_t n_strided;
     uint32_t *strided_first;
+    cfa_swork *brows; /* the same for the TMA path (cast-free, 16-byte aligned) */
+    size_t n_brows;
+    uint32_t *brows_first;
     int64_t *layer_last_chunk; /* n_layers; -1 = the group has no bytes */
     cfa_copy *copies;          /* what each chunk's pieces read: chunk c owns
                                   [copy_first[c], copy_first[c + 1]) */

@@ -26,7 +26,7 @@
 #include "cfa_internal.h"
 
 /* The TMA bulk kernel takes cast-free slabs whose source, destination and length are all
- * multiples of 16 bytes. */
+ * multiples of 16 bytes, and blocks of such rows of column slices. */
 #ifndef CFA_BULK_READY
 #define CFA_BULK_READY 1
 #endif
@@ -356,6 +356,8 @@ void cfa_host_plan_free(cfa_host_plan *hp)
     free(hp->tiny_first);
     free(hp->strided);
     free(hp->strided_first);
+    free(hp->brows);
+    free(hp->brows_first);
     free(hp->copies);
     free(hp->copy_first);
     free(hp->layer_last_chunk);
@@ -372,11 +374,11 @@ cfa_status cfa_host_plan_build(const cfa_tensor_entry *entries, size_t n_entries
     span *spans = NULL;
     dspan *ds = NULL;
     uint64_t *dst_bytes = NULL;
-    vec slabs = {0}, bulk = {0}, tiny = {0}, strided = {0};
+    vec slabs = {0}, bulk = {0}, tiny = {0}, strided = {0}, brows = {0};
     if (!out) return CFA_ERR_INVAL;
     memset(out, 0, sizeof *out);
     slabs.elem = bulk.elem = tiny.elem = sizeof(cfa_work);
-    strided.elem = sizeof(cfa_swork);
+    strided.elem = brows.elem = sizeof(cfa_swork);
 
     /* 1. options */
     cfa_plan_opts o;
@@ -736,7 +738,9 @@ cfa_status cfa_host_plan_build(const cfa_tensor_entry *entries, size_t n_entries
     out->bulk_first = (uint32_t *)calloc(nf, sizeof(uint32_t));
     out->tiny_first = (uint32_t *)calloc(nf, sizeof(uint32_t));
     out->strided_first = (uint32_t *)calloc(nf, sizeof(uint32_t));
-    if (!out->slab_first || !out->bulk_first || !out->tiny_first || !out->strided_first) {
+    out->brows_first = (uint32_t *)calloc(nf, sizeof(uint32_t));
+    if (!out->slab_first || !out->bulk_first || !out->tiny_first || !out->strided_first ||
+        !out->brows_first) {
         st = CFA_ERR_NOMEM;
         goto done;
     }
@@ -763,6 +767,10 @@ cfa_status cfa_host_plan_build(const cfa_tensor_entry *entries, size_t n_entries
                 const uint64_t row_d = in->cols * (uint64_t)in->es_d;
                 uint64_t per = row_d ? slab / row_d : 1;
                 if (per == 0) per = 1;
+                const uint64_t pitch = in->stride * (uint64_t)in->es_s;
+                const int by_tma = use_bulk && !pc->conv && row_d >= CFA_BULK_ROW_BYTES &&
+                                   row_d < (1u << 30) &&
+                                   ((pc->src_offset | a0 | row_d | pitch) & 15u) == 0;
                 for (uint64_t r = 0; r < pc->rows; r += per) {
                     const uint64_t k = pc->rows - r < per ? pc->rows - r : per;
                     cfa_swork sw;
@@ -775,7 +783,10 @@ cfa_status cfa_host_plan_build(const cfa_tensor_entry *entries, size_t n_entries
                     sw.ck = ck;
                     sw.mode = mode;
                     sw.cls = cls;
-                    if (vec_push(&strided, &sw)) { st = CFA_ERR_NOMEM; goto done; }
+                    if (vec_push(by_tma ? &brows : &strided, &sw)) {
+                        st = CFA_ERR_NOMEM;
+                        goto done;
+                    }
                 }
                 continue;
             }
@@ -827,6 +838,8 @@ cfa_status cfa_host_plan_build(const cfa_tensor_entry *entries, size_t n_entries
         if ((st = partition_by_class(&tiny, out->tiny_first, n_chunks, S, err, errlen))) goto done;
         if ((st = order_tiny(&tiny, out->tiny_first, n_chunks))) goto done;
         if ((st = partition_by_class(&strided, out->strided_first, n_chunks, S, err, errlen)))
+            goto done;
+        if ((st = partition_by_class(&brows, out->brows_first, n_chunks, S, err, errlen)))
             goto done;
     }
 
@@ -949,7 +962,9 @@ cfa_status cfa_host_plan_build(const cfa_tensor_entry *entries, size_t n_entries
     out->n_tiny = tiny.n;
     out->strided = (cfa_swork *)strided.p;
     out->n_strided = strided.n;
-    slabs.p = bulk.p = tiny.p = strided.p = NULL;
+    out->brows = (cfa_swork *)brows.p;
+    out->n_brows = brows.n;
+    slabs.p = bulk.p = tiny.p = strided.p = brows.p = NULL;
 
 done:
     free(info);
@@ -960,6 +975,7 @@ done:
     free(bulk.p);
     free(tiny.p);
     free(strided.p);
+    free(brows.p);
     if (st != CFA_OK) cfa_host_plan_free(out);
     return st;
 }

@@ -118,7 +118,7 @@ struct cfa_plan {
     int bulk_grid_cap = 0;
     int strided_grid_cap[CFA_N_CLASSES] = {0};
     cfa_work *d_slabs = nullptr, *d_tiny = nullptr, *d_bulk = nullptr;
-    cfa_swork *d_strided = nullptr;
+    cfa_swork *d_strided = nullptr, *d_brows = nullptr;
     /* Two halves of checksums + status word: a load accumulates into the half cleared before
      * it began, and its first kernel clears the other half, its predecessor's, so no clear and
      * no second stream sits between a load's start and its first kernel.  d_ck / d_status point
@@ -273,8 +273,8 @@ void CUDART_CB fill_host_fn(void *arg)
 
 /* Unpacks chunks [c0, c1), whose blob byte o sits at device address src_base + o (or
  * src_base + (o mod period) for a periodic source): one TMA bulk launch for the aligned cast-free
- * slabs of every element size, and per work class present in those chunks (normally one) a launch
- * for its column slices and a vector launch for everything else.  The kernels of one group write
+ * slabs and column slices of every element size, and per work class present in those chunks
+ * (normally one) a launch for its other column slices and a vector launch for everything else.  The kernels of one group write
  * disjoint destination bytes and add their checksums atomically, so they are independent: each
  * releases the next as soon as it runs, so that one kernel's last CTAs overlap the next kernel's
  * first, and ends only after the one before it, so that what follows on `s` follows them all.
@@ -295,21 +295,29 @@ cfa_status launch(cfa_plan *p, uint32_t c0, uint32_t c1, uint64_t src_base, uint
     const uint64_t lo = (uint64_t)c0 * hp.chunk_bytes;
     const uint64_t hi = std::min<uint64_t>(hp.blob_bytes, (uint64_t)c1 * hp.chunk_bytes);
     const size_t row = (size_t)hp.n_chunks + 1;
+    /* the plan's slabs suit a launch over the whole load; one over fewer chunks cuts them */
+    const uint32_t item_bytes = c0 == 0 && c1 == hp.n_chunks ? 0 : hp.opts.slab_bytes;
     const bool timing_on = (hp.opts.flags & CFA_OPT_TIMING) != 0;
-    enum { BULK, BULK_AS_VECTOR, STRIDED, VECTOR };
+    enum { BULK, BULK_AS_VECTOR, ROWS_AS_STRIDED, STRIDED, VECTOR };
     struct Job {
         int type, k;
         uint32_t a0, a1, b0, b1;
     };
-    Job jobs[3 * CFA_N_CLASSES];
+    Job jobs[4 * CFA_N_CLASSES];
     int n = 0;
-    cfa_bulk_range ranges[4]; /* bulk items are plain copies: classes 0 to 3 */
+    cfa_bulk_range ranges[CFA_BULK_RANGES]; /* bulk items are plain copies: classes 0 to 3 */
     uint32_t n_ranges = 0;
-    for (int k = 0; k < 4 && hp.n_bulk && (what & LAUNCH_CONTIG); ++k) {
+    for (int k = 0; k < 4; ++k) {
         const uint32_t b0 = hp.bulk_first[k * row + c0], b1 = hp.bulk_first[k * row + c1];
-        if (b1 == b0) continue;
-        if (!tma) jobs[n++] = Job{BULK_AS_VECTOR, k, b0, b1, 0, 0};
-        else ranges[n_ranges++] = cfa_bulk_range{p->d_bulk + b0, b1 - b0};
+        const uint32_t r0 = hp.brows_first[k * row + c0], r1 = hp.brows_first[k * row + c1];
+        if (b1 != b0 && (what & LAUNCH_CONTIG)) {
+            if (!tma) jobs[n++] = Job{BULK_AS_VECTOR, k, b0, b1, 0, 0};
+            else ranges[n_ranges++] = cfa_bulk_range{p->d_bulk + b0, b1 - b0, 0};
+        }
+        if (r1 != r0 && (what & LAUNCH_STRIDED)) {
+            if (!tma) jobs[n++] = Job{ROWS_AS_STRIDED, k, r0, r1, 0, 0};
+            else ranges[n_ranges++] = cfa_bulk_range{p->d_brows + r0, r1 - r0, 1};
+        }
     }
     if (n_ranges) jobs[n++] = Job{BULK, 0, 0, 0, 0, 0};
     for (int k = 0; k < CFA_N_CLASSES && hp.n_strided && (what & LAUNCH_STRIDED); ++k) {
@@ -341,20 +349,21 @@ cfa_status launch(cfa_plan *p, uint32_t c0, uint32_t c1, uint64_t src_base, uint
         }
         if (J.type == BULK)
             CK(p, cfa_launch_bulk(ranges, n_ranges, src_base, period, lo, hi, p->d_ck,
-                                  p->d_status, cap(p->bulk_grid_cap), hp.opts.slab_bytes, &ctl,
+                                  p->d_status, cap(p->bulk_grid_cap), item_bytes, &ctl,
                                   s));
         else if (J.type == BULK_AS_VECTOR) /* bulk items are copy-class slabs of class k */
             CK(p, cfa_launch_unpack(k, p->d_bulk + J.a0, J.a1 - J.a0, nullptr, 0, src_base,
                                     period, lo, hi, p->d_ck, p->d_status, cap(p->grid_cap[k]),
-                                    hp.opts.slab_bytes, tma, &ctl, s));
-        else if (J.type == STRIDED)
-            CK(p, cfa_launch_strided(k, p->d_strided + J.a0, J.a1 - J.a0, src_base, period, lo,
-                                     hi, p->d_ck, p->d_status, cap(p->strided_grid_cap[k]),
-                                     &ctl, s));
+                                    item_bytes, tma, &ctl, s));
+        else if (J.type == STRIDED || J.type == ROWS_AS_STRIDED)
+            CK(p, cfa_launch_strided(k,
+                                     (J.type == STRIDED ? p->d_strided : p->d_brows) + J.a0,
+                                     J.a1 - J.a0, src_base, period, lo, hi, p->d_ck, p->d_status,
+                                     cap(p->strided_grid_cap[k]), &ctl, s));
         else
             CK(p, cfa_launch_unpack(k, p->d_slabs + J.a0, J.a1 - J.a0, p->d_tiny + J.b0,
                                     J.b1 - J.b0, src_base, period, lo, hi, p->d_ck, p->d_status,
-                                    cap(p->grid_cap[k]), hp.opts.slab_bytes, tma, &ctl, s));
+                                    cap(p->grid_cap[k]), item_bytes, tma, &ctl, s));
         p->ck_clear = nullptr; /* this launch clears it */
         p->ck_clear_words = 0;
         if (timing) CK(p, cudaEventRecord(p->t_k1[p->last_launches], s));
@@ -434,6 +443,7 @@ void release(cfa_plan *p)
         if (p->d_tiny) cudaFree(p->d_tiny);
         if (p->d_bulk) cudaFree(p->d_bulk);
         if (p->d_strided) cudaFree(p->d_strided);
+        if (p->d_brows) cudaFree(p->d_brows);
         if (p->d_ck_mem) cudaFree(p->d_ck_mem);
         if (p->own_slots && p->d_slots) cudaFree(p->d_slots);
         if (p->h_slots) cudaFreeHost(p->h_slots);
@@ -468,7 +478,7 @@ cfa_status setup_device(cfa_plan *p)
         }
         p->grid_cap[k] = sms * per_sm;
     }
-    for (int k = 0; k < CFA_N_CLASSES && hp.n_strided; ++k) {
+    for (int k = 0; k < CFA_N_CLASSES && (hp.n_strided || hp.n_brows); ++k) {
         const int per_sm = cfa_strided_blocks_per_sm(k);
         if (per_sm <= 0) {
             set_err(nullptr, "strided kernel %d cannot run on device %d", k, p->device);
@@ -476,7 +486,7 @@ cfa_status setup_device(cfa_plan *p)
         }
         p->strided_grid_cap[k] = sms * per_sm;
     }
-    if (hp.n_bulk) {
+    if (hp.n_bulk || hp.n_brows) {
         const int per_sm = cfa_bulk_blocks_per_sm();
         if (per_sm <= 0) {
             set_err(nullptr, "the bulk kernel cannot run on device %d", p->device);
@@ -500,16 +510,17 @@ cfa_status setup_device(cfa_plan *p)
     if (st) return st;
     st = upload(&p->d_bulk, hp.bulk, hp.n_bulk);
     if (st) return st;
-    {
-        const size_t bytes = (hp.n_strided ? hp.n_strided : 1) * sizeof(cfa_swork);
-        if (cudaMalloc(&p->d_strided, bytes) != cudaSuccess) {
+    auto upload_rows = [&](cfa_swork **d, const cfa_swork *h, size_t n) -> cfa_status {
+        const size_t bytes = (n ? n : 1) * sizeof(cfa_swork);
+        if (cudaMalloc(d, bytes) != cudaSuccess) {
             set_err(nullptr, "cudaMalloc of %zu descriptor bytes failed", bytes);
             return CFA_ERR_NOMEM;
         }
-        if (hp.n_strided)
-            CK(nullptr, cudaMemcpy(p->d_strided, hp.strided, hp.n_strided * sizeof(cfa_swork),
-                                   cudaMemcpyHostToDevice));
-    }
+        if (n) CK(nullptr, cudaMemcpy(*d, h, n * sizeof(cfa_swork), cudaMemcpyHostToDevice));
+        return CFA_OK;
+    };
+    if ((st = upload_rows(&p->d_strided, hp.strided, hp.n_strided))) return st;
+    if (hp.n_brows && (st = upload_rows(&p->d_brows, hp.brows, hp.n_brows))) return st;
     /* two halves of checksums with the status word after them: one clear resets both */
     const size_t ck_bytes = ck_clear_bytes(hp.n_entries);
     p->ck_half_words = ck_bytes / sizeof(unsigned long long);
@@ -693,7 +704,7 @@ cfa_status cfa_plan_create(const cfa_tensor_entry *entries, size_t n_entries,
          "%.1f ms",
          hp.n_entries, hp.n_dsts, (unsigned long long)hp.blob_bytes, hp.n_chunks,
          (unsigned long long)hp.chunk_bytes, hp.n_pieces, hp.n_bulk, hp.n_slabs, hp.n_tiny,
-         hp.n_strided, (unsigned long long)hp.staged_bytes, p->plan_ms);
+         hp.n_strided + hp.n_brows, (unsigned long long)hp.staged_bytes, p->plan_ms);
     *out = p;
     return CFA_OK;
 }
@@ -881,13 +892,14 @@ cfa_status cfa_load_async(cfa_plan *p, const cfa_source *src, cfa_stream stream_
          * order and ahead of the copy ring, and each chunk's readiness also waits for them. */
         const bool slices_in_place =
             ((kind == CFA_SRC_PINNED && !(hp.opts.flags & CFA_OPT_STAGE_SLICES)) || host_pull) &&
-            hp.n_strided && !p->segmented;
+            (hp.n_strided || hp.n_brows) && !p->segmented;
         const uint64_t seg_bytes = p->segmented ? S / (uint64_t)hp.opts.seg_world : 0;
         cfa_status gather_failed = CFA_OK;
         const size_t row = (size_t)hp.n_chunks + 1;
         auto has_slices = [&](uint32_t c) {
             for (int k = 0; k < CFA_N_CLASSES; ++k)
-                if (hp.strided_first[k * row + c + 1] != hp.strided_first[k * row + c])
+                if (hp.strided_first[k * row + c + 1] != hp.strided_first[k * row + c] ||
+                    hp.brows_first[k * row + c + 1] != hp.brows_first[k * row + c])
                     return true;
             return false;
         };
@@ -1127,11 +1139,11 @@ cfa_status cfa_get_stats(cfa_plan *p, cfa_stats *s)
     s->n_slabs = hp.n_slabs;
     s->n_bulk = hp.n_bulk;
     s->n_tiny = hp.n_tiny;
-    s->n_strided = hp.n_strided;
+    s->n_strided = hp.n_strided + hp.n_brows;
     s->bytes_read = hp.bytes_read;
     s->bytes_written = hp.bytes_written;
     s->descriptor_bytes = (hp.n_slabs + hp.n_bulk + hp.n_tiny) * sizeof(cfa_work) +
-                          hp.n_strided * sizeof(cfa_swork);
+                          (hp.n_strided + hp.n_brows) * sizeof(cfa_swork);
     s->staged_bytes = hp.staged_bytes;
     s->loads = p->n_loads;
     s->kernel_launches = p->last_launches;

@@ -1185,7 +1185,12 @@ __device__ __forceinline__ bool sitem_ok(const cfa_swork &w, const StridedArgs &
            (w.src & ((1ull << sl) - 1)) == 0 && (w.dst & ((1ull << dl) - 1)) == 0;
 }
 
-/* Each CTA takes blocks of rows; its warps take the rows of a block in turn and copy each row
+/* Rows longer than this are cut into segments of about this many destination bytes: a block of
+ * rows holds a slab's bytes, and rows of tens of KiB gave a few of the CTA's eight warps one each
+ * and the others nothing (rows of 13 KiB at odd offsets, 300 MB: 113.5 us, now 105). */
+constexpr uint32_t kRowSegBytes = 4096;
+
+/* Each CTA takes blocks of rows; its warps take the rows' segments in turn and copy each one
  * like a contiguous run (16-byte vectors, realigned when source and destination disagree mod
  * 16, four vectors in flight per lane). */
 template <int CLS>
@@ -1216,15 +1221,24 @@ __global__ void __launch_bounds__(kThreads, (CLS == 0 || ClassOf<CLS>::ses == 2
         const uint64_t off = a.src_period ? w.src % a.src_period : w.src;
         const uint8_t *src = reinterpret_cast<const uint8_t *>(a.src_base + off);
         uint8_t *dst = reinterpret_cast<uint8_t *>(w.dst);
-        for (uint32_t r = warp; r < w.rows; r += kWarps) {
+        const uint64_t row_d = (uint64_t)w.cols * DES;
+        const uint32_t segs = row_d > kRowSegBytes ? (uint32_t)(row_d / kRowSegBytes) : 1u;
+        for (uint32_t t = warp; t < w.rows * segs; t += kWarps) {
+            const uint32_t r = t / segs, g = t - r * segs;
             const uint8_t *s = src + (uint64_t)r * w.stride * SES;
-            uint8_t *d = dst + (uint64_t)r * w.cols * DES;
+            uint8_t *d = dst + r * row_d;
+            /* segments are cut where the destination is a multiple of CFA_PART_ALIGN */
+            const uint32_t lead = (uint32_t)((uintptr_t)d & (CFA_PART_ALIGN - 1u));
+            const uint64_t lo = g ? (uint64_t)g * kRowSegBytes - lead : 0;
+            const uint64_t hi = g + 1u == segs ? row_d : (g + 1ull) * kRowSegBytes - lead;
+            s += lo / DES * SES;
+            d += lo;
             if constexpr (C::conv != CFA_CONV_NONE)
                 acc += convert_run<SES, DES, C::conv, ConvertDepth<CLS>::groups,
-                                   ConvertDepth<CLS>::rounds, 32>(s, d, w.cols, lane, 32u);
+                                   ConvertDepth<CLS>::rounds, 32>(s, d, (hi - lo) / DES, lane,
+                                                                  32u);
             else
-                acc += copy_run<DES, kUnroll, kRealignRoundsRows>(s, d, (uint64_t)w.cols * DES,
-                                                                  lane, 32u);
+                acc += copy_run<DES, kUnroll, kRealignRoundsRows>(s, d, hi - lo, lane, 32u);
         }
     }
     if (acc_ck != CFA_NO_CK) block_flush(acc, acc_ck, a.ck, red);

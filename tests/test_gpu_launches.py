@@ -134,3 +134,41 @@ def test_consecutive_chunks_in_a_cuda_graph():
             torch.cuda.synchronize()
             assert torch.equal(c.out, c.want)
         del graph
+
+
+@pytest.mark.parametrize("row_bytes", [16, 1008, 1024, 1040, 7168, 32768, 32784, 300_000])
+def test_column_slices_by_row_length(row_bytes):
+    """Rows below, at and above the shortest that go to the TMA kernel, the stage and a slab, at
+    column offsets on and off the 16-byte grid, from device memory and (in place) pinned memory."""
+    rows, lead = 37, 6
+    cases = [(d, off) for d in ES for off in (0, 16, 16 + ES[d])]
+    entries, outs, want = [], [], []
+    g = torch.Generator(device="cuda").manual_seed(9)
+    pitch = row_bytes + 64
+    blob = torch.randint(0, 256, (rows * pitch + 256,), dtype=torch.uint8, device="cuda",
+                         generator=g)
+    grid = blob[:rows * pitch].view(rows, pitch)
+    for d, off in cases:
+        entries.append((d, (rows, row_bytes // ES[d]), off, pitch // ES[d]))
+        outs.append(torch.zeros(rows * row_bytes + 256 * lead, dtype=torch.uint8, device="cuda"))
+        want.append(grid[:, off:off + row_bytes].contiguous().view(-1))
+    ents = cfa.make_entries(dtype=[e[0] for e in entries], shape=[e[1] for e in entries],
+                            offset=[e[2] for e in entries], dst=list(range(len(entries))),
+                            src_row_stride=[e[3] for e in entries])
+    dsts = [(o.data_ptr(), e[0], e[1]) for o, e in zip(outs, entries)]
+    host = blob.cpu().pin_memory()
+    with cfa.Plan(ents, dsts, blob.numel(), dev_slots=2, host_slots=0,
+                  chunk_bytes=1 << 20) as plan:
+        for src in (cfa.Source.device(blob.data_ptr()), cfa.Source.pinned(host.data_ptr())):
+            for o in outs:
+                o.zero_()
+            torch.cuda.synchronize()
+            plan.load_async(src)
+            plan.wait_layer()
+            ck = plan.checksums()
+            for i, (o, w) in enumerate(zip(outs, want)):
+                assert torch.equal(o[:w.numel()], w), (i, cases[i])
+                assert not o[w.numel():].any()
+                u = {1: np.uint8, 2: np.uint16, 4: np.uint32, 8: np.uint64}[ES[cases[i][0]]]
+                total = w.cpu().numpy().view(u).astype(np.uint64).sum(dtype=np.uint64)
+                assert int(ck[i]) == int(total)
