@@ -137,6 +137,9 @@ struct cfa_plan {
     int n_dev_slots = 0;
     uint8_t *h_slots = nullptr;
     int n_host_slots = 0;
+    /* page-locked words for reading the status word, and a half of up to kReadWords words, back */
+    unsigned long long *h_read = nullptr;
+    std::mutex read_mu;
     cudaStream_t fill_stream = nullptr, copy_stream = nullptr, aux_stream = nullptr;
     /* pinned sources: column slices read in place over the host link, beside the copy ring */
     cudaStream_t direct_stream = nullptr;
@@ -394,6 +397,13 @@ cfa_status make_event(cfa_plan *p, cudaEvent_t *ev, bool timing)
     return CFA_OK;
 }
 
+/* Contexts of finished loads are dropped once there are this many. */
+constexpr size_t kKeptLoads = 4;
+
+/* Halves of up to this many words (64 KiB) are read back in one copy, status word and all,
+ * through page-locked memory. */
+constexpr size_t kReadWords = 8192;
+
 /* Points d_ck / d_status at half h of the checksum buffer. */
 void use_ck_half(cfa_plan *p, int h)
 {
@@ -447,6 +457,7 @@ void release(cfa_plan *p)
         if (p->d_ck_mem) cudaFree(p->d_ck_mem);
         if (p->own_slots && p->d_slots) cudaFree(p->d_slots);
         if (p->h_slots) cudaFreeHost(p->h_slots);
+        if (p->h_read) cudaFreeHost(p->h_read);
     }
     p->pool.reset();
     cfa_host_plan_free(&p->hp);
@@ -530,6 +541,12 @@ cfa_status setup_device(cfa_plan *p)
     }
     CK(nullptr, cudaMemset(p->d_ck_mem, 0, 2 * ck_bytes));
     use_ck_half(p, 0);
+    if (cudaHostAlloc(&p->h_read, std::min(kReadWords, p->ck_half_words) * sizeof *p->h_read,
+                      cudaHostAllocDefault) != cudaSuccess) {
+        cudaGetLastError();
+        set_err(nullptr, "cudaHostAlloc of the read-back buffer failed");
+        return CFA_ERR_NOMEM;
+    }
 
     p->n_dev_slots = o.dev_slots;
     p->n_host_slots = o.host_slots;
@@ -597,12 +614,9 @@ cfa_status setup_device(cfa_plan *p)
     return CFA_OK;
 }
 
-cfa_status check_status_word(cfa_plan *p)
+/* The error that status word h stands for. */
+cfa_status check_status(cfa_plan *p, int h)
 {
-    int h = 0;
-    CK(p, cudaStreamWaitEvent(p->aux_stream, p->ev_all, 0));
-    CK(p, cudaMemcpyAsync(&h, p->d_status, sizeof(int), cudaMemcpyDeviceToHost, p->aux_stream));
-    CK(p, cudaStreamSynchronize(p->aux_stream));
     if (h == 3) {
         set_err(p, "a TMA bulk-copy wait ran out and so did the wait for the CTA's own loads in "
                    "flight (status word 3): treat the CUDA context as suspect");
@@ -618,10 +632,24 @@ cfa_status check_status_word(cfa_plan *p)
     return CFA_OK;
 }
 
-/* Polls `ev` from the host, sleeping between queries, until it completes or timeout_ns passes
- * (timeout_ns < 0: no limit).  The sleep doubles from 2 us up to kPollSleepMaxUs, so a load is
- * noticed within about that much (plus the thread's timer slack) of its end: a 1 ms cap cost
- * the end-to-end figure of a 76 ms load a whole millisecond. */
+/* Reads the status word of the load that p->ev_all has completed. */
+cfa_status check_status_word(cfa_plan *p)
+{
+    std::lock_guard<std::mutex> lk(p->read_mu);
+    CK(p, cudaMemcpyAsync(p->h_read, p->d_status, sizeof(int), cudaMemcpyDeviceToHost,
+                          p->aux_stream));
+    CK(p, cudaStreamSynchronize(p->aux_stream));
+    int h;
+    std::memcpy(&h, p->h_read, sizeof h);
+    return check_status(p, h);
+}
+
+/* Polls `ev` from the host until it completes or timeout_ns passes (timeout_ns < 0: no limit):
+ * without a pause for the first kPollSpinUs, then sleeping between queries, 2 us doubling up to
+ * kPollSleepMaxUs.  A sleep ends late by the thread's timer slack (50 us by default), so the
+ * sleeps made a 10 us load of one adapter return after 60 us or more, and rounded every load under
+ * a millisecond up by tens of microseconds; a longer load is noticed within about 100 us. */
+constexpr int64_t kPollSpinUs = 2000;
 constexpr int64_t kPollSleepMaxUs = 50;
 
 cfa_status wait_event_host(cfa_plan *p, cudaEvent_t ev, int64_t timeout_ns)
@@ -635,18 +663,27 @@ cfa_status wait_event_host(cfa_plan *p, cudaEvent_t ev, int64_t timeout_ns)
             set_err(p, "cudaEventQuery failed: %s", cudaGetErrorString(q));
             return CFA_ERR_CUDA;
         }
-        if (timeout_ns >= 0) {
-            const int64_t el = std::chrono::duration_cast<std::chrono::nanoseconds>(
-                                   std::chrono::steady_clock::now() - t0)
-                                   .count();
-            if (el >= timeout_ns) {
-                set_err(p, "wait timed out after %lld ns", (long long)timeout_ns);
-                return CFA_ERR_TIMEOUT;
-            }
+        const int64_t el = std::chrono::duration_cast<std::chrono::nanoseconds>(
+                               std::chrono::steady_clock::now() - t0)
+                               .count();
+        if (timeout_ns >= 0 && el >= timeout_ns) {
+            set_err(p, "wait timed out after %lld ns", (long long)timeout_ns);
+            return CFA_ERR_TIMEOUT;
         }
+        if (el < kPollSpinUs * 1000) continue;
         std::this_thread::sleep_for(std::chrono::microseconds(sleep_us));
         sleep_us = std::min<int64_t>(sleep_us * 2, kPollSleepMaxUs);
     }
+}
+
+/* The same, and the error of the load's source, if it had one. */
+cfa_status wait_on_host(cfa_plan *p, cudaEvent_t ev, int64_t timeout_ns)
+{
+    cfa_status st = wait_event_host(p, ev, timeout_ns);
+    if (st) return st;
+    const int e = p->last->error.load();
+    if (e && e != CFA_ERR_GATHER) set_err(p, "the source callback failed");
+    return e;
 }
 
 } // namespace
@@ -794,7 +831,7 @@ cfa_status cfa_load_async(cfa_plan *p, const cfa_source *src, cfa_stream stream_
     cudaStream_t cs = reinterpret_cast<cudaStream_t>(stream_);
 
     /* contexts of loads that have fully completed are no longer referenced by host functions */
-    if (!p->loads.empty() && cudaEventQuery(p->ev_all) == cudaSuccess &&
+    if (p->loads.size() >= kKeptLoads && cudaEventQuery(p->ev_all) == cudaSuccess &&
         cudaStreamQuery(p->fill_stream) == cudaSuccess)
         p->loads.clear();
     if (staged && hp.n_chunks && !p->h_slots) {
@@ -1096,13 +1133,8 @@ cfa_status cfa_wait_layer(cfa_plan *p, int32_t layer, cfa_stream consumer, int64
         const int e = p->last->error.load();
         return e ? e : CFA_OK;
     }
-    cfa_status st = wait_event_host(p, ev, timeout_ns);
+    cfa_status st = wait_on_host(p, ev, timeout_ns);
     if (st) return st;
-    const int e = p->last->error.load();
-    if (e) {
-        if (e != CFA_ERR_GATHER) set_err(p, "the source callback failed");
-        return e;
-    }
     if (layer == CFA_ALL) return check_status_word(p);
     return CFA_OK;
 }
@@ -1114,14 +1146,25 @@ cfa_status cfa_get_checksums(cfa_plan *p, uint64_t *host_out, size_t n)
         set_err(p, "no load has been enqueued");
         return CFA_ERR_INVAL;
     }
-    cfa_status st = cfa_wait_layer(p, CFA_ALL, nullptr, -1);
-    if (st) return st;
-    if (!n) return CFA_OK;
     DeviceGuard g(p->device);
-    CK(p, cudaStreamWaitEvent(p->aux_stream, p->ev_all, 0));
-    CK(p, cudaMemcpyAsync(host_out, p->d_ck, n * sizeof(uint64_t), cudaMemcpyDeviceToHost,
-                          p->aux_stream));
+    cfa_status st = wait_on_host(p, p->ev_all, -1);
+    if (st) return st;
+    if (p->ck_half_words > kReadWords) {
+        if ((st = check_status_word(p)) || !n) return st;
+        CK(p, cudaMemcpyAsync(host_out, p->d_ck, n * sizeof(uint64_t), cudaMemcpyDeviceToHost,
+                              p->aux_stream));
+        CK(p, cudaStreamSynchronize(p->aux_stream));
+        return CFA_OK;
+    }
+    /* the status word lies behind the checksums: one copy reads both */
+    std::lock_guard<std::mutex> lk(p->read_mu);
+    CK(p, cudaMemcpyAsync(p->h_read, p->d_ck, p->ck_half_words * sizeof *p->h_read,
+                          cudaMemcpyDeviceToHost, p->aux_stream));
     CK(p, cudaStreamSynchronize(p->aux_stream));
+    int h;
+    std::memcpy(&h, p->h_read + (p->ck_half_words - 1), sizeof h);
+    if ((st = check_status(p, h))) return st;
+    if (n) std::memcpy(host_out, p->h_read, n * sizeof(uint64_t));
     return CFA_OK;
 }
 
