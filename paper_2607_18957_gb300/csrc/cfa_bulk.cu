@@ -38,6 +38,7 @@ namespace {
 
 using cfa_dev::launch_begin;
 using cfa_dev::launch_ctl;
+using cfa_dev::launch_early;
 using cfa_dev::launch_end;
 using cfa_dev::vsum;
 using cfa_dev::warp_sum;
@@ -152,14 +153,14 @@ __device__ __forceinline__ bool bulk_item_ok(const BulkItem &w, const BulkArgs &
 {
     const uint32_t l = w.mode & 3u;
     const uint64_t row = (uint64_t)w.cols << l, pitch = (uint64_t)w.stride << l;
-    if (w.mode != CFA_MODE(l, l, 0) || w.rows == 0 || w.cols == 0 || pitch < row) return false;
-    /* no product overflows: rows and columns below 2^32, so bounded before it is taken */
-    if (row >= (1ull << 31) || w.rows > (1ull << 31) / row) return false;
+    const uint64_t total = row * w.rows; /* may wrap only when row alone is refused below */
+    if (w.mode != CFA_MODE(l, l, 0) || w.rows == 0 || w.cols == 0 || pitch < row ||
+        row >= (1ull << 31) || total >= (1ull << 31) ||
+        ((w.src | w.dst | row | (w.rows > 1 ? pitch : 0) | a.src_base | a.src_period) & 15u) != 0)
+        return false;
+    /* row is 16 at least here, so there are fewer than 2^27 rows of a pitch below 2^35 */
     const uint64_t extent = (w.rows - 1) * pitch + row;
-    return w.src >= a.src_lo && w.src <= a.src_hi && extent <= a.src_hi - w.src &&
-           row * w.rows < (1ull << 31) &&
-           ((w.src | w.dst | row | (w.rows > 1 ? pitch : 0) | a.src_base | a.src_period) & 15u) ==
-               0;
+    return w.src >= a.src_lo && w.src <= a.src_hi && extent <= a.src_hi - w.src;
 }
 
 /* Bytes [*at, *at + *len) of a checked item of `total` bytes at destination `dst` that are part k
@@ -182,32 +183,52 @@ __device__ __forceinline__ bool bulk_part(uint64_t dst, uint32_t total, uint32_t
     return true;
 }
 
-/* Descriptor of part `v` of the launch. */
-__device__ __forceinline__ BulkItem bulk_fetch(const BulkArgs &a, uint32_t v)
+/* A descriptor as it lies in memory (cfa_work, or cfa_swork with its fifth word).  It is fetched one
+ * part ahead and decoded only when its part comes up: any arithmetic at the fetch, even a copy of
+ * one of its words, would wait for the load there and then (8-bit checkpoint in 64 MiB chunks: 1244
+ * us, now 1233). */
+struct RawItem {
+    uint64_t q[5];
+    uint32_t rows;
+};
+
+template <bool ROWS>
+__device__ __forceinline__ RawItem bulk_fetch(const BulkArgs &a, uint32_t v)
 {
     uint32_t i = v >> a.parts_log2;
     int r = 0;
     while (i >= a.range[r].n) i -= a.range[r++].n;
-    BulkItem b;
-    if (a.range[r].rows) {
-        const cfa_swork w = static_cast<const cfa_swork *>(a.range[r].items)[i];
-        b.src = w.src;
-        b.dst = w.dst;
-        b.rows = w.rows;
-        b.cols = w.cols;
-        b.stride = w.stride;
-        b.ck = w.ck;
-        b.mode = w.mode;
-    } else {
-        const cfa_work w = static_cast<const cfa_work *>(a.range[r].items)[i];
-        b.src = w.src;
-        b.dst = w.dst;
-        b.rows = 1;
-        b.cols = b.stride = w.n;
-        b.ck = w.ck;
-        b.mode = w.mode;
-    }
+    RawItem b;
+    b.rows = ROWS ? a.range[r].rows : 0;
+    const size_t bytes = b.rows ? sizeof(cfa_swork) : sizeof(cfa_work);
+    const uint64_t *p = reinterpret_cast<const uint64_t *>(
+        static_cast<const uint8_t *>(a.range[r].items) + i * bytes);
+#pragma unroll
+    for (int k = 0; k < 4; ++k) b.q[k] = __ldg(reinterpret_cast<const unsigned long long *>(p) + k);
+    if (b.rows) b.q[4] = __ldg(reinterpret_cast<const unsigned long long *>(p) + 4);
     return b;
+}
+
+static_assert(sizeof(cfa_work) == 32 && sizeof(cfa_swork) == 40, "descriptor layouts");
+
+template <bool ROWS> __device__ __forceinline__ BulkItem bulk_decode(const RawItem &b)
+{
+    BulkItem w;
+    w.src = b.q[0];
+    w.dst = b.q[1];
+    if (ROWS && b.rows) {
+        w.rows = (uint32_t)b.q[2];
+        w.cols = (uint32_t)(b.q[2] >> 32);
+        w.stride = (uint32_t)b.q[3];
+        w.ck = (uint32_t)(b.q[3] >> 32);
+        w.mode = (uint32_t)b.q[4];
+    } else {
+        w.rows = 1;
+        w.cols = w.stride = (uint32_t)b.q[2];
+        w.ck = (uint32_t)(b.q[2] >> 32);
+        w.mode = (uint32_t)b.q[3];
+    }
+    return w;
 }
 
 /* Sum of a staged sub-block's elements over this lane's vectors: eight independent shared loads
@@ -237,6 +258,9 @@ struct StageMeta {
     uint32_t log2es;
 };
 
+/* ROWS: some items are row blocks.  Launches without any (all but tensor-parallel ranks) have none
+ * of that arithmetic on the loader's path (44 registers against 52). */
+template <bool ROWS>
 __global__ void __launch_bounds__(kThreads) cfa_bulk_kernel(const BulkArgs a)
 {
     extern __shared__ __align__(128) uint8_t stage[];
@@ -256,12 +280,13 @@ __global__ void __launch_bounds__(kThreads) cfa_bulk_kernel(const BulkArgs a)
         n_issued = 0;
         n_consumed = 0;
     }
+    launch_early(a.ctl);
     /* the loader's first two descriptors (the plan's own memory, written before any launch) are
      * on their way while the launch waits for what is before it on the stream */
-    BulkItem w{}, nxt{};
+    RawItem cur{}, nxt{};
     if (threadIdx.x == 0) {
-        if (blockIdx.x < a.n_items) w = bulk_fetch(a, blockIdx.x);
-        if (blockIdx.x + gridDim.x < a.n_items) nxt = bulk_fetch(a, blockIdx.x + gridDim.x);
+        if (blockIdx.x < a.n_items) cur = bulk_fetch<ROWS>(a, blockIdx.x);
+        if (blockIdx.x + gridDim.x < a.n_items) nxt = bulk_fetch<ROWS>(a, blockIdx.x + gridDim.x);
     }
     launch_begin(a.ctl);
     __syncthreads();
@@ -275,6 +300,7 @@ __global__ void __launch_bounds__(kThreads) cfa_bulk_kernel(const BulkArgs a)
         if (lane == 0) {
             /* part `it` is being issued from w, bytes [off, end) left; the descriptor of part
              * it + gridDim.x is in flight into nxt */
+            BulkItem w = bulk_decode<ROWS>(cur);
             uint32_t it = blockIdx.x, p = 0, off = 0, end = 0;
             bool have = it < a.n_items;
             uint32_t it_n = it + gridDim.x;
@@ -282,9 +308,9 @@ __global__ void __launch_bounds__(kThreads) cfa_bulk_kernel(const BulkArgs a)
                 it = it_n;
                 have = it < a.n_items;
                 if (have) {
-                    w = nxt;
+                    w = bulk_decode<ROWS>(nxt);
                     it_n = it + gridDim.x;
-                    if (it_n < a.n_items) nxt = bulk_fetch(a, it_n);
+                    if (it_n < a.n_items) nxt = bulk_fetch<ROWS>(a, it_n);
                 }
             };
             auto settle = [&]() { /* skip items that fail the checks, and empty parts */
@@ -415,14 +441,18 @@ __global__ void __launch_bounds__(kThreads) cfa_bulk_kernel(const BulkArgs a)
 /* Resident CTAs per SM of the bulk kernel (0 if it cannot run). */
 extern "C" int cfa_bulk_blocks_per_sm(void)
 {
-    if (cudaFuncSetAttribute(cfa_bulk_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)kSmemBytes) != cudaSuccess)
-        return 0;
-    int n = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, cfa_bulk_kernel, kThreads,
-                                                      kSmemBytes) != cudaSuccess)
-        return 0;
-    return n;
+    int least = 0;
+    for (int rows = 0; rows < 2; ++rows) {
+        void (*fn)(const BulkArgs) = rows ? cfa_bulk_kernel<true> : cfa_bulk_kernel<false>;
+        int n = 0;
+        if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 (int)kSmemBytes) != cudaSuccess ||
+            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, fn, kThreads, kSmemBytes) !=
+                cudaSuccess)
+            return 0;
+        least = rows && least < n ? least : n;
+    }
+    return least;
 }
 
 /* Launches the bulk unpack over up to CFA_BULK_RANGES lists of items whose source, destination and
@@ -437,9 +467,11 @@ extern "C" cudaError_t cfa_launch_bulk(const cfa_bulk_range *ranges, uint32_t n_
     if (n_ranges > CFA_BULK_RANGES || grid_cap <= 0) return cudaErrorInvalidValue;
     BulkArgs a{};
     uint64_t n_items = 0;
+    bool rows = false;
     for (uint32_t r = 0, k = 0; r < n_ranges; ++r) {
         if (!ranges[r].n) continue;
         a.range[k++] = ranges[r];
+        rows |= ranges[r].rows != 0;
         n_items += ranges[r].n;
     }
     if (n_items == 0) return cudaSuccess;
@@ -455,7 +487,7 @@ extern "C" cudaError_t cfa_launch_bulk(const cfa_bulk_range *ranges, uint32_t n_
     a.status = status;
     const uint32_t grid = a.n_items < (uint32_t)grid_cap ? a.n_items : (uint32_t)grid_cap;
     a.ctl = ctl ? *ctl : cfa_launch_ctl{};
-    return launch_ctl(cfa_bulk_kernel, grid, kThreads, kSmemBytes, stream, a);
+    return launch_ctl(rows ? cfa_bulk_kernel<true> : cfa_bulk_kernel<false>, grid, kThreads, kSmemBytes, stream, a);
 }
 
 /* Self-test of the bounded waits: one CTA of the TMA kernel over one valid 16-byte item, with a
@@ -470,7 +502,7 @@ extern "C" cudaError_t cfa_bulk_selftest_timeout(int *status_host)
     cudaError_t e = cudaSuccess;
     if (!status_host) return cudaErrorInvalidValue;
     *status_host = -1;
-    if ((e = cudaFuncSetAttribute(cfa_bulk_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    if ((e = cudaFuncSetAttribute(cfa_bulk_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                   (int)kSmemBytes)) != cudaSuccess)
         return e;
     if ((e = cudaMalloc(&d_item, sizeof(cfa_work))) != cudaSuccess) goto out;
@@ -497,7 +529,7 @@ extern "C" cudaError_t cfa_bulk_selftest_timeout(int *status_host)
         a.src_hi = 256;
         a.ck = d_ck;
         a.status = d_status;
-        cfa_bulk_kernel<<<1, kThreads, kSmemBytes>>>(a);
+        cfa_bulk_kernel<false><<<1, kThreads, kSmemBytes>>>(a);
         if ((e = cudaGetLastError()) != cudaSuccess) goto out;
         if ((e = cudaDeviceSynchronize()) != cudaSuccess) goto out;
         e = cudaMemcpy(status_host, d_status, sizeof(int), cudaMemcpyDeviceToHost);

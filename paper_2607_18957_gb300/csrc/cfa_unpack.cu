@@ -33,6 +33,7 @@ namespace {
 
 using cfa_dev::launch_begin;
 using cfa_dev::launch_ctl;
+using cfa_dev::launch_early;
 using cfa_dev::launch_end;
 using cfa_dev::vsum;
 using cfa_dev::warp_sum;
@@ -665,6 +666,7 @@ __global__ void __launch_bounds__(kThreads, unpack_min_blocks(CLS))
     cfa_unpack_kernel(const UnpackArgs a)
 {
     __shared__ unsigned long long red[kWarps];
+    launch_early(a.ctl);
     launch_begin(a.ctl);
     const uint32_t n_groups = (a.n_tiny + kTinyPerGroup - 1) / kTinyPerGroup;
     const uint32_t n_slabs = a.n_slabs << a.parts_log2; /* parts of slabs */
@@ -1078,6 +1080,7 @@ template <int CLS>
 __global__ void __launch_bounds__(kThreads, (CLS == 0 ? kCopyMinBlocks : unpack_min_blocks(CLS)))
     cfa_tiny_kernel(const UnpackArgs a)
 {
+    launch_early(a.ctl);
     launch_begin(a.ctl);
     if constexpr (CLS < 4) {
         /* device-memory sources take the shared-memory pipeline; host memory read in place over
@@ -1204,6 +1207,7 @@ __global__ void __launch_bounds__(kThreads, (CLS == 0 || ClassOf<CLS>::ses == 2
     constexpr int DES = C::des;
     __shared__ unsigned long long red[kWarps];
     const uint32_t lane = threadIdx.x & 31u, warp = threadIdx.x >> 5;
+    launch_early(a.ctl);
     launch_begin(a.ctl);
     uint64_t acc = 0;
     uint32_t acc_ck = CFA_NO_CK;
