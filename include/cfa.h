@@ -449,10 +449,8 @@ cfa_status cfa_unpack_chunks_async(cfa_plan *plan, uint32_t chunk_begin, uint32_
  *   - the first call on a device does a one-time set-up (it looks up the array's device address
  *     and the kernels' occupancy); make it before any stream capture.  That address belongs to
  *     the device's context: do not call this again in a process after cudaDeviceReset;
- *   - the call blocks the host: the descriptors go up as a copy from pageable host memory,
- *     which CUDA completes before returning, and which first waits for the work already
- *     queued on `stream`.  The unpack kernels are enqueued behind it and run after the call
- *     returns.
+ *   - the call only enqueues: the descriptors go up as kernel parameters, in stream order, and
+ *     the unpack kernels behind them (entries and dsts may be changed once it returns).
  *
  *   entries, n_entries, dsts, n_dsts   as for cfa_plan_create (host arrays, read during the call)
  *   blob_dev, blob_bytes   the blob in device memory (256-byte aligned); must stay valid and

@@ -16,10 +16,10 @@
  * capture.  The cached address belongs to the device's current context: after a
  * cudaDeviceReset the library must not be used again in the process.
  *
- * Blocking: the descriptors go up with a copy from pageable host memory, which returns only
- * once the bytes have been copied, so the call blocks the host until the work already queued
- * on the stream has run and the copy is done; the unpack kernels themselves run after it
- * returns.
+ * Upload: the descriptors go up as the parameters of a small kernel (cfa_put_kernel), which also
+ * clears the status word and the checksums; it runs in stream order like everything else, so the
+ * call enqueues its work and returns.  (A copy from pageable host memory first waited for the work
+ * already queued on the stream, and left the GPU idle while the host went on.)
  *
  * Sharing: every call on a device uses the same scratch array, which keeps the last call's
  * contents.  Calls are serialised on the host by a mutex, but two calls whose GPU work overlaps
@@ -30,8 +30,10 @@
 
 #include <cstdarg>
 #include <cstdio>
+#include <cstring>
 #include <mutex>
 
+#include "cfa_device.cuh"
 #include "cfa_internal.h"
 
 extern "C" int cfa_unpack_blocks_per_sm(int cls);
@@ -59,9 +61,77 @@ static __device__ __align__(256) NoallocScratch g_noalloc_scratch;
 /* Host twin of the descriptors, filled before each upload (guarded by g_mutex). */
 static cfa_work g_host_items[CFA_NOALLOC_MAX_ITEMS];
 
+/* Descriptors that one launch of the upload carries in its parameters (at most 32,764 bytes), and
+ * what the call's first launch clears: the unpack's status word and checksums. */
+template <int CAP> struct PutArgs {
+    cfa_work *to;
+    uint32_t n;
+    cfa_launch_ctl ctl;
+    int *status;
+    __align__(16) cfa_work items[CAP];
+};
+constexpr int kPutSmall = 112; /* under 4 KiB of parameters: the cheaper launch */
+constexpr int kPutLarge = 1000;
+constexpr int kPutThreads = 256;
+
+/* Bound by its launch: 64 KiB at most, written once; one thread per 16 bytes of descriptor. */
+template <int CAP>
+__global__ void __launch_bounds__(kPutThreads)
+    cfa_put_kernel(const __grid_constant__ PutArgs<CAP> a)
+{
+    /* what follows waits for this kernel's end before it reads anything */
+    cfa_dev::launch_begin(a.ctl);
+    const uint32_t i = blockIdx.x * kPutThreads + threadIdx.x;
+    if (i == 0 && a.status) *a.status = 0;
+    const uint4 *from = reinterpret_cast<const uint4 *>(a.items);
+    if (i < 2u * a.n) reinterpret_cast<uint4 *>(a.to)[i] = from[i];
+}
+
+/* The launch's parameters, filled under g_mutex; the launch copies them. */
+static PutArgs<kPutSmall> g_put_small;
+static PutArgs<kPutLarge> g_put_large;
+
 std::mutex g_mutex;
 NoallocScratch *g_scratch_dev[kMaxDevices];
 int g_grid_cap[kMaxDevices][CFA_N_CLASSES];
+
+template <int CAP>
+cudaError_t put(PutArgs<CAP> &a, cfa_work *to, const cfa_work *from, uint32_t n, int *status,
+                const cfa_launch_ctl &ctl, cudaStream_t stream)
+{
+    a.to = to;
+    a.n = n;
+    a.status = status;
+    a.ctl = ctl;
+    if (n) std::memcpy(a.items, from, (size_t)n * sizeof(cfa_work));
+    /* enough CTAs for the items, and one per 16 Ki checksums to clear */
+    uint64_t grid = (2ull * n + kPutThreads - 1) / kPutThreads;
+    const uint64_t clear = ctl.clear_words >> 14;
+    if (grid < clear) grid = clear < 152 ? clear : 152;
+    if (grid == 0) grid = 1;
+    return cfa_dev::launch_ctl(cfa_put_kernel<CAP>, (unsigned)grid, kPutThreads, 0, stream, a);
+}
+
+/* Uploads n descriptors to `to` in stream order; the first launch clears what ctl and status say. */
+cudaError_t put_items(cfa_work *to, const cfa_work *from, uint32_t n, int *status,
+                      unsigned long long *clear, uint64_t clear_words, cudaStream_t stream)
+{
+    cfa_launch_ctl ctl{};
+    ctl.clear = clear;
+    ctl.clear_words = clear_words;
+    for (uint32_t at = 0;;) {
+        const uint32_t left = n - at;
+        const uint32_t k = left < (uint32_t)kPutLarge ? left : (uint32_t)kPutLarge;
+        if (k == left) ctl.flags = CFA_LAUNCH_RELEASE;
+        const cudaError_t e = k <= (uint32_t)kPutSmall
+                                  ? put(g_put_small, to + at, from + at, k, status, ctl, stream)
+                                  : put(g_put_large, to + at, from + at, k, status, ctl, stream);
+        at += k;
+        if (e != cudaSuccess || at == n) return e;
+        ctl = cfa_launch_ctl{};
+        status = nullptr;
+    }
+}
 
 /* The caller's message buffer for the current call (may be NULL). */
 thread_local char *g_err = nullptr;
@@ -107,6 +177,9 @@ uint64_t tiny_items(uint64_t dst0, uint64_t nb)
 {
     return (dst0 + nb - 1) / CFA_TINY_SEG_BYTES - dst0 / CFA_TINY_SEG_BYTES + 1;
 }
+
+/* Kinds of work items. */
+enum { SLAB, TINY, kKinds };
 
 cfa_status fail(cfa_status st, const char *msg, size_t i)
 {
@@ -236,7 +309,7 @@ extern "C" cfa_status cfa_unpack_noalloc(const cfa_tensor_entry *entries, size_t
     std::lock_guard<std::mutex> lock(g_mutex);
 
     /* validate every entry and count the work items, per class, without storing anything */
-    uint32_t count[CFA_N_CLASSES][2] = {};
+    uint32_t count[CFA_N_CLASSES][kKinds] = {};
     for (size_t i = 0; i < n_entries; ++i) {
         uint64_t n, off;
         int es_s, es_d, conv;
@@ -250,21 +323,22 @@ extern "C" cfa_status cfa_unpack_noalloc(const cfa_tensor_entry *entries, size_t
         const uint64_t items = nb < kTinyBytes ? tiny_items(dst0, nb)
                                                : (nb + kSlabBytes - 1) / kSlabBytes;
         uint64_t total = items;
-        for (int k = 0; k < CFA_N_CLASSES; ++k) total += count[k][0] + count[k][1];
+        for (int k = 0; k < CFA_N_CLASSES; ++k)
+            for (int t = 0; t < kKinds; ++t) total += count[k][t];
         if (total > CFA_NOALLOC_MAX_ITEMS) {
             say("cfa_unpack_noalloc: the manifest needs more than the %d work items of the "
                 "fixed scratch (one per 2 MiB of destination, one per 512 bytes of a tensor "
                 "under 8 KiB); use cfa_plan_create", CFA_NOALLOC_MAX_ITEMS);
             return CFA_ERR_INVAL;
         }
-        count[cls][nb < kTinyBytes ? 1 : 0] += (uint32_t)items;
+        count[cls][nb < kTinyBytes ? TINY : SLAB] += (uint32_t)items;
     }
 
     /* lay the items out as [class 0 slabs][class 0 tiny][class 1 slabs] ... */
-    uint32_t base[CFA_N_CLASSES][2], cursor[CFA_N_CLASSES][2];
+    uint32_t base[CFA_N_CLASSES][kKinds], cursor[CFA_N_CLASSES][kKinds];
     uint32_t total = 0;
     for (int k = 0; k < CFA_N_CLASSES; ++k)
-        for (int t = 0; t < 2; ++t) {
+        for (int t = 0; t < kKinds; ++t) {
             base[k][t] = cursor[k][t] = total;
             total += count[k][t];
         }
@@ -289,7 +363,7 @@ extern "C" cfa_status cfa_unpack_noalloc(const cfa_tensor_entry *entries, size_t
                 w.src = entries[i].blob_offset + (pos - dst0) / (uint64_t)es_d * (uint64_t)es_s;
                 w.dst = pos;
                 w.n = (uint32_t)((next - pos) / (uint64_t)es_d);
-                g_host_items[cursor[cls][1]++] = w;
+                g_host_items[cursor[cls][TINY]++] = w;
                 pos = next;
             }
             continue;
@@ -300,7 +374,7 @@ extern "C" cfa_status cfa_unpack_noalloc(const cfa_tensor_entry *entries, size_t
             w.src = entries[i].blob_offset + e0 * (uint64_t)es_s;
             w.dst = dst0 + e0 * (uint64_t)es_d;
             w.n = (uint32_t)k;
-            g_host_items[cursor[cls][0]++] = w;
+            g_host_items[cursor[cls][SLAB]++] = w;
         }
     }
 
@@ -315,22 +389,21 @@ extern "C" cfa_status cfa_unpack_noalloc(const cfa_tensor_entry *entries, size_t
     if (st) return st;
 
     /* the kernels' status word (the caller's, or the scratch's own) and the checksums start at
-     * zero; the descriptors are uploaded from the host array (a pageable copy: the call returns
-     * once the bytes are on the device, after the work queued before it on the stream) */
+     * zero; then the descriptors, and the kernels chained behind them (cfa_launch_ctl): the first
+     * waits for the upload, the others only end in order */
     int *status = status_dev ? status_dev : &scratch->status;
-    e = cudaMemsetAsync(status, 0, sizeof(int), stream);
-    if (e == cudaSuccess && cksum_dev && n_entries)
-        e = cudaMemsetAsync(cksum_dev, 0, n_entries * sizeof(uint64_t), stream);
-    if (e == cudaSuccess && total)
-        e = cudaMemcpyAsync(scratch->items, g_host_items, (size_t)total * sizeof(cfa_work),
-                            cudaMemcpyHostToDevice, stream);
+    unsigned long long *ck = reinterpret_cast<unsigned long long *>(cksum_dev);
+    e = put_items(scratch->items, g_host_items, total, status, ck, ck ? n_entries : 0, stream);
+    const uint64_t src = (uint64_t)(uintptr_t)blob_dev;
+    cfa_launch_ctl ctl{};
+    ctl.flags = CFA_LAUNCH_EARLY | CFA_LAUNCH_WAIT_FIRST | CFA_LAUNCH_RELEASE;
     for (int k = 0; e == cudaSuccess && k < CFA_N_CLASSES; ++k) {
-        if (!count[k][0] && !count[k][1]) continue;
-        e = cfa_launch_unpack(k, scratch->items + base[k][0], count[k][0],
-                              scratch->items + base[k][1], count[k][1],
-                              (uint64_t)(uintptr_t)blob_dev, 0, 0, blob_bytes,
-                              reinterpret_cast<unsigned long long *>(cksum_dev), status,
-                              g_grid_cap[dev][k], (uint32_t)kSlabBytes, 1, nullptr, stream);
+        if (!count[k][SLAB] && !count[k][TINY]) continue;
+        e = cfa_launch_unpack(k, scratch->items + base[k][SLAB], count[k][SLAB],
+                              scratch->items + base[k][TINY], count[k][TINY], src, 0, 0,
+                              blob_bytes, ck, status, g_grid_cap[dev][k], (uint32_t)kSlabBytes, 1,
+                              &ctl, stream);
+        ctl.flags = CFA_LAUNCH_EARLY | CFA_LAUNCH_WAIT_LAST | CFA_LAUNCH_RELEASE;
     }
     if (e != cudaSuccess) {
         say("cfa_unpack_noalloc: CUDA error %s", cudaGetErrorString(e));
