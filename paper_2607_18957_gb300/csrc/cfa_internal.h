@@ -147,6 +147,7 @@ typedef struct cfa_host_plan {
     size_t n_copies;
     uint32_t *copy_first;
     uint64_t staged_bytes;
+    uint32_t odd_slab_bytes; /* slab size of copies off the 16-byte grid (opts.slab_bytes: others) */
     uint64_t bytes_read, bytes_written;
     int any_cksum;
 } cfa_host_plan;

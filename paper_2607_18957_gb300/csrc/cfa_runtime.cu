@@ -299,7 +299,9 @@ cfa_status launch(cfa_plan *p, uint32_t c0, uint32_t c1, uint64_t src_base, uint
     const uint64_t hi = std::min<uint64_t>(hp.blob_bytes, (uint64_t)c1 * hp.chunk_bytes);
     const size_t row = (size_t)hp.n_chunks + 1;
     /* the plan's slabs suit a launch over the whole load; one over fewer chunks cuts them */
-    const uint32_t item_bytes = c0 == 0 && c1 == hp.n_chunks ? 0 : hp.opts.slab_bytes;
+    const bool whole = c0 == 0 && c1 == hp.n_chunks;
+    const uint32_t item_bytes = whole ? 0 : hp.opts.slab_bytes;
+    const uint32_t slab_item_bytes = whole ? 0 : std::max(item_bytes, hp.odd_slab_bytes);
     const bool timing_on = (hp.opts.flags & CFA_OPT_TIMING) != 0;
     enum { BULK, BULK_AS_VECTOR, ROWS_AS_STRIDED, STRIDED, VECTOR };
     struct Job {
@@ -366,7 +368,7 @@ cfa_status launch(cfa_plan *p, uint32_t c0, uint32_t c1, uint64_t src_base, uint
         else
             CK(p, cfa_launch_unpack(k, p->d_slabs + J.a0, J.a1 - J.a0, p->d_tiny + J.b0,
                                     J.b1 - J.b0, src_base, period, lo, hi, p->d_ck, p->d_status,
-                                    cap(p->grid_cap[k]), item_bytes, tma, &ctl, s));
+                                    cap(p->grid_cap[k]), slab_item_bytes, tma, &ctl, s));
         p->ck_clear = nullptr; /* this launch clears it */
         p->ck_clear_words = 0;
         if (timing) CK(p, cudaEventRecord(p->t_k1[p->last_launches], s));
