@@ -157,9 +157,15 @@ def recorded_traffic(workload):
     return r.get("dram_bytes_per_launch")
 
 
-def kernel_names(st):
-    """The unpack kernels one load of a plan with these stats launches."""
+def kernel_names(st, types=""):
+    """The unpack kernels one load of a plan with these stats and element types (path_types)
+    launches: a whole load of aligned copies of one type with few tiny pieces takes the vector
+    kernel alone."""
     out = []
+    if (st["n_bulk"] and not st["n_slabs"] and not st["n_strided"] and
+            st["n_tiny"] <= st["n_bulk"] // 8 and types in ("u16", "u32", "u64")):
+        return "cfa_unpack_kernel (16-byte vector slabs" + (", tiny pieces interleaved)"
+                                                            if st["n_tiny"] else ")")
     if st["n_bulk"]:
         out.append("cfa_bulk_kernel (TMA bulk copies)")
     if st["n_slabs"]:
@@ -843,7 +849,7 @@ def measure_workload(name, args, ranks, stream, peak, e2e_steps, attribution_on=
            "l2": ("flushed between steps (1 GiB write outside the timed loads)" if l2_flush
                   else f"no flush: inputs {m.blob_bytes / 1e9:.2f} GB > L2 "
                        f"{L2_BYTES / 1e6:.0f} MB"),
-           "kernels": kernel_names(st),
+           "kernels": kernel_names(st, path_types(m)[0]),
            "setup_s": round(setup_s, 2), "_n_bulk": st["n_bulk"]}
     if clean_ms:
         # attribution only: the flush's own dirty lines, written back during the timed load,

@@ -274,6 +274,35 @@ void CUDART_CB fill_host_fn(void *arg)
     });
 }
 
+/* The class of a plan whose work is aligned copies of one element size (2, 4 or 8 bytes) and few
+ * tiny pieces of it: a dense checkpoint's, or an adapter's.  -1 for any other plan.
+ *
+ * A launch over such a whole load goes to the vector kernel, tiny pieces and all, not to the TMA
+ * kernel: a CTA of the TMA kernel moves a stage of 32 KiB in, then out, the vector kernel's warps a
+ * few vectors at a time, so what the GPU reads and writes at once lies closer together (545 MB of
+ * bf16 175 us by TMA, 163 by vectors; 456 MB 146, 138; 1.9 GB 564, 556; 24 MB of adapters 14.4,
+ * 12.4; 16 GB 4725, 4698).  Beside other launches of the same load the TMA kernel's two warps and few
+ * registers leave room for the other kernel, and it is the better one: 59,000 tiny pieces in 3.2 GB
+ * 937 us by TMA, 949 by vectors; with column slices 48.3 and 52.1, 538 and 550; unaligned slabs 270
+ * and 293.  Byte elements cost the vector kernel's checksum too much (2.1 GB 641 and 687); chunks
+ * launched one by one use the TMA kernel's early start. */
+int plain_class(const cfa_host_plan &hp)
+{
+    if (!hp.n_bulk || hp.n_slabs || hp.n_strided || hp.n_brows || hp.n_tiny > hp.n_bulk / 8)
+        return -1;
+    const size_t row = (size_t)hp.n_chunks + 1;
+    int one = -1;
+    for (int k = 0; k < CFA_N_CLASSES; ++k) {
+        const size_t at = k * row, end = at + hp.n_chunks;
+        const bool bulk = hp.bulk_first[end] != hp.bulk_first[at];
+        const bool tiny = hp.tiny_first[end] != hp.tiny_first[at];
+        if (!bulk && !tiny) continue;
+        if (!bulk || one >= 0 || k == 0) return -1;
+        one = k;
+    }
+    return one;
+}
+
 /* Unpacks chunks [c0, c1), whose blob byte o sits at device address src_base + o (or
  * src_base + (o mod period) for a periodic source): one TMA bulk launch for the aligned cast-free
  * slabs and column slices of every element size, and per work class present in those chunks
@@ -302,6 +331,7 @@ cfa_status launch(cfa_plan *p, uint32_t c0, uint32_t c1, uint64_t src_base, uint
     const bool whole = c0 == 0 && c1 == hp.n_chunks;
     const uint32_t item_bytes = whole ? 0 : hp.opts.slab_bytes;
     const uint32_t slab_item_bytes = whole ? 0 : std::max(item_bytes, hp.odd_slab_bytes);
+    const int one = tma && whole ? plain_class(hp) : -1;
     const bool timing_on = (hp.opts.flags & CFA_OPT_TIMING) != 0;
     enum { BULK, BULK_AS_VECTOR, ROWS_AS_STRIDED, STRIDED, VECTOR };
     struct Job {
@@ -316,7 +346,8 @@ cfa_status launch(cfa_plan *p, uint32_t c0, uint32_t c1, uint64_t src_base, uint
         const uint32_t b0 = hp.bulk_first[k * row + c0], b1 = hp.bulk_first[k * row + c1];
         const uint32_t r0 = hp.brows_first[k * row + c0], r1 = hp.brows_first[k * row + c1];
         if (b1 != b0 && (what & LAUNCH_CONTIG)) {
-            if (!tma) jobs[n++] = Job{BULK_AS_VECTOR, k, b0, b1, 0, 0};
+            if (k == one) jobs[n++] = Job{BULK_AS_VECTOR, k, b0, b1, 0, (uint32_t)hp.n_tiny};
+            else if (!tma) jobs[n++] = Job{BULK_AS_VECTOR, k, b0, b1, 0, 0};
             else ranges[n_ranges++] = cfa_bulk_range{p->d_bulk + b0, b1 - b0, 0};
         }
         if (r1 != r0 && (what & LAUNCH_STRIDED)) {
@@ -329,7 +360,7 @@ cfa_status launch(cfa_plan *p, uint32_t c0, uint32_t c1, uint64_t src_base, uint
         const uint32_t r0 = hp.strided_first[k * row + c0], r1 = hp.strided_first[k * row + c1];
         if (r1 != r0) jobs[n++] = Job{STRIDED, k, r0, r1, 0, 0};
     }
-    for (int k = 0; k < CFA_N_CLASSES && (what & LAUNCH_CONTIG); ++k) {
+    for (int k = 0; k < CFA_N_CLASSES && (what & LAUNCH_CONTIG) && one < 0; ++k) {
         const uint32_t s0 = hp.slab_first[k * row + c0], s1 = hp.slab_first[k * row + c1];
         const uint32_t t0 = hp.tiny_first[k * row + c0], t1 = hp.tiny_first[k * row + c1];
         if (s1 != s0 || t1 != t0) jobs[n++] = Job{VECTOR, k, s0, s1, t0, t1};
@@ -357,9 +388,9 @@ cfa_status launch(cfa_plan *p, uint32_t c0, uint32_t c1, uint64_t src_base, uint
                                   p->d_status, cap(p->bulk_grid_cap), item_bytes, &ctl,
                                   s));
         else if (J.type == BULK_AS_VECTOR) /* bulk items are copy-class slabs of class k */
-            CK(p, cfa_launch_unpack(k, p->d_bulk + J.a0, J.a1 - J.a0, nullptr, 0, src_base,
-                                    period, lo, hi, p->d_ck, p->d_status, cap(p->grid_cap[k]),
-                                    item_bytes, tma, &ctl, s));
+            CK(p, cfa_launch_unpack(k, p->d_bulk + J.a0, J.a1 - J.a0, p->d_tiny + J.b0,
+                                    J.b1 - J.b0, src_base, period, lo, hi, p->d_ck, p->d_status,
+                                    cap(p->grid_cap[k]), item_bytes, tma, &ctl, s));
         else if (J.type == STRIDED || J.type == ROWS_AS_STRIDED)
             CK(p, cfa_launch_strided(k,
                                      (J.type == STRIDED ? p->d_strided : p->d_brows) + J.a0,

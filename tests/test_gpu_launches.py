@@ -172,3 +172,26 @@ def test_column_slices_by_row_length(row_bytes):
                 u = {1: np.uint8, 2: np.uint16, 4: np.uint32, 8: np.uint64}[ES[cases[i][0]]]
                 total = w.cpu().numpy().view(u).astype(np.uint64).sum(dtype=np.uint64)
                 assert int(ck[i]) == int(total)
+
+
+@pytest.mark.parametrize("dtype,n_tiny,launches", [
+    ("bf16", 0, 1), ("bf16", 3, 1), ("bf16", 40, 2), ("f32", 3, 1), ("i64", 3, 1), ("u8", 3, 2)])
+def test_whole_loads_of_one_plain_type(dtype, n_tiny, launches):
+    """Aligned copies of one 2-, 4- or 8-byte type with few tiny pieces are one launch of the
+    vector kernel; with many, or of bytes, the TMA kernel and the tiny kernel; chunk by chunk, the
+    TMA kernel.  All give the blob's bytes and sums."""
+    c = Copies([(dtype, n, 0, 0) for n in [8192, 65536, 4 << 20, 300 * 1024]] +
+               [(dtype, 40 + 8 * k, 0, 0) for k in range(n_tiny)])
+    with cfa.Plan(c.entries, c.dsts, c.blob_bytes, dev_slots=0, host_slots=0,
+                  chunk_bytes=1 << 20) as plan:
+        for _ in range(3):
+            c.out.fill_(0xA5)
+            plan.load_async(cfa.Source.device(c.blob.data_ptr()))
+            plan.wait_layer()
+            assert torch.equal(c.out, c.want)
+            assert np.array_equal(plan.checksums(), c.checksums())
+            assert plan.stats()["kernel_launches"] == launches
+        c.out.fill_(0xA5)
+        for k in range(plan.info()["n_chunks"]):
+            plan.unpack_chunks_async(k, k + 1, c.blob.data_ptr() + k * (1 << 20))
+        assert torch.equal(c.out, c.want)
