@@ -73,6 +73,9 @@ static int cfa_default_fill_threads(void)
  * realigning loop that fills and drains (876 MB 270 us with 128 KiB, 292 with 32; 300 MB of a
  * tensor-parallel rank 105 with 64, 111 with 32). */
 #define CFA_SLAB_ITEMS 16384u
+/* Conversions to a wider type write twice what they read, and gain from small slabs at every size:
+ * bf16 -> fp32 8.8 GB written 2060 us with 32 KiB, 2094 with 64, 2135 with 256. */
+#define CFA_WIDEN_SLAB (32u << 10)
 #define CFA_ODD_SLAB_ITEMS 4096u
 static uint32_t cfa_auto_slab(uint64_t dst_bytes, uint32_t items)
 {
@@ -752,8 +755,9 @@ cfa_status cfa_host_plan_build(const cfa_tensor_entry *entries, size_t n_entries
         st = CFA_ERR_NOMEM;
         goto done;
     }
+    const int auto_slab = o.slab_bytes == 0;
     out->odd_slab_bytes = o.slab_bytes;
-    if (o.slab_bytes == 0) {
+    if (auto_slab) {
         uint64_t dst_total = 0;
         for (size_t i = 0; i < n_entries; ++i) dst_total += info[i].n * (uint64_t)info[i].es_d;
         o.slab_bytes = cfa_auto_slab(dst_total, CFA_SLAB_ITEMS);
@@ -771,8 +775,9 @@ cfa_status cfa_host_plan_build(const cfa_tensor_entry *entries, size_t n_entries
             const uint32_t cls =
                 pc->conv ? CFA_CLASS_OF_CONV(pc->conv) : (uint32_t)log2_small(in->es_s);
             const uint64_t a0 = (uint64_t)(uintptr_t)dsts[pc->dst_index].dev_ptr + pc->dst_offset;
-            const uint64_t slab = pc->conv || ((pc->src_offset | a0) & 15u) == 0
-                                      ? o.slab_bytes : out->odd_slab_bytes;
+            uint64_t slab = pc->conv || ((pc->src_offset | a0) & 15u) == 0 ? o.slab_bytes
+                                                                        : out->odd_slab_bytes;
+            if (auto_slab && pc->conv && in->es_d > in->es_s) slab = CFA_WIDEN_SLAB;
             if (pc->rows > 1) {
                 /* blocks of whole rows, about slab_bytes of destination each */
                 const uint64_t row_d = in->cols * (uint64_t)in->es_d;
