@@ -508,7 +508,8 @@ extern "C" cudaError_t cfa_launch_bulk(const cfa_bulk_range *ranges, uint32_t n_
     }
     if (n_items == 0) return cudaSuccess;
     if (n_items >= (1ull << 31)) return cudaErrorInvalidValue;
-    a.parts_log2 = cfa_parts_log2((uint32_t)n_items, (uint32_t)grid_cap, item_bytes);
+    a.parts_log2 = cfa_parts_log2((uint32_t)n_items, (uint32_t)grid_cap, item_bytes,
+                                  CFA_MIN_PART_BYTES);
     a.n_items = (uint32_t)n_items << a.parts_log2;
     a.spin_limit = kSpinLimit;
     a.src_base = src_base;

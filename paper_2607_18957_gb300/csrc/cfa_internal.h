@@ -153,22 +153,27 @@ typedef struct cfa_host_plan {
 } cfa_host_plan;
 
 /*
- * Block-level items are cut once more at launch when there are fewer than eight of them per
- * resident CTA: into 2^cfa_parts_log2 equal parts each, until there are eight, but of at least
- * CFA_MIN_PART_BYTES (source or destination bytes, whichever is more), and cut where the
- * destination is a multiple of CFA_PART_ALIGN.  The plan's slabs suit the whole load, and the
- * no-alloc entry point's items (2 MiB) its fixed scratch; a launch over one chunk, or over a
- * small checkpoint, would otherwise leave most CTAs without work.  item_bytes is the caller's
- * usual item size: 16 KiB parts cost more in descriptors and half-filled stages than they gained
- * (1,000 tensors of up to 1 MiB: 49.3 us against 46.7 with items of 32 KiB left whole).
+ * Block-level items are cut once more at launch when there are too few of them for the grid: into
+ * 2^cfa_parts_log2 equal parts each, cut where the destination is a multiple of CFA_PART_ALIGN,
+ * until there are CFA_PARTS_PER_CTA for each resident CTA or the parts of an item of the caller's
+ * usual size, item_bytes, are down to part_bytes (source or destination bytes, whichever is more; a
+ * smaller item has fewer parts, none below CFA_MIN_PART_BYTES).  The plan's slabs suit the whole
+ * load (item_bytes 0: left whole), and the no-alloc entry point's items (2 MiB) its fixed scratch; a
+ * launch over one chunk, or over a small checkpoint, would otherwise leave most CTAs without work,
+ * and large items spread the addresses in flight over too much memory (cfa_auto_slab).  A chunk's
+ * items go down to 32 KiB.  The no-alloc items stop at 64 KiB: fp32 -> bf16, 252 MB, 118 us
+ * so, 125 with 32 KiB parts; 945 MB 417 and 429, with eight parts a CTA 433; bf16, 1.1 GB, 673 with
+ * 64 KiB, 680 with 128, 686 with 512.
  */
 #define CFA_MIN_PART_BYTES 32768u
 #define CFA_PART_ALIGN 128u
-static inline uint32_t cfa_parts_log2(uint32_t n_items, uint32_t grid_cap, uint32_t item_bytes)
+#define CFA_PARTS_PER_CTA 64u
+static inline uint32_t cfa_parts_log2(uint32_t n_items, uint32_t grid_cap, uint64_t item_bytes,
+                                      uint32_t part_bytes)
 {
     uint32_t k = 0;
-    while (n_items && (item_bytes >> (k + 1)) >= CFA_MIN_PART_BYTES &&
-           ((uint64_t)n_items << k) < 8ull * grid_cap)
+    while (n_items && (item_bytes >> (k + 1)) >= part_bytes &&
+           ((uint64_t)n_items << k) < (uint64_t)CFA_PARTS_PER_CTA * grid_cap)
         ++k;
     return k;
 }

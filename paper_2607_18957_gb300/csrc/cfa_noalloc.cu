@@ -42,13 +42,15 @@ extern "C" cudaError_t cfa_launch_unpack(int cls, const cfa_work *slabs, uint32_
                                          uint64_t src_base, uint64_t src_period,
                                          uint64_t src_lo, uint64_t src_hi,
                                          unsigned long long *ck, int *status, int grid_cap,
-                                         uint32_t item_bytes, int dev_src,
-                                         const cfa_launch_ctl *ctl, cudaStream_t stream);
+                                         uint32_t item_bytes, uint32_t part_bytes,
+                                         int dev_src, const cfa_launch_ctl *ctl,
+                                         cudaStream_t stream);
 
 namespace {
 
 constexpr int kMaxDevices = 64;
 constexpr uint64_t kSlabBytes = 2ull << 20; /* destination bytes per block-level item */
+constexpr uint32_t kPartBytes = 64u << 10; /* they are cut down to at launch (cfa_parts_log2) */
 constexpr uint64_t kTinyBytes = 8192;      /* below this, one warp per tensor */
 
 /* Device scratch: CFA_NOALLOC_MAX_ITEMS descriptors, then the status word. */
@@ -401,7 +403,8 @@ extern "C" cfa_status cfa_unpack_noalloc(const cfa_tensor_entry *entries, size_t
         if (!count[k][SLAB] && !count[k][TINY]) continue;
         e = cfa_launch_unpack(k, scratch->items + base[k][SLAB], count[k][SLAB],
                               scratch->items + base[k][TINY], count[k][TINY], src, 0, 0,
-                              blob_bytes, ck, status, g_grid_cap[dev][k], (uint32_t)kSlabBytes, 1,
+                              blob_bytes, ck, status, g_grid_cap[dev][k], (uint32_t)kSlabBytes,
+                              kPartBytes, 1,
                               &ctl, stream);
         ctl.flags = CFA_LAUNCH_EARLY | CFA_LAUNCH_WAIT_LAST | CFA_LAUNCH_RELEASE;
     }

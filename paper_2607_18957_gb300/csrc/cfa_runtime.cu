@@ -63,8 +63,9 @@ extern "C" cudaError_t cfa_launch_unpack(int cls, const cfa_work *slabs, uint32_
                                          uint64_t src_base, uint64_t src_period,
                                          uint64_t src_lo, uint64_t src_hi,
                                          unsigned long long *ck, int *status, int grid_cap,
-                                         uint32_t item_bytes, int dev_src,
-                                         const cfa_launch_ctl *ctl, cudaStream_t stream);
+                                         uint32_t item_bytes, uint32_t part_bytes,
+                                         int dev_src, const cfa_launch_ctl *ctl,
+                                         cudaStream_t stream);
 
 namespace {
 
@@ -390,7 +391,8 @@ cfa_status launch(cfa_plan *p, uint32_t c0, uint32_t c1, uint64_t src_base, uint
         else if (J.type == BULK_AS_VECTOR) /* bulk items are copy-class slabs of class k */
             CK(p, cfa_launch_unpack(k, p->d_bulk + J.a0, J.a1 - J.a0, p->d_tiny + J.b0,
                                     J.b1 - J.b0, src_base, period, lo, hi, p->d_ck, p->d_status,
-                                    cap(p->grid_cap[k]), item_bytes, tma, &ctl, s));
+                                    cap(p->grid_cap[k]), item_bytes, CFA_MIN_PART_BYTES, tma,
+                                    &ctl, s));
         else if (J.type == STRIDED || J.type == ROWS_AS_STRIDED)
             CK(p, cfa_launch_strided(k,
                                      (J.type == STRIDED ? p->d_strided : p->d_brows) + J.a0,
@@ -399,7 +401,8 @@ cfa_status launch(cfa_plan *p, uint32_t c0, uint32_t c1, uint64_t src_base, uint
         else
             CK(p, cfa_launch_unpack(k, p->d_slabs + J.a0, J.a1 - J.a0, p->d_tiny + J.b0,
                                     J.b1 - J.b0, src_base, period, lo, hi, p->d_ck, p->d_status,
-                                    cap(p->grid_cap[k]), slab_item_bytes, tma, &ctl, s));
+                                    cap(p->grid_cap[k]), slab_item_bytes, CFA_MIN_PART_BYTES, tma,
+                                    &ctl, s));
         p->ck_clear = nullptr; /* this launch clears it */
         p->ck_clear_words = 0;
         if (timing) CK(p, cudaEventRecord(p->t_k1[p->last_launches], s));

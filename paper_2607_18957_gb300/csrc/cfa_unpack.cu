@@ -1302,15 +1302,17 @@ extern "C" cudaError_t cfa_launch_unpack(int cls, const cfa_work *slabs, uint32_
                                          uint64_t src_base, uint64_t src_period,
                                          uint64_t src_lo, uint64_t src_hi,
                                          unsigned long long *ck, int *status, int grid_cap,
-                                         uint32_t item_bytes, int dev_src,
-                                         const cfa_launch_ctl *ctl, cudaStream_t stream)
+                                         uint32_t item_bytes, uint32_t part_bytes,
+                                         int dev_src, const cfa_launch_ctl *ctl,
+                                         cudaStream_t stream)
 {
     if (cls < 0 || cls >= CFA_N_CLASSES || grid_cap <= 0) return cudaErrorInvalidValue;
     /* the fp32 -> 16-bit classes read twice what they write */
     const bool narrows = cls == CFA_CLASS_OF_CONV(CFA_CONV_F32_BF16) ||
                          cls == CFA_CLASS_OF_CONV(CFA_CONV_F32_F16);
-    const uint32_t parts_log2 =
-        cfa_parts_log2(n_slabs, (uint32_t)grid_cap, narrows ? 2 * item_bytes : item_bytes);
+    const uint32_t parts_log2 = cfa_parts_log2(n_slabs, (uint32_t)grid_cap,
+                                               (uint64_t)item_bytes << (narrows ? 1 : 0),
+                                               part_bytes);
     const uint64_t items =
         ((uint64_t)n_slabs << parts_log2) + (n_tiny + kTinyPerGroup - 1) / kTinyPerGroup;
     if (items == 0) return cudaSuccess;
