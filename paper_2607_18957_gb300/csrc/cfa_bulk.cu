@@ -183,8 +183,8 @@ __device__ __forceinline__ bool bulk_part(uint64_t dst, uint32_t total, uint32_t
     return true;
 }
 
-/* A descriptor as it lies in memory (cfa_work, or cfa_swork with its fifth word).  It is fetched one
- * part ahead and decoded only when its part comes up: any arithmetic at the fetch, even a copy of
+/* A descriptor as it lies in memory (cfa_work, or cfa_swork with its fifth word).  It is fetched
+ * one part ahead and decoded only when its part comes up: any arithmetic at the fetch, even a copy of
  * one of its words, would wait for the load there and then (8-bit checkpoint in 64 MiB chunks: 1244
  * us, now 1233). */
 struct RawItem {
@@ -520,7 +520,8 @@ extern "C" cudaError_t cfa_launch_bulk(const cfa_bulk_range *ranges, uint32_t n_
     a.status = status;
     const uint32_t grid = a.n_items < (uint32_t)grid_cap ? a.n_items : (uint32_t)grid_cap;
     a.ctl = ctl ? *ctl : cfa_launch_ctl{};
-    return launch_ctl(rows ? cfa_bulk_kernel<true> : cfa_bulk_kernel<false>, grid, kThreads, kSmemBytes, stream, a);
+    return launch_ctl(rows ? cfa_bulk_kernel<true> : cfa_bulk_kernel<false>, grid, kThreads,
+                      kSmemBytes, stream, a);
 }
 
 /* Self-test of the bounded waits: one CTA of the TMA kernel over one valid 16-byte item, with a
@@ -535,7 +536,8 @@ extern "C" cudaError_t cfa_bulk_selftest_timeout(int *status_host)
     cudaError_t e = cudaSuccess;
     if (!status_host) return cudaErrorInvalidValue;
     *status_host = -1;
-    if ((e = cudaFuncSetAttribute(cfa_bulk_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    if ((e = cudaFuncSetAttribute(cfa_bulk_kernel<false>,
+                                  cudaFuncAttributeMaxDynamicSharedMemorySize,
                                   (int)kSmemBytes)) != cudaSuccess)
         return e;
     if ((e = cudaMalloc(&d_item, sizeof(cfa_work))) != cudaSuccess) goto out;

@@ -114,7 +114,8 @@ cudaError_t put(PutArgs<CAP> &a, cfa_work *to, const cfa_work *from, uint32_t n,
     return cfa_dev::launch_ctl(cfa_put_kernel<CAP>, (unsigned)grid, kPutThreads, 0, stream, a);
 }
 
-/* Uploads n descriptors to `to` in stream order; the first launch clears what ctl and status say. */
+/* Uploads n descriptors to `to` in stream order; the first launch clears the status word and the
+ * checksums. */
 cudaError_t put_items(cfa_work *to, const cfa_work *from, uint32_t n, int *status,
                       unsigned long long *clear, uint64_t clear_words, cudaStream_t stream)
 {

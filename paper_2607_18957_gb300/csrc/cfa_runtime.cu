@@ -54,7 +54,8 @@ extern "C" cudaError_t cfa_launch_bulk(const cfa_bulk_range *ranges, uint32_t n_
                                        uint64_t src_base, uint64_t src_period,
                                        uint64_t src_lo, uint64_t src_hi,
                                        unsigned long long *ck, int *status, int grid_cap,
-                                       uint32_t item_bytes, const cfa_launch_ctl *ctl, cudaStream_t stream);
+                                       uint32_t item_bytes, const cfa_launch_ctl *ctl,
+                                       cudaStream_t stream);
 extern "C" cudaError_t cfa_bulk_selftest_timeout(int *status_host);
 extern "C" cudaError_t cfa_launch_pull(const void *src, void *dst, uint64_t bytes, int grid,
                                        cudaStream_t stream);
@@ -282,8 +283,8 @@ void CUDART_CB fill_host_fn(void *arg)
  * kernel: a CTA of the TMA kernel moves a stage of 32 KiB in, then out, the vector kernel's warps a
  * few vectors at a time, so what the GPU reads and writes at once lies closer together (545 MB of
  * bf16 175 us by TMA, 163 by vectors; 456 MB 146, 138; 1.9 GB 564, 556; 24 MB of adapters 14.4,
- * 12.4; 16 GB 4725, 4698).  Beside other launches of the same load the TMA kernel's two warps and few
- * registers leave room for the other kernel, and it is the better one: 59,000 tiny pieces in 3.2 GB
+ * 12.4; 16 GB 4725, 4698).  Beside other launches of the same load the TMA kernel's two warps and
+ * few registers leave room for the other kernel, and it is the better one: 59,000 tiny pieces in 3.2 GB
  * 937 us by TMA, 949 by vectors; with column slices 48.3 and 52.1, 538 and 550; unaligned slabs 270
  * and 293.  Byte elements cost the vector kernel's checksum too much (2.1 GB 641 and 687); chunks
  * launched one by one use the TMA kernel's early start. */
@@ -307,7 +308,8 @@ int plain_class(const cfa_host_plan &hp)
 /* Unpacks chunks [c0, c1), whose blob byte o sits at device address src_base + o (or
  * src_base + (o mod period) for a periodic source): one TMA bulk launch for the aligned cast-free
  * slabs and column slices of every element size, and per work class present in those chunks
- * (normally one) a launch for its other column slices and a vector launch for everything else.  The kernels of one group write
+ * (normally one) a launch for its other column slices and a vector launch for everything else.
+ * The kernels of one group write
  * disjoint destination bytes and add their checksums atomically, so they are independent: each
  * releases the next as soon as it runs, so that one kernel's last CTAs overlap the next kernel's
  * first, and ends only after the one before it, so that what follows on `s` follows them all.

@@ -193,7 +193,7 @@ template <int CONV> __device__ __forceinline__ uint32_t convert1(uint32_t x)
  * instructions; the NaN results that the format fixes differently (convert1) are put right
  * afterwards.  With convert1's integer forms on every element the 16-bit classes were bound by
  * instructions and divergent branches: fp16 -> bf16, 1.9 GB: 1170 us, now 580 (0.49 and 0.99 of
- * the copy rate); fp32 -> fp16, 1.0 GB: 583, now 460 (0.78, 0.99).  convert1 serves a run's ends. */
+ * the copy rate); fp32 -> fp16, 1.0 GB: 583, now 446 (0.78, 1.0).  convert1 serves a run's ends. */
 
 /* fp32 pair -> bf16 pair, round to nearest even.  The instruction's only NaN result is 0x7FFF; the
  * signed minimum with 0x7FC0 turns it into the quiet NaN that convert1 gives and changes nothing
@@ -955,9 +955,72 @@ __device__ __forceinline__ TinyItem tiny_fetch(const UnpackArgs &a, uint32_t gro
     return it;
 }
 
+/* A lane's share of an item's checksum: 8- and 16-bit elements add up to less than 2^32 over an
+ * item (CFA_TINY_SEG_BYTES), so one dot-product instruction with ones per word and 32 bits do. */
+template <int ES> struct TinySum {
+    typedef uint64_t T;
+    static __device__ __forceinline__ void add(T &acc, const uint4 &v) { acc += vsum<ES>(v); }
+};
+template <> struct TinySum<1> {
+    typedef uint32_t T;
+    static __device__ __forceinline__ void add(T &acc, const uint4 &v)
+    {
+        acc = __dp4a(v.x, 0x01010101u, acc);
+        acc = __dp4a(v.y, 0x01010101u, acc);
+        acc = __dp4a(v.z, 0x01010101u, acc);
+        acc = __dp4a(v.w, 0x01010101u, acc);
+    }
+};
+template <> struct TinySum<2> {
+    typedef uint32_t T;
+    static __device__ __forceinline__ void add(T &acc, const uint4 &v)
+    {
+        acc = __dp2a_lo(v.x, 0x0101u, acc);
+        acc = __dp2a_lo(v.y, 0x0101u, acc);
+        acc = __dp2a_lo(v.z, 0x0101u, acc);
+        acc = __dp2a_lo(v.w, 0x0101u, acc);
+    }
+};
+
+/* Bytes [0, n) of v kept, the others zeroed. */
+__device__ __forceinline__ uint4 keep_first(uint4 v, uint32_t n)
+{
+    auto mask = [n](uint32_t at) {
+        return n >= at + 4u ? 0xFFFFFFFFu : n > at ? (1u << (8u * (n - at))) - 1u : 0u;
+    };
+    return make_uint4(v.x & mask(0), v.y & mask(4), v.z & mask(8), v.w & mask(12));
+}
+
+/* Stores the first n < 16 bytes of v (a multiple of ES) at the aligned block d: 8, 4, 2 and 1
+ * bytes as the bits of n say. */
+template <int ES> __device__ __forceinline__ void store_first(uint8_t *d, uint4 v, uint32_t n)
+{
+    if (n & 8u) {
+        *reinterpret_cast<uint2 *>(d) = make_uint2(v.x, v.y);
+        v.x = v.z;
+        v.y = v.w;
+    }
+    if constexpr (ES <= 4) {
+        if (n & 4u) {
+            *reinterpret_cast<uint32_t *>(d + (n & 8u)) = v.x;
+            v.x = v.y;
+        }
+    }
+    if constexpr (ES <= 2) {
+        if (n & 2u) {
+            *reinterpret_cast<uint16_t *>(d + (n & 12u)) = (uint16_t)v.x;
+            v.x >>= 16;
+        }
+    }
+    if constexpr (ES == 1) {
+        if (n & 1u) d[n & 14u] = (uint8_t)v.x;
+    }
+}
+
 /* Issues the cp.async copies of an item's aligned source vectors into `stage` (lanes sub, sub +
- * 8, ...).  Items that fail the kernel's checks, or exceed CFA_TINY_SEG_BYTES, are flagged in
- * the status word and dropped. */
+ * L, ..., every copy predicated: no loop whose length differs between the items of a warp).  Items
+ * that fail the kernel's checks, or exceed CFA_TINY_SEG_BYTES, are flagged in the status word and
+ * dropped. */
 template <int CLS, int L>
 __device__ __forceinline__ void tiny_issue(const UnpackArgs &a, TinyItem &it, uint4 *stage,
                                            uint32_t sub)
@@ -972,27 +1035,33 @@ __device__ __forceinline__ void tiny_issue(const UnpackArgs &a, TinyItem &it, ui
     const uint64_t off = a.src_period ? it.w.src % a.src_period : it.w.src;
     const uint64_t src = a.src_base + off;
     const uint32_t ps = (uint32_t)(src & 15u);
-    const uint32_t nv = (ps + bytes + 15u) >> 4;
-    const uint4 *s = reinterpret_cast<const uint4 *>(src - ps);
-    for (uint32_t v = sub; v < nv; v += L) cp_async16(stage + v, s + v);
+    const uint32_t nv = (ps + bytes + 15u) >> 4; /* CFA_TINY_SEG_BYTES / 16 + 1 at most */
+    const uint4 *s = reinterpret_cast<const uint4 *>(src - ps) + sub;
+    stage += sub;
+#pragma unroll
+    for (uint32_t v = 0; v < CFA_TINY_SEG_BYTES / 16 + 1; v += L)
+        if (v + sub < nv) cp_async16(stage + v, s + v);
 }
 
 /* Writes a staged item to its destination: destination vector i (aligned) holds staged bytes
  * [16 i + delta, 16 i + delta + 16), delta = source phase - destination phase, so with
  * delta = 16 j0 + k it is staged vector i + j0 (k = 0) or bytes k .. of vectors i + j0 and
- * i + j0 + 1.  The whole vectors go in a tight loop over the segment's lanes; the partial first
- * and last ones (when the item covers them only in part) go to lanes 0 and 1, element by
- * element.  Returns this lane's checksum share. */
+ * i + j0 + 1.  The whole vectors go over the segment's lanes, every store predicated; the partial
+ * first and last ones (when the item covers them only in part) go to lanes 0 and 1.  Returns this
+ * lane's checksum share. */
 template <int CLS, int L>
-__device__ __forceinline__ uint64_t tiny_store(const UnpackArgs &a, const TinyItem &it,
-                                               const uint4 *stage, uint32_t sub)
+__device__ __forceinline__ typename TinySum<(1 << CLS)>::T
+tiny_store(const UnpackArgs &a, const TinyItem &it, const uint4 *stage, uint32_t sub)
 {
     constexpr int ES = 1 << CLS;
-    if (!it.live) return 0;
+    typedef TinySum<ES> Sum;
+    constexpr uint32_t kFull = CFA_TINY_SEG_BYTES / 16; /* whole vectors of an item, at most */
+    typename Sum::T acc = 0;
+    if (!it.live) return acc;
     const uint32_t bytes = it.w.n << CLS;
-    const uint64_t off = a.src_period ? it.w.src % a.src_period : it.w.src;
-    const uint32_t ps = (uint32_t)((a.src_base + off) & 15u);
-    const uint32_t dp = (uint32_t)(it.w.dst & 15u);
+    /* only the low bits matter; a period is a whole number of chunks, so a multiple of 256 */
+    const uint32_t ps = ((uint32_t)a.src_base + (uint32_t)it.w.src) & 15u;
+    const uint32_t dp = (uint32_t)it.w.dst & 15u;
     uint4 *d = reinterpret_cast<uint4 *>(it.w.dst - dp);
     const uint32_t end = dp + bytes;
     const uint32_t nv = (end + 15u) >> 4;
@@ -1001,21 +1070,29 @@ __device__ __forceinline__ uint64_t tiny_store(const UnpackArgs &a, const TinyIt
     const uint32_t k = (uint32_t)delta & 15u;
     const bool part0 = dp != 0 || (nv == 1 && (end & 15u) != 0);
     const bool part1 = nv > 1 && (end & 15u) != 0;
-    const uint32_t f0 = part0 ? 1u : 0u, f1 = part1 ? nv - 1u : (nv > f0 ? nv : f0);
-    uint64_t acc = 0;
-    if (k == 0) {
-        for (uint32_t i = f0 + sub; i < f1; i += L) {
-            const uint4 v = stage[i]; /* k == 0 means delta == 0 */
-            st_stream(d + i, v);
-            acc += vsum<ES>(v);
-        }
+    const uint32_t f0 = part0 ? 1u : 0u;
+    const uint32_t first = f0 + sub, last = nv - (part1 ? 1u : 0u); /* whole ones: [f0, last) */
+    if (k == 0) { /* delta == 0 */
+        const uint4 *s = stage + first;
+        uint4 *t = d + first;
+#pragma unroll
+        for (uint32_t v = 0; v < kFull; v += L)
+            if (first + v < last) {
+                const uint4 x = s[v];
+                st_stream(t + v, x);
+                Sum::add(acc, x);
+            }
     } else {
-        for (uint32_t i = f0 + sub; i < f1; i += L) {
-            const int j = (int)i + j0; /* >= 0: i >= 1 here when j0 = -1 (part0 is then set) */
-            const uint4 v = funnel16(stage[j], stage[j + 1], k);
-            st_stream(d + i, v);
-            acc += vsum<ES>(v);
-        }
+        /* j0 = -1 only with part0 set, so first + j0 >= 0 */
+        const uint4 *s = stage + ((int)first + j0);
+        uint4 *t = d + first;
+#pragma unroll 2
+        for (uint32_t v = 0; v < kFull; v += L)
+            if (first + v < last) {
+                const uint4 x = funnel16(s[v], s[v + 1], k);
+                st_stream(t + v, x);
+                Sum::add(acc, x);
+            }
     }
     if ((sub == 0 && part0) || (sub == 1 && part1)) {
         const uint32_t i = sub == 0 ? 0u : nv - 1u;
@@ -1024,8 +1101,13 @@ __device__ __forceinline__ uint64_t tiny_store(const UnpackArgs &a, const TinyIt
         const uint4 v = k ? funnel16(lo_v, stage[j + 1], k) : lo_v;
         const uint32_t lo = i == 0 ? dp : 0u;
         const uint32_t hi = end - 16u * i < 16u ? end - 16u * i : 16u;
-        store_part<ES>(reinterpret_cast<uint8_t *>(d + i), v, lo, hi);
-        acc += vsum<ES>(keep_bytes(v, lo, hi));
+        if (lo == 0) { /* the item's last bytes */
+            store_first<ES>(reinterpret_cast<uint8_t *>(d + i), v, hi);
+            Sum::add(acc, keep_first(v, hi));
+        } else {
+            store_part<ES>(reinterpret_cast<uint8_t *>(d + i), v, lo, hi);
+            Sum::add(acc, keep_bytes(v, lo, hi));
+        }
     }
     return acc;
 }
@@ -1036,7 +1118,11 @@ __device__ __forceinline__ uint64_t tiny_store(const UnpackArgs &a, const TinyIt
  * meanwhile.  The source bytes wait in shared memory (dynamic: two slots per lane group), not
  * in registers, so memory-level parallelism does not cost occupancy; with four lanes per item a
  * warp carries eight items at once, so the per-item work (descriptor, checks, checksum
- * reduction) takes half the warp instructions it would with eight lanes. */
+ * reduction) takes half the warp instructions it would with eight lanes.  Copies and stores are
+ * predicated, not looped over, and 8- and 16-bit sums take one dot product a word (200,000 tensors
+ * of 4 B - 4 KiB, 117 MB: 56.7 us a load with loops, 53.9 now; 49 of them in the kernel, bound by the
+ * latency of each item's two fetches.  Items of 256 bytes with three in flight per group took 57.7:
+ * more items cost more than more bytes in flight gained). */
 constexpr int kStagedLanes = 4;
 constexpr int kStagedPerWarp = 32 / kStagedLanes;
 constexpr uint32_t kStagedPerGroup = kWarps * kStagedPerWarp;
@@ -1065,10 +1151,11 @@ __device__ __forceinline__ void tiny_staged(const UnpackArgs &a)
         cp_async_commit();
         cp_async_wait_1(); /* this lane's copies of item k have landed */
         __syncwarp(mask);  /* and the other lanes' of the group */
-        uint64_t v = tiny_store<CLS, L>(a, cur, (k & 1) ? buf1 : buf0, sub);
+        auto v = tiny_store<CLS, L>(a, cur, (k & 1) ? buf1 : buf0, sub);
 #pragma unroll
         for (int q = L / 2; q > 0; q >>= 1) v += __shfl_down_sync(mask, v, q, L);
-        if (sub == 0 && cur.live && cur.w.ck != CFA_NO_CK) atomicAdd(a.ck + cur.w.ck, v);
+        if (sub == 0 && cur.live && cur.w.ck != CFA_NO_CK)
+            atomicAdd(a.ck + cur.w.ck, (unsigned long long)v);
         __syncwarp(mask);  /* the slot of item k is read; item k + 2 may be copied into it */
         cur = nxt;
         nxt = after;
