@@ -159,11 +159,12 @@ def recorded_traffic(workload):
 
 def kernel_names(st, types=""):
     """The unpack kernels one load of a plan with these stats and element types (path_types)
-    launches: a whole load of aligned copies of one type with few tiny pieces takes the vector
-    kernel alone."""
+    launches: a whole load of up to 32 GiB of aligned copies of one type with few tiny pieces takes
+    the vector kernel alone."""
     out = []
     if (st["n_bulk"] and not st["n_slabs"] and not st["n_strided"] and
-            st["n_tiny"] <= st["n_bulk"] // 8 and types in ("u16", "u32", "u64")):
+            st["n_tiny"] <= st["n_bulk"] // 8 and types in ("u16", "u32", "u64") and
+            st["bytes_written"] <= 32 << 30):
         return "cfa_unpack_kernel (16-byte vector slabs" + (", tiny pieces interleaved)"
                                                             if st["n_tiny"] else ")")
     if st["n_bulk"]:

@@ -287,10 +287,15 @@ void CUDART_CB fill_host_fn(void *arg)
  * few registers leave room for the other kernel, and it is the better one: 59,000 tiny pieces in 3.2 GB
  * 937 us by TMA, 949 by vectors; with column slices 48.3 and 52.1, 538 and 550; unaligned slabs 270
  * and 293.  Byte elements cost the vector kernel's checksum too much (2.1 GB 641 and 687); chunks
- * launched one by one use the TMA kernel's early start. */
+ * launched one by one use the TMA kernel's early start.  Very large loads keep the TMA kernel as well:
+ * 141 GB out of an 8 GiB periodic source took 42.8 ms by vectors, 41.1 by TMA; the line lies between
+ * the two sizes measured. */
+constexpr uint64_t kPlainMost = 32ull << 30; /* destination bytes */
+
 int plain_class(const cfa_host_plan &hp)
 {
-    if (!hp.n_bulk || hp.n_slabs || hp.n_strided || hp.n_brows || hp.n_tiny > hp.n_bulk / 8)
+    if (hp.bytes_written > kPlainMost || !hp.n_bulk || hp.n_slabs || hp.n_strided ||
+        hp.n_brows || hp.n_tiny > hp.n_bulk / 8)
         return -1;
     const size_t row = (size_t)hp.n_chunks + 1;
     int one = -1;
