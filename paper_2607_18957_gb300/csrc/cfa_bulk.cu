@@ -16,7 +16,7 @@
  * An item is a contiguous run, or a block of rows of a column slice: then one bulk load per row
  * gathers the rows back to back in the stage and one bulk store writes them.
  * One launch takes the items of every element size (the consumer sums each stage by its item's
- * size), cut into parts where there are too few for the grid (cfa_parts_log2).  With a launch per
+ * size), cut into parts (cfa_parts_log2).  With a launch per
  * element size, forked and joined with events, and whole 256 KiB slabs, an 8-bit checkpoint with
  * block scales unpacked in 64 MiB chunks (1.4 to 3 launches a chunk, 256 items for 456 CTAs) took
  * 1630 us for 3.4 GB; one launch of parts 1370.
@@ -493,7 +493,8 @@ extern "C" cudaError_t cfa_launch_bulk(const cfa_bulk_range *ranges, uint32_t n_
                                        uint64_t src_base, uint64_t src_period,
                                        uint64_t src_lo, uint64_t src_hi,
                                        unsigned long long *ck, int *status, int grid_cap,
-                                       uint32_t item_bytes, const cfa_launch_ctl *ctl,
+                                       uint32_t item_bytes, uint32_t part_bytes,
+                                       const cfa_launch_ctl *ctl,
                                        cudaStream_t stream)
 {
     if (n_ranges > CFA_BULK_RANGES || grid_cap <= 0) return cudaErrorInvalidValue;
@@ -508,8 +509,8 @@ extern "C" cudaError_t cfa_launch_bulk(const cfa_bulk_range *ranges, uint32_t n_
     }
     if (n_items == 0) return cudaSuccess;
     if (n_items >= (1ull << 31)) return cudaErrorInvalidValue;
-    a.parts_log2 = cfa_parts_log2((uint32_t)n_items, (uint32_t)grid_cap, item_bytes,
-                                  CFA_MIN_PART_BYTES);
+    a.parts_log2 = cfa_parts_log2(item_bytes, part_bytes);
+    if ((n_items << a.parts_log2) >= (1ull << 31)) return cudaErrorInvalidValue;
     a.n_items = (uint32_t)n_items << a.parts_log2;
     a.spin_limit = kSpinLimit;
     a.src_base = src_base;

@@ -147,34 +147,28 @@ typedef struct cfa_host_plan {
     size_t n_copies;
     uint32_t *copy_first;
     uint64_t staged_bytes;
-    uint32_t odd_slab_bytes; /* slab size of copies off the 16-byte grid (opts.slab_bytes: others) */
+    uint32_t part_bytes; /* a launch over the whole load cuts its slabs to; 0: leaves them whole */
     uint64_t bytes_read, bytes_written;
     int any_cksum;
 } cfa_host_plan;
 
 /*
- * Block-level items are cut once more at launch when there are too few of them for the grid: into
- * 2^cfa_parts_log2 equal parts each, cut where the destination is a multiple of CFA_PART_ALIGN,
- * until there are CFA_PARTS_PER_CTA for each resident CTA or the parts of an item of the caller's
- * usual size, item_bytes, are down to part_bytes (source or destination bytes, whichever is more; a
- * smaller item has fewer parts, none below CFA_MIN_PART_BYTES).  The plan's slabs suit the whole
- * load (item_bytes 0: left whole), and the no-alloc entry point's items (2 MiB) its fixed scratch; a
- * launch over one chunk, or over a small checkpoint, would otherwise leave most CTAs without work,
- * and large items spread the addresses in flight over too much memory (cfa_auto_slab).  A chunk's
- * items go down to 32 KiB.  The no-alloc items stop at 64 KiB: fp32 -> bf16, 252 MB, 118 us
- * so, 125 with 32 KiB parts; 945 MB 417 and 429, with eight parts a CTA 433; bf16, 1.1 GB, 673 with
- * 64 KiB, 680 with 128, 686 with 512.
+ * Block-level items are cut once more at launch: into 2^cfa_parts_log2 equal parts each, cut where
+ * the destination is a multiple of CFA_PART_ALIGN, so that the parts of an item of the caller's usual
+ * size, item_bytes, hold part_bytes or more (source or destination bytes, whichever is more; a
+ * smaller item has fewer parts, none below CFA_MIN_PART_BYTES).  The plan's slabs, and the no-alloc
+ * entry point's 2 MiB items, are few and large for the sake of their descriptors; a launch over one
+ * chunk or a small checkpoint would leave most CTAs without work, and large items spread the
+ * addresses in flight over too much memory (cfa_auto_part).  A chunk's items go down to 32 KiB.
+ * The no-alloc items stop at 64 KiB: fp32 -> bf16, 252 MB, 118 us so, 125 with 32 KiB parts; 945 MB
+ * 417 and 429; bf16, 1.1 GB, 673 with 64 KiB, 680 with 128, 686 with 512.
  */
 #define CFA_MIN_PART_BYTES 32768u
 #define CFA_PART_ALIGN 128u
-#define CFA_PARTS_PER_CTA 64u
-static inline uint32_t cfa_parts_log2(uint32_t n_items, uint32_t grid_cap, uint64_t item_bytes,
-                                      uint32_t part_bytes)
+static inline uint32_t cfa_parts_log2(uint64_t item_bytes, uint32_t part_bytes)
 {
     uint32_t k = 0;
-    while (n_items && (item_bytes >> (k + 1)) >= part_bytes &&
-           ((uint64_t)n_items << k) < (uint64_t)CFA_PARTS_PER_CTA * grid_cap)
-        ++k;
+    while (part_bytes && (item_bytes >> (k + 1)) >= part_bytes) ++k;
     return k;
 }
 

@@ -61,26 +61,28 @@ static int cfa_default_fill_threads(void)
     return n > 32 ? 32 : n;
 }
 
-/* Slab size when the caller leaves it to the plan: a power of two in [32 KiB, 256 KiB] that gives
- * about `items` block-level items over the load.
- *
- * Aligned copies and conversions: 16 Ki items (256 KiB from 4 GiB on).  The CTAs of a launch take
- * neighbouring slabs, so small slabs keep what the whole GPU reads and writes at a time close together
- * in memory: 545 MB of bf16 took 164 us with 32 KiB, 170 with 64, 174 with 128; 1.9 GB 572, 556, 561
- * and 571 with 256; 16 GB gained nothing below 256 KiB (4722 us with 64, 4692 with 256).
- *
- * Copies off the 16-byte grid: 4 Ki items.  A slab there starts and ends with partial vectors and a
- * realigning loop that fills and drains (876 MB 270 us with 128 KiB, 292 with 32; 300 MB of a
- * tensor-parallel rank 105 with 64, 111 with 32). */
-#define CFA_SLAB_ITEMS 16384u
-/* Conversions to a wider type write twice what they read, and gain from small slabs at every size:
- * bf16 -> fp32 8.8 GB written 2060 us with 32 KiB, 2094 with 64, 2135 with 256. */
-#define CFA_WIDEN_SLAB (32u << 10)
-#define CFA_ODD_SLAB_ITEMS 4096u
-static uint32_t cfa_auto_slab(uint64_t dst_bytes, uint32_t items)
+/* Slab size when the caller leaves it to the plan: about 4096 block-level items over the load
+ * (the persistent grids hold 456-608 CTAs), as a power of two in [32 KiB, 256 KiB].  Loads of a
+ * gigabyte and more get 256 KiB (the size a sweep of 64 KiB - 1 MiB picked on the 8B, 70B,
+ * Mixtral and fp32 checkpoints); a 125 MiB load of 1,000 tensors gets 32 KiB, where 256 KiB left
+ * one slab per CTA and a launch of 0.073 ms instead of 0.054. */
+static uint32_t cfa_auto_slab(uint64_t dst_bytes)
 {
     uint64_t s = 32u << 10;
-    while (s < (256u << 10) && s * 2 * items <= dst_bytes) s *= 2;
+    while (s < (256u << 10) && s * 2 * 4096 <= dst_bytes) s *= 2;
+    return (uint32_t)s;
+}
+
+/* Parts that a launch over the whole load cuts aligned copies and conversions into when the slab
+ * size is the plan's choice: about 16 Ki of them, in [32 KiB, 256 KiB] (256 KiB from 4 GiB on).  The
+ * CTAs of a launch take neighbouring parts, so small ones keep what the whole GPU reads and writes
+ * at a time close together in memory: 545 MB of bf16 took 164 us in 32 KiB, 170 in 64, 174 in 128;
+ * 1.9 GB 572, 556, 561 and 571 in 256; 16 GB gained nothing below 256 KiB (4722 us in 64, 4692 in
+ * 256). */
+static uint32_t cfa_auto_part(uint64_t dst_bytes)
+{
+    uint64_t s = 32u << 10;
+    while (s < (256u << 10) && s * 2 * 16384 <= dst_bytes) s *= 2;
     return (uint32_t)s;
 }
 
@@ -755,16 +757,15 @@ cfa_status cfa_host_plan_build(const cfa_tensor_entry *entries, size_t n_entries
         st = CFA_ERR_NOMEM;
         goto done;
     }
-    const int auto_slab = o.slab_bytes == 0;
-    out->odd_slab_bytes = o.slab_bytes;
-    if (auto_slab) {
+    if (o.slab_bytes == 0) {
         uint64_t dst_total = 0;
         for (size_t i = 0; i < n_entries; ++i) dst_total += info[i].n * (uint64_t)info[i].es_d;
-        o.slab_bytes = cfa_auto_slab(dst_total, CFA_SLAB_ITEMS);
-        out->odd_slab_bytes = cfa_auto_slab(dst_total, CFA_ODD_SLAB_ITEMS);
+        o.slab_bytes = cfa_auto_slab(dst_total);
+        out->part_bytes = cfa_auto_part(dst_total);
     }
     {
         const int use_bulk = CFA_BULK_READY && (o.flags & CFA_OPT_BULK);
+        const uint64_t slab = o.slab_bytes;
         /* pass 1: items in chunk order, tagged with their class */
         for (size_t p = 0; p < n_pieces; ++p) {
             const cfa_piece *pc = &out->pieces[p];
@@ -775,9 +776,6 @@ cfa_status cfa_host_plan_build(const cfa_tensor_entry *entries, size_t n_entries
             const uint32_t cls =
                 pc->conv ? CFA_CLASS_OF_CONV(pc->conv) : (uint32_t)log2_small(in->es_s);
             const uint64_t a0 = (uint64_t)(uintptr_t)dsts[pc->dst_index].dev_ptr + pc->dst_offset;
-            uint64_t slab = pc->conv || ((pc->src_offset | a0) & 15u) == 0 ? o.slab_bytes
-                                                                        : out->odd_slab_bytes;
-            if (auto_slab && pc->conv && in->es_d > in->es_s) slab = CFA_WIDEN_SLAB;
             if (pc->rows > 1) {
                 /* blocks of whole rows, about slab_bytes of destination each */
                 const uint64_t row_d = in->cols * (uint64_t)in->es_d;

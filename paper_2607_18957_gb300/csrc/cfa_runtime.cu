@@ -54,7 +54,8 @@ extern "C" cudaError_t cfa_launch_bulk(const cfa_bulk_range *ranges, uint32_t n_
                                        uint64_t src_base, uint64_t src_period,
                                        uint64_t src_lo, uint64_t src_hi,
                                        unsigned long long *ck, int *status, int grid_cap,
-                                       uint32_t item_bytes, const cfa_launch_ctl *ctl,
+                                       uint32_t item_bytes, uint32_t part_bytes,
+                                       const cfa_launch_ctl *ctl,
                                        cudaStream_t stream);
 extern "C" cudaError_t cfa_bulk_selftest_timeout(int *status_host);
 extern "C" cudaError_t cfa_launch_pull(const void *src, void *dst, uint64_t bytes, int grid,
@@ -335,10 +336,23 @@ cfa_status launch(cfa_plan *p, uint32_t c0, uint32_t c1, uint64_t src_base, uint
     const uint64_t lo = (uint64_t)c0 * hp.chunk_bytes;
     const uint64_t hi = std::min<uint64_t>(hp.blob_bytes, (uint64_t)c1 * hp.chunk_bytes);
     const size_t row = (size_t)hp.n_chunks + 1;
-    /* the plan's slabs suit a launch over the whole load; one over fewer chunks cuts them */
+    /* What the slabs are cut to (cfa_parts_log2): over fewer chunks than all, to the least part; over
+     * the whole load, aligned copies and conversions to the plan's parts (conversions to a wider
+     * type, which write twice what they read, to 32 KiB: 8.8 GB of fp32 from bf16 2060 us so, 2094
+     * with 64 KiB, 2135 with 256), and copies off the 16-byte grid not at all: each part there would
+     * start and end with partial vectors (876 MB 270 us in 128 KiB, 292 in 32). */
     const bool whole = c0 == 0 && c1 == hp.n_chunks;
-    const uint32_t item_bytes = whole ? 0 : hp.opts.slab_bytes;
-    const uint32_t slab_item_bytes = whole ? 0 : std::max(item_bytes, hp.odd_slab_bytes);
+    const uint32_t item_bytes = hp.opts.slab_bytes;
+    const uint32_t bulk_part = whole ? hp.part_bytes : CFA_MIN_PART_BYTES;
+    auto slab_part = [&](int k) -> uint32_t {
+        if (!whole) return CFA_MIN_PART_BYTES;
+        if (k < 4 || !hp.part_bytes) return 0;
+        const bool widens = k == CFA_CLASS_OF_CONV(CFA_CONV_BF16_F32) ||
+                            k == CFA_CLASS_OF_CONV(CFA_CONV_F16_F32);
+        const bool narrows = k == CFA_CLASS_OF_CONV(CFA_CONV_F32_BF16) ||
+                             k == CFA_CLASS_OF_CONV(CFA_CONV_F32_F16);
+        return widens ? CFA_MIN_PART_BYTES : hp.part_bytes << (narrows ? 1 : 0);
+    };
     const int one = tma && whole ? plain_class(hp) : -1;
     const bool timing_on = (hp.opts.flags & CFA_OPT_TIMING) != 0;
     enum { BULK, BULK_AS_VECTOR, ROWS_AS_STRIDED, STRIDED, VECTOR };
@@ -393,13 +407,12 @@ cfa_status launch(cfa_plan *p, uint32_t c0, uint32_t c1, uint64_t src_base, uint
         }
         if (J.type == BULK)
             CK(p, cfa_launch_bulk(ranges, n_ranges, src_base, period, lo, hi, p->d_ck,
-                                  p->d_status, cap(p->bulk_grid_cap), item_bytes, &ctl,
-                                  s));
+                                  p->d_status, cap(p->bulk_grid_cap), item_bytes, bulk_part,
+                                  &ctl, s));
         else if (J.type == BULK_AS_VECTOR) /* bulk items are copy-class slabs of class k */
             CK(p, cfa_launch_unpack(k, p->d_bulk + J.a0, J.a1 - J.a0, p->d_tiny + J.b0,
                                     J.b1 - J.b0, src_base, period, lo, hi, p->d_ck, p->d_status,
-                                    cap(p->grid_cap[k]), item_bytes, CFA_MIN_PART_BYTES, tma,
-                                    &ctl, s));
+                                    cap(p->grid_cap[k]), item_bytes, bulk_part, tma, &ctl, s));
         else if (J.type == STRIDED || J.type == ROWS_AS_STRIDED)
             CK(p, cfa_launch_strided(k,
                                      (J.type == STRIDED ? p->d_strided : p->d_brows) + J.a0,
@@ -408,8 +421,7 @@ cfa_status launch(cfa_plan *p, uint32_t c0, uint32_t c1, uint64_t src_base, uint
         else
             CK(p, cfa_launch_unpack(k, p->d_slabs + J.a0, J.a1 - J.a0, p->d_tiny + J.b0,
                                     J.b1 - J.b0, src_base, period, lo, hi, p->d_ck, p->d_status,
-                                    cap(p->grid_cap[k]), slab_item_bytes, CFA_MIN_PART_BYTES, tma,
-                                    &ctl, s));
+                                    cap(p->grid_cap[k]), item_bytes, slab_part(k), tma, &ctl, s));
         p->ck_clear = nullptr; /* this launch clears it */
         p->ck_clear_words = 0;
         if (timing) CK(p, cudaEventRecord(p->t_k1[p->last_launches], s));

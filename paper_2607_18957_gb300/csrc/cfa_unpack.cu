@@ -1397,9 +1397,9 @@ extern "C" cudaError_t cfa_launch_unpack(int cls, const cfa_work *slabs, uint32_
     /* the fp32 -> 16-bit classes read twice what they write */
     const bool narrows = cls == CFA_CLASS_OF_CONV(CFA_CONV_F32_BF16) ||
                          cls == CFA_CLASS_OF_CONV(CFA_CONV_F32_F16);
-    const uint32_t parts_log2 = cfa_parts_log2(n_slabs, (uint32_t)grid_cap,
-                                               (uint64_t)item_bytes << (narrows ? 1 : 0),
-                                               part_bytes);
+    const uint32_t parts_log2 =
+        n_slabs ? cfa_parts_log2((uint64_t)item_bytes << (narrows ? 1 : 0), part_bytes) : 0;
+    if (((uint64_t)n_slabs << parts_log2) >= (1ull << 31)) return cudaErrorInvalidValue;
     const uint64_t items =
         ((uint64_t)n_slabs << parts_log2) + (n_tiny + kTinyPerGroup - 1) / kTinyPerGroup;
     if (items == 0) return cudaSuccess;
