@@ -488,13 +488,13 @@ extern "C" int cfa_bulk_blocks_per_sm(void)
 }
 
 /* Launches the bulk unpack over up to CFA_BULK_RANGES lists of items whose source, destination and
- * byte length are multiples of 16; grid_cap bounds the persistent grid. */
+ * byte length are multiples of 16, cut into parts as `cut` says; grid_cap bounds the persistent
+ * grid. */
 extern "C" cudaError_t cfa_launch_bulk(const cfa_bulk_range *ranges, uint32_t n_ranges,
                                        uint64_t src_base, uint64_t src_period,
                                        uint64_t src_lo, uint64_t src_hi,
                                        unsigned long long *ck, int *status, int grid_cap,
-                                       uint32_t item_bytes, uint32_t part_bytes,
-                                       const cfa_launch_ctl *ctl,
+                                       const cfa_cut *cut, const cfa_launch_ctl *ctl,
                                        cudaStream_t stream)
 {
     if (n_ranges > CFA_BULK_RANGES || grid_cap <= 0) return cudaErrorInvalidValue;
@@ -508,9 +508,8 @@ extern "C" cudaError_t cfa_launch_bulk(const cfa_bulk_range *ranges, uint32_t n_
         n_items += ranges[r].n;
     }
     if (n_items == 0) return cudaSuccess;
-    if (n_items >= (1ull << 31)) return cudaErrorInvalidValue;
-    a.parts_log2 = cfa_parts_log2(item_bytes, part_bytes);
-    if ((n_items << a.parts_log2) >= (1ull << 31)) return cudaErrorInvalidValue;
+    if (n_items >= CFA_MOST_VISITS) return cudaErrorInvalidValue;
+    a.parts_log2 = cfa_parts_log2(cut, n_items, (uint32_t)grid_cap);
     a.n_items = (uint32_t)n_items << a.parts_log2;
     a.spin_limit = kSpinLimit;
     a.src_base = src_base;

@@ -99,6 +99,13 @@ typedef struct cfa_copy {
     ((uint32_t)(src_log2) | ((uint32_t)(dst_log2) << 2) | ((uint32_t)(conv) << 4))
 #define CFA_MODE_CONV(mode) (((mode) >> 4) & 15u)
 
+/* Whether a work class reads twice what it writes. */
+static inline int cfa_class_narrows(int cls)
+{
+    return cls == CFA_CLASS_OF_CONV(CFA_CONV_F32_BF16) ||
+           cls == CFA_CLASS_OF_CONV(CFA_CONV_F32_F16);
+}
+
 /* Conversion for a (source, destination) dtype pair, 0 if the pair has none. */
 static inline int cfa_conversion(int32_t src, int32_t dst)
 {
@@ -125,13 +132,15 @@ typedef struct cfa_host_plan {
     size_t n_pieces;
     /* work items ordered by (class, chunk): class k of chunk c owns
      * [first[k * (n_chunks + 1) + c], first[k * (n_chunks + 1) + c + 1]) of each array, so the
-     * items of one class over a run of chunks are contiguous */
+     * items of one class over a run of chunks are contiguous; the `units` beside slabs, bulk and
+     * brows count the bytes before each of those bounds (source or destination bytes, whichever
+     * is more) in whole CFA_MIN_PART_BYTES */
     cfa_work *slabs; /* block-level, LSU vector path */
     size_t n_slabs;
-    uint32_t *slab_first;
+    uint32_t *slab_first, *slab_units;
     cfa_work *bulk;  /* block-level, TMA bulk path (cast-free, 16-byte aligned) */
     size_t n_bulk;
-    uint32_t *bulk_first;
+    uint32_t *bulk_first, *bulk_units;
     cfa_work *tiny;  /* warp-level */
     size_t n_tiny;
     uint32_t *tiny_first;
@@ -140,7 +149,7 @@ typedef struct cfa_host_plan {
     uint32_t *strided_first;
     cfa_swork *brows; /* the same for the TMA path (cast-free, 16-byte aligned) */
     size_t n_brows;
-    uint32_t *brows_first;
+    uint32_t *brows_first, *brows_units;
     int64_t *layer_last_chunk; /* n_layers; -1 = the group has no bytes */
     cfa_copy *copies;          /* what each chunk's pieces read: chunk c owns
                                   [copy_first[c], copy_first[c + 1]) */
@@ -155,20 +164,41 @@ typedef struct cfa_host_plan {
 /*
  * Block-level items are cut once more at launch: into 2^cfa_parts_log2 equal parts each, cut where
  * the destination is a multiple of CFA_PART_ALIGN, so that the parts of an item of the caller's usual
- * size, item_bytes, hold part_bytes or more (source or destination bytes, whichever is more; a
+ * size, cut->item_bytes, hold part_bytes or more (source or destination bytes, whichever is more; a
  * smaller item has fewer parts, none below CFA_MIN_PART_BYTES).  The plan's slabs, and the no-alloc
  * entry point's 2 MiB items, are few and large for the sake of their descriptors; a launch over one
  * chunk or a small checkpoint would leave most CTAs without work, and large items spread the
  * addresses in flight over too much memory (cfa_auto_part).  A chunk's items go down to 32 KiB.
  * The no-alloc items stop at 64 KiB: fp32 -> bf16, 252 MB, 118 us so, 125 with 32 KiB parts; 945 MB
  * 417 and 429; bf16, 1.1 GB, 673 with 64 KiB, 680 with 128, 686 with 512.
+ *
+ * The kernels visit 2^k parts of every item, and the surplus parts of an item smaller than
+ * item_bytes are empty: each costs a CTA a descriptor fetch and the checks.  So k also depends on
+ * what the launch holds, n_items items of cut->bytes in all: visits beyond one per CTA of a full
+ * grid stay within 3/2 of the parts that the bytes would fill.  Full items are cut as their size
+ * says; items below the part size on average are not cut.  With k from item_bytes alone 16,000
+ * tensors of 8 to 64 KiB took 1149 us through the no-alloc entry point (k = 5), 416 at k = 0, and
+ * as many of 8 to 32 KiB, in chunks of a plan with 64 MiB slabs (k = 11), 37 ms and 0.13.
  */
 #define CFA_MIN_PART_BYTES 32768u
 #define CFA_PART_ALIGN 128u
-static inline uint32_t cfa_parts_log2(uint64_t item_bytes, uint32_t part_bytes)
+#define CFA_MOST_VISITS (1ull << 31) /* the kernels count visits in 32 bits */
+typedef struct cfa_cut {
+    uint64_t item_bytes; /* of the caller's usual item */
+    uint64_t bytes;      /* of all block-level items of the launch */
+    uint32_t part_bytes; /* 0: whole items */
+} cfa_cut;
+
+static inline uint32_t cfa_parts_log2(const cfa_cut *cut, uint64_t n_items, uint32_t grid)
 {
+    const uint64_t part_bytes = cut->part_bytes;
+    if (part_bytes == 0) return 0;
+    const uint64_t filled = cut->bytes / part_bytes;
+    uint64_t most = filled + filled / 2;
     uint32_t k = 0;
-    while (part_bytes && (item_bytes >> (k + 1)) >= part_bytes) ++k;
+    if (most < grid) most = grid;
+    if (most >= CFA_MOST_VISITS) most = CFA_MOST_VISITS - 1;
+    while ((cut->item_bytes >> (k + 1)) >= part_bytes && (n_items << (k + 1)) <= most) ++k;
     return k;
 }
 

@@ -42,8 +42,8 @@ extern "C" cudaError_t cfa_launch_unpack(int cls, const cfa_work *slabs, uint32_
                                          uint64_t src_base, uint64_t src_period,
                                          uint64_t src_lo, uint64_t src_hi,
                                          unsigned long long *ck, int *status, int grid_cap,
-                                         uint32_t item_bytes, uint32_t part_bytes,
-                                         int dev_src, const cfa_launch_ctl *ctl,
+                                         const cfa_cut *cut, int dev_src,
+                                         const cfa_launch_ctl *ctl,
                                          cudaStream_t stream);
 
 namespace {
@@ -313,6 +313,7 @@ extern "C" cfa_status cfa_unpack_noalloc(const cfa_tensor_entry *entries, size_t
 
     /* validate every entry and count the work items, per class, without storing anything */
     uint32_t count[CFA_N_CLASSES][kKinds] = {};
+    uint64_t slab_bytes[CFA_N_CLASSES] = {}; /* of all slabs: source or destination, the wider */
     for (size_t i = 0; i < n_entries; ++i) {
         uint64_t n, off;
         int es_s, es_d, conv;
@@ -335,6 +336,7 @@ extern "C" cfa_status cfa_unpack_noalloc(const cfa_tensor_entry *entries, size_t
             return CFA_ERR_INVAL;
         }
         count[cls][nb < kTinyBytes ? TINY : SLAB] += (uint32_t)items;
+        if (nb >= kTinyBytes) slab_bytes[cls] += n * (uint64_t)(es_s > es_d ? es_s : es_d);
     }
 
     /* lay the items out as [class 0 slabs][class 0 tiny][class 1 slabs] ... */
@@ -402,11 +404,11 @@ extern "C" cfa_status cfa_unpack_noalloc(const cfa_tensor_entry *entries, size_t
     ctl.flags = CFA_LAUNCH_EARLY | CFA_LAUNCH_WAIT_FIRST | CFA_LAUNCH_RELEASE;
     for (int k = 0; e == cudaSuccess && k < CFA_N_CLASSES; ++k) {
         if (!count[k][SLAB] && !count[k][TINY]) continue;
+        const cfa_cut cut = {kSlabBytes << (cfa_class_narrows(k) ? 1 : 0), slab_bytes[k],
+                             kPartBytes};
         e = cfa_launch_unpack(k, scratch->items + base[k][SLAB], count[k][SLAB],
                               scratch->items + base[k][TINY], count[k][TINY], src, 0, 0,
-                              blob_bytes, ck, status, g_grid_cap[dev][k], (uint32_t)kSlabBytes,
-                              kPartBytes, 1,
-                              &ctl, stream);
+                              blob_bytes, ck, status, g_grid_cap[dev][k], &cut, 1, &ctl, stream);
         ctl.flags = CFA_LAUNCH_EARLY | CFA_LAUNCH_WAIT_LAST | CFA_LAUNCH_RELEASE;
     }
     if (e != cudaSuccess) {

@@ -326,6 +326,36 @@ static cfa_status partition_by_class(vec *v, uint32_t *first, uint32_t n_chunks,
     return CFA_OK;
 }
 
+/* Bytes of an item, of its source or its destination, whichever are more. */
+static uint64_t item_bytes(const vec *v, size_t q)
+{
+    uint64_t n;
+    uint32_t mode;
+    if (v->elem == sizeof(cfa_swork)) {
+        const cfa_swork *w = (const cfa_swork *)v->p + q;
+        n = (uint64_t)w->rows * w->cols;
+        mode = w->mode;
+    } else {
+        const cfa_work *w = (const cfa_work *)v->p + q;
+        n = w->n;
+        mode = w->mode;
+    }
+    const uint32_t s = mode & 3u, d = (mode >> 2) & 3u;
+    return n << (s > d ? s : d);
+}
+
+/* For items in the order of partition_by_class: units[i] is the bytes of the items before
+ * first[i] in whole CFA_MIN_PART_BYTES. */
+static void count_units(const vec *v, const uint32_t *first, size_t nf, uint32_t *units)
+{
+    uint64_t bytes = 0;
+    size_t q = 0;
+    for (size_t i = 0; i < nf; ++i) {
+        for (; q < first[i]; ++q) bytes += item_bytes(v, q);
+        units[i] = (uint32_t)(bytes / CFA_MIN_PART_BYTES);
+    }
+}
+
 /* Within each (class, chunk) range of tiny items, the pieces of at most CFA_TINY_SEG_BYTES
  * destination bytes first (stable), so the kernel's warps mostly get pieces of one kind. */
 static cfa_status order_tiny(vec *v, const uint32_t *first, uint32_t n_chunks)
@@ -363,14 +393,17 @@ void cfa_host_plan_free(cfa_host_plan *hp)
     free(hp->pieces);
     free(hp->slabs);
     free(hp->slab_first);
+    free(hp->slab_units);
     free(hp->bulk);
     free(hp->bulk_first);
+    free(hp->bulk_units);
     free(hp->tiny);
     free(hp->tiny_first);
     free(hp->strided);
     free(hp->strided_first);
     free(hp->brows);
     free(hp->brows_first);
+    free(hp->brows_units);
     free(hp->copies);
     free(hp->copy_first);
     free(hp->layer_last_chunk);
@@ -752,8 +785,11 @@ cfa_status cfa_host_plan_build(const cfa_tensor_entry *entries, size_t n_entries
     out->tiny_first = (uint32_t *)calloc(nf, sizeof(uint32_t));
     out->strided_first = (uint32_t *)calloc(nf, sizeof(uint32_t));
     out->brows_first = (uint32_t *)calloc(nf, sizeof(uint32_t));
+    out->slab_units = (uint32_t *)calloc(nf, sizeof(uint32_t));
+    out->bulk_units = (uint32_t *)calloc(nf, sizeof(uint32_t));
+    out->brows_units = (uint32_t *)calloc(nf, sizeof(uint32_t));
     if (!out->slab_first || !out->bulk_first || !out->tiny_first || !out->strided_first ||
-        !out->brows_first) {
+        !out->brows_first || !out->slab_units || !out->bulk_units || !out->brows_units) {
         st = CFA_ERR_NOMEM;
         goto done;
     }
@@ -855,6 +891,9 @@ cfa_status cfa_host_plan_build(const cfa_tensor_entry *entries, size_t n_entries
             goto done;
         if ((st = partition_by_class(&brows, out->brows_first, n_chunks, S, err, errlen)))
             goto done;
+        count_units(&slabs, out->slab_first, nf, out->slab_units);
+        count_units(&bulk, out->bulk_first, nf, out->bulk_units);
+        count_units(&brows, out->brows_first, nf, out->brows_units);
     }
 
     /* 4b. what each chunk's pieces read: contiguous ranges merged across gaps of at most

@@ -54,8 +54,7 @@ extern "C" cudaError_t cfa_launch_bulk(const cfa_bulk_range *ranges, uint32_t n_
                                        uint64_t src_base, uint64_t src_period,
                                        uint64_t src_lo, uint64_t src_hi,
                                        unsigned long long *ck, int *status, int grid_cap,
-                                       uint32_t item_bytes, uint32_t part_bytes,
-                                       const cfa_launch_ctl *ctl,
+                                       const cfa_cut *cut, const cfa_launch_ctl *ctl,
                                        cudaStream_t stream);
 extern "C" cudaError_t cfa_bulk_selftest_timeout(int *status_host);
 extern "C" cudaError_t cfa_launch_pull(const void *src, void *dst, uint64_t bytes, int grid,
@@ -65,8 +64,8 @@ extern "C" cudaError_t cfa_launch_unpack(int cls, const cfa_work *slabs, uint32_
                                          uint64_t src_base, uint64_t src_period,
                                          uint64_t src_lo, uint64_t src_hi,
                                          unsigned long long *ck, int *status, int grid_cap,
-                                         uint32_t item_bytes, uint32_t part_bytes,
-                                         int dev_src, const cfa_launch_ctl *ctl,
+                                         const cfa_cut *cut, int dev_src,
+                                         const cfa_launch_ctl *ctl,
                                          cudaStream_t stream);
 
 namespace {
@@ -342,17 +341,18 @@ cfa_status launch(cfa_plan *p, uint32_t c0, uint32_t c1, uint64_t src_base, uint
      * with 64 KiB, 2135 with 256), and copies off the 16-byte grid not at all: each part there would
      * start and end with partial vectors (876 MB 270 us in 128 KiB, 292 in 32). */
     const bool whole = c0 == 0 && c1 == hp.n_chunks;
-    const uint32_t item_bytes = hp.opts.slab_bytes;
     const uint32_t bulk_part = whole ? hp.part_bytes : CFA_MIN_PART_BYTES;
     auto slab_part = [&](int k) -> uint32_t {
         if (!whole) return CFA_MIN_PART_BYTES;
         if (k < 4 || !hp.part_bytes) return 0;
         const bool widens = k == CFA_CLASS_OF_CONV(CFA_CONV_BF16_F32) ||
                             k == CFA_CLASS_OF_CONV(CFA_CONV_F16_F32);
-        const bool narrows = k == CFA_CLASS_OF_CONV(CFA_CONV_F32_BF16) ||
-                             k == CFA_CLASS_OF_CONV(CFA_CONV_F32_F16);
-        return widens ? CFA_MIN_PART_BYTES : hp.part_bytes << (narrows ? 1 : 0);
+        return widens ? CFA_MIN_PART_BYTES : hp.part_bytes << (cfa_class_narrows(k) ? 1 : 0);
     };
+    auto bytes_of = [&](const uint32_t *units, int k) { /* of class k's items in these chunks */
+        return (uint64_t)(units[k * row + c1] - units[k * row + c0]) * CFA_MIN_PART_BYTES;
+    };
+    cfa_cut bulk_cut = {hp.opts.slab_bytes, 0, bulk_part};
     const int one = tma && whole ? plain_class(hp) : -1;
     const bool timing_on = (hp.opts.flags & CFA_OPT_TIMING) != 0;
     enum { BULK, BULK_AS_VECTOR, ROWS_AS_STRIDED, STRIDED, VECTOR };
@@ -370,11 +370,17 @@ cfa_status launch(cfa_plan *p, uint32_t c0, uint32_t c1, uint64_t src_base, uint
         if (b1 != b0 && (what & LAUNCH_CONTIG)) {
             if (k == one) jobs[n++] = Job{BULK_AS_VECTOR, k, b0, b1, 0, (uint32_t)hp.n_tiny};
             else if (!tma) jobs[n++] = Job{BULK_AS_VECTOR, k, b0, b1, 0, 0};
-            else ranges[n_ranges++] = cfa_bulk_range{p->d_bulk + b0, b1 - b0, 0};
+            else {
+                ranges[n_ranges++] = cfa_bulk_range{p->d_bulk + b0, b1 - b0, 0};
+                bulk_cut.bytes += bytes_of(hp.bulk_units, k);
+            }
         }
         if (r1 != r0 && (what & LAUNCH_STRIDED)) {
             if (!tma) jobs[n++] = Job{ROWS_AS_STRIDED, k, r0, r1, 0, 0};
-            else ranges[n_ranges++] = cfa_bulk_range{p->d_brows + r0, r1 - r0, 1};
+            else {
+                ranges[n_ranges++] = cfa_bulk_range{p->d_brows + r0, r1 - r0, 1};
+                bulk_cut.bytes += bytes_of(hp.brows_units, k);
+            }
         }
     }
     if (n_ranges) jobs[n++] = Job{BULK, 0, 0, 0, 0, 0};
@@ -407,21 +413,24 @@ cfa_status launch(cfa_plan *p, uint32_t c0, uint32_t c1, uint64_t src_base, uint
         }
         if (J.type == BULK)
             CK(p, cfa_launch_bulk(ranges, n_ranges, src_base, period, lo, hi, p->d_ck,
-                                  p->d_status, cap(p->bulk_grid_cap), item_bytes, bulk_part,
-                                  &ctl, s));
-        else if (J.type == BULK_AS_VECTOR) /* bulk items are copy-class slabs of class k */
+                                  p->d_status, cap(p->bulk_grid_cap), &bulk_cut, &ctl, s));
+        else if (J.type == BULK_AS_VECTOR) { /* bulk items are copy-class slabs of class k */
+            const cfa_cut cut = {hp.opts.slab_bytes, bytes_of(hp.bulk_units, k), bulk_part};
             CK(p, cfa_launch_unpack(k, p->d_bulk + J.a0, J.a1 - J.a0, p->d_tiny + J.b0,
                                     J.b1 - J.b0, src_base, period, lo, hi, p->d_ck, p->d_status,
-                                    cap(p->grid_cap[k]), item_bytes, bulk_part, tma, &ctl, s));
-        else if (J.type == STRIDED || J.type == ROWS_AS_STRIDED)
+                                    cap(p->grid_cap[k]), &cut, tma, &ctl, s));
+        } else if (J.type == STRIDED || J.type == ROWS_AS_STRIDED)
             CK(p, cfa_launch_strided(k,
                                      (J.type == STRIDED ? p->d_strided : p->d_brows) + J.a0,
                                      J.a1 - J.a0, src_base, period, lo, hi, p->d_ck, p->d_status,
                                      cap(p->strided_grid_cap[k]), &ctl, s));
-        else
+        else {
+            const cfa_cut cut = {(uint64_t)hp.opts.slab_bytes << (cfa_class_narrows(k) ? 1 : 0),
+                                 bytes_of(hp.slab_units, k), slab_part(k)};
             CK(p, cfa_launch_unpack(k, p->d_slabs + J.a0, J.a1 - J.a0, p->d_tiny + J.b0,
                                     J.b1 - J.b0, src_base, period, lo, hi, p->d_ck, p->d_status,
-                                    cap(p->grid_cap[k]), item_bytes, slab_part(k), tma, &ctl, s));
+                                    cap(p->grid_cap[k]), &cut, tma, &ctl, s));
+        }
         p->ck_clear = nullptr; /* this launch clears it */
         p->ck_clear_words = 0;
         if (timing) CK(p, cudaEventRecord(p->t_k1[p->last_launches], s));

@@ -1382,6 +1382,7 @@ extern "C" int cfa_unpack_blocks_per_sm(int cls)
 }
 
 /* Launches the class-cls unpack over the given work items; grid_cap bounds the persistent grid.
+ * `cut` (needed for slabs only) says what the slabs are cut into.
  * Blob byte o is read at src_base + o, or at src_base + (o mod src_period) for a periodic
  * source (a work item never straddles a period: periods are whole chunks). */
 extern "C" cudaError_t cfa_launch_unpack(int cls, const cfa_work *slabs, uint32_t n_slabs,
@@ -1389,17 +1390,13 @@ extern "C" cudaError_t cfa_launch_unpack(int cls, const cfa_work *slabs, uint32_
                                          uint64_t src_base, uint64_t src_period,
                                          uint64_t src_lo, uint64_t src_hi,
                                          unsigned long long *ck, int *status, int grid_cap,
-                                         uint32_t item_bytes, uint32_t part_bytes,
-                                         int dev_src, const cfa_launch_ctl *ctl,
+                                         const cfa_cut *cut, int dev_src,
+                                         const cfa_launch_ctl *ctl,
                                          cudaStream_t stream)
 {
     if (cls < 0 || cls >= CFA_N_CLASSES || grid_cap <= 0) return cudaErrorInvalidValue;
-    /* the fp32 -> 16-bit classes read twice what they write */
-    const bool narrows = cls == CFA_CLASS_OF_CONV(CFA_CONV_F32_BF16) ||
-                         cls == CFA_CLASS_OF_CONV(CFA_CONV_F32_F16);
-    const uint32_t parts_log2 =
-        n_slabs ? cfa_parts_log2((uint64_t)item_bytes << (narrows ? 1 : 0), part_bytes) : 0;
-    if (((uint64_t)n_slabs << parts_log2) >= (1ull << 31)) return cudaErrorInvalidValue;
+    const uint32_t parts_log2 = n_slabs ? cfa_parts_log2(cut, n_slabs, (uint32_t)grid_cap) : 0;
+    if (n_slabs >= CFA_MOST_VISITS) return cudaErrorInvalidValue;
     const uint64_t items =
         ((uint64_t)n_slabs << parts_log2) + (n_tiny + kTinyPerGroup - 1) / kTinyPerGroup;
     if (items == 0) return cudaSuccess;

@@ -95,6 +95,25 @@ def chunk_plan(c, chunk):
     return cfa.Plan(c.entries, c.dsts, c.blob_bytes, chunk_bytes=chunk, dev_slots=0, host_slots=0)
 
 
+def test_a_chunk_of_very_many_small_items_under_large_slabs():
+    """2^20 block-level items in one chunk launch of a plan whose slabs are 64 MiB: the cut into
+    parts gives way, the call is not refused."""
+    n, es = 1 << 20, 2
+    per = 64 // es
+    entries = cfa.make_entries(dtype=["bf16"] * (n + 1),
+                               shape=[(per,)] * (n + 1), offset=np.arange(n + 1) * 64,
+                               dst=np.zeros(n + 1, np.int64), row=np.arange(n + 1) * per)
+    blob = torch.randint(0, 256, ((n + 1) * 64,), dtype=torch.uint8, device="cuda")
+    out = torch.zeros_like(blob)
+    with cfa.Plan(entries, [(out.data_ptr(), "bf16", ((n + 1) * per,))], blob.numel(),
+                  chunk_bytes=n * 64, slab_bytes=64 << 20, tiny_bytes=0, dev_slots=0,
+                  host_slots=0) as plan:
+        assert plan.stats()["n_bulk"] == n + 1
+        for k in range(2):
+            plan.unpack_chunks_async(k, k + 1, blob.data_ptr() + k * n * 64)
+        assert torch.equal(out, blob)
+
+
 def unpack_through_one_slot(c, plan, chunk, slot):
     for k in range(plan.info()["n_chunks"]):
         part = c.blob[k * chunk:(k + 1) * chunk]

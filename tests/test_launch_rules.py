@@ -1,0 +1,60 @@
+"""The rules that launches follow, on the host: the inline functions of cfa_internal.h compiled on
+their own."""
+import ctypes
+import os
+import subprocess
+
+import pytest
+
+ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+
+CODE = r"""
+#include "cfa_internal.h"
+uint32_t parts_log2(uint64_t item_bytes, uint64_t bytes, uint32_t part_bytes, uint64_t n_items,
+                    uint32_t grid)
+{
+    const cfa_cut cut = {item_bytes, bytes, part_bytes};
+    return cfa_parts_log2(&cut, n_items, grid);
+}
+"""
+
+KIB, MIB = 1 << 10, 1 << 20
+GRID = 456
+
+
+@pytest.fixture(scope="module")
+def rules(tmp_path_factory):
+    d = tmp_path_factory.mktemp("rules")
+    (d / "rules.c").write_text(CODE)
+    subprocess.run(["gcc", "-O1", "-std=c11", "-Wall", "-Werror", "-shared", "-fPIC",
+                    "-I", os.path.join(ROOT, "include"),
+                    "-I", os.path.join(ROOT, "paper_2607_18957_gb300", "csrc"),
+                    str(d / "rules.c"), "-o", str(d / "rules.so")], check=True)
+    lib = ctypes.CDLL(str(d / "rules.so"))
+    lib.parts_log2.argtypes = [ctypes.c_uint64, ctypes.c_uint64, ctypes.c_uint32,
+                               ctypes.c_uint64, ctypes.c_uint32]
+    lib.parts_log2.restype = ctypes.c_uint32
+    return lib
+
+
+@pytest.mark.parametrize("item,part", [(256 * KIB, 32 * KIB), (2 * MIB, 64 * KIB),
+                                       (64 * MIB, 32 * KIB), (32 * KIB, 32 * KIB)])
+@pytest.mark.parametrize("n", [1, 7, 256, 4096, 100_000])
+def test_full_items_are_cut_to_the_part_size(rules, item, part, n):
+    assert item >> rules.parts_log2(item, n * item, part, n, GRID) == part
+
+
+@pytest.mark.parametrize("item,part", [(256 * KIB, 32 * KIB), (2 * MIB, 64 * KIB),
+                                       (4 * MIB, 64 * KIB), (64 * MIB, 32 * KIB)])
+@pytest.mark.parametrize("n", [1, 300, 457, 16_000, 1 << 20, 1 << 24, (1 << 31) - 1])
+@pytest.mark.parametrize("mean", [16, 8 * KIB, 24 * KIB, 33 * KIB, 100 * KIB, 3 * MIB])
+def test_visits_stay_near_the_parts_that_hold_bytes(rules, item, part, n, mean):
+    """Items of any size are visited at most once, or once per CTA, or half as often again as there
+    are parts with bytes in them; and never 2^31 times or more."""
+    visits = n << rules.parts_log2(item, n * mean, part, n, GRID)
+    assert visits < 1 << 31
+    assert visits <= max(n, GRID, n * mean // part * 3 // 2)
+
+
+def test_no_cut_without_a_part_size(rules):
+    assert rules.parts_log2(64 * MIB, 1 << 40, 0, 1 << 14, GRID) == 0
