@@ -65,10 +65,9 @@ __device__ __forceinline__ void launch_end(const cfa_launch_ctl &c)
         asm volatile("griddepcontrol.wait;" ::: "memory");
 }
 
-/* Host side: launches fn(args) as the ctl in its arguments says. */
-template <typename Args>
-inline cudaError_t launch_ctl(void (*fn)(const Args), unsigned grid, unsigned threads, size_t smem,
-                              cudaStream_t stream, const Args &args)
+/* Host side: launches kernel fn as ctl says; args are the addresses of its parameters. */
+inline cudaError_t launch_ctl(const void *fn, unsigned grid, unsigned threads, size_t smem,
+                              cudaStream_t stream, const cfa_launch_ctl &ctl, void **args)
 {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(grid);
@@ -76,13 +75,23 @@ inline cudaError_t launch_ctl(void (*fn)(const Args), unsigned grid, unsigned th
     cfg.dynamicSmemBytes = smem;
     cfg.stream = stream;
     cudaLaunchAttribute attr = {};
-    if (args.ctl.flags & CFA_LAUNCH_EARLY) {
+    if (ctl.flags & CFA_LAUNCH_EARLY) {
         attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
         attr.val.programmaticStreamSerializationAllowed = 1;
         cfg.attrs = &attr;
         cfg.numAttrs = 1;
     }
-    return cudaLaunchKernelEx(&cfg, fn, args);
+    return cudaLaunchKernelExC(&cfg, fn, args);
+}
+
+/* The same for a kernel whose one parameter holds its ctl. */
+template <typename Args>
+inline cudaError_t launch_ctl(void (*fn)(const Args), unsigned grid, unsigned threads, size_t smem,
+                              cudaStream_t stream, const Args &args)
+{
+    void *p[] = {const_cast<Args *>(&args)};
+    return launch_ctl(reinterpret_cast<const void *>(fn), grid, threads, smem, stream, args.ctl,
+                      p);
 }
 
 /* Sum over the 32 lanes of a warp; lane 0 holds the total. */

@@ -30,7 +30,6 @@
 
 #include <cstdarg>
 #include <cstdio>
-#include <cstring>
 #include <mutex>
 
 #include "cfa_device.cuh"
@@ -60,79 +59,81 @@ struct NoallocScratch {
 };
 static __device__ __align__(256) NoallocScratch g_noalloc_scratch;
 
-/* Host twin of the descriptors, filled before each upload (guarded by g_mutex). */
-static cfa_work g_host_items[CFA_NOALLOC_MAX_ITEMS];
-
-/* Descriptors that one launch of the upload carries in its parameters (at most 32,764 bytes), and
- * what the call's first launch clears: the unpack's status word and checksums. */
-template <int CAP> struct PutArgs {
-    cfa_work *to;
-    uint32_t n;
-    cfa_launch_ctl ctl;
-    int *status;
-    __align__(16) cfa_work items[CAP];
-};
+/* Descriptors that one launch of the upload carries in its parameters (32,764 bytes at most in
+ * all), and the rest of them: where they go, and what the call's first launch clears (the
+ * unpack's status word and checksums). */
 constexpr int kPutSmall = 112; /* under 4 KiB of parameters: the cheaper launch */
 constexpr int kPutLarge = 1000;
 constexpr int kPutThreads = 256;
+template <int CAP> struct PutItems {
+    __align__(16) cfa_work items[CAP];
+};
+struct PutArgs {
+    cfa_work *to;
+    int *status;
+    cfa_launch_ctl ctl;
+    uint32_t n;
+};
 
-/* Bound by its launch: 64 KiB at most, written once; one thread per 16 bytes of descriptor. */
+/* Host twin of the descriptors, filled before each upload (guarded by g_mutex).  A launch's
+ * parameters are read straight from it, PutItems and all, so there is room for one behind the
+ * last item.  (With the items copied into a struct of all parameters first the host took 35 us
+ * for 1,000 tensors of 8 to 64 KiB and 412 for 16,000; now 26 and 308.  A copy from pageable
+ * memory, which makes the host wait for the stream, took 33 and 294.) */
+static __align__(16) cfa_work g_host_items[CFA_NOALLOC_MAX_ITEMS + kPutLarge];
+
+/* Bound by its launch: 32 KB at most, written once; one thread per 16 bytes of descriptor. */
 template <int CAP>
 __global__ void __launch_bounds__(kPutThreads)
-    cfa_put_kernel(const __grid_constant__ PutArgs<CAP> a)
+    cfa_put_kernel(const PutArgs a, const __grid_constant__ PutItems<CAP> p)
 {
     /* what follows waits for this kernel's end before it reads anything */
     cfa_dev::launch_begin(a.ctl);
     const uint32_t i = blockIdx.x * kPutThreads + threadIdx.x;
     if (i == 0 && a.status) *a.status = 0;
-    const uint4 *from = reinterpret_cast<const uint4 *>(a.items);
+    const uint4 *from = reinterpret_cast<const uint4 *>(p.items);
     if (i < 2u * a.n) reinterpret_cast<uint4 *>(a.to)[i] = from[i];
+    cfa_dev::launch_end(a.ctl);
 }
-
-/* The launch's parameters, filled under g_mutex; the launch copies them. */
-static PutArgs<kPutSmall> g_put_small;
-static PutArgs<kPutLarge> g_put_large;
 
 std::mutex g_mutex;
 NoallocScratch *g_scratch_dev[kMaxDevices];
 int g_grid_cap[kMaxDevices][CFA_N_CLASSES];
 
-template <int CAP>
-cudaError_t put(PutArgs<CAP> &a, cfa_work *to, const cfa_work *from, uint32_t n, int *status,
-                const cfa_launch_ctl &ctl, cudaStream_t stream)
+template <int CAP> cudaError_t put(PutArgs &a, cfa_work *from, cudaStream_t stream)
 {
-    a.to = to;
-    a.n = n;
-    a.status = status;
-    a.ctl = ctl;
-    if (n) std::memcpy(a.items, from, (size_t)n * sizeof(cfa_work));
     /* enough CTAs for the items, and one per 16 Ki checksums to clear */
-    uint64_t grid = (2ull * n + kPutThreads - 1) / kPutThreads;
-    const uint64_t clear = ctl.clear_words >> 14;
+    uint64_t grid = (2ull * a.n + kPutThreads - 1) / kPutThreads;
+    const uint64_t clear = a.ctl.clear_words >> 14;
     if (grid < clear) grid = clear < 152 ? clear : 152;
     if (grid == 0) grid = 1;
-    return cfa_dev::launch_ctl(cfa_put_kernel<CAP>, (unsigned)grid, kPutThreads, 0, stream, a);
+    void *args[] = {&a, from};
+    return cfa_dev::launch_ctl(reinterpret_cast<const void *>(cfa_put_kernel<CAP>),
+                               (unsigned)grid, kPutThreads, 0, stream, a.ctl, args);
 }
 
-/* Uploads n descriptors to `to` in stream order; the first launch clears the status word and the
- * checksums. */
-cudaError_t put_items(cfa_work *to, const cfa_work *from, uint32_t n, int *status,
-                      unsigned long long *clear, uint64_t clear_words, cudaStream_t stream)
+/* Uploads the first n of g_host_items to `to` in stream order; the first launch clears the status
+ * word and the checksums.  The launches write disjoint bytes: each starts once the one before it
+ * runs and ends after it. */
+cudaError_t put_items(cfa_work *to, uint32_t n, int *status, unsigned long long *clear,
+                      uint64_t clear_words, cudaStream_t stream)
 {
-    cfa_launch_ctl ctl{};
-    ctl.clear = clear;
-    ctl.clear_words = clear_words;
+    PutArgs a{};
+    a.status = status;
+    a.ctl.clear = clear;
+    a.ctl.clear_words = clear_words;
+    a.ctl.flags = CFA_LAUNCH_RELEASE;
     for (uint32_t at = 0;;) {
         const uint32_t left = n - at;
-        const uint32_t k = left < (uint32_t)kPutLarge ? left : (uint32_t)kPutLarge;
-        if (k == left) ctl.flags = CFA_LAUNCH_RELEASE;
-        const cudaError_t e = k <= (uint32_t)kPutSmall
-                                  ? put(g_put_small, to + at, from + at, k, status, ctl, stream)
-                                  : put(g_put_large, to + at, from + at, k, status, ctl, stream);
-        at += k;
+        a.to = to + at;
+        a.n = left < (uint32_t)kPutLarge ? left : (uint32_t)kPutLarge;
+        const cudaError_t e = a.n <= (uint32_t)kPutSmall
+                                  ? put<kPutSmall>(a, g_host_items + at, stream)
+                                  : put<kPutLarge>(a, g_host_items + at, stream);
+        at += a.n;
         if (e != cudaSuccess || at == n) return e;
-        ctl = cfa_launch_ctl{};
-        status = nullptr;
+        a = PutArgs{};
+        a.ctl.flags = CFA_LAUNCH_EARLY | CFA_LAUNCH_WAIT_LAST | CFA_LAUNCH_RELEASE;
     }
 }
 
@@ -314,6 +315,7 @@ extern "C" cfa_status cfa_unpack_noalloc(const cfa_tensor_entry *entries, size_t
     /* validate every entry and count the work items, per class, without storing anything */
     uint32_t count[CFA_N_CLASSES][kKinds] = {};
     uint64_t slab_bytes[CFA_N_CLASSES] = {}; /* of all slabs: source or destination, the wider */
+    uint64_t total = 0;
     for (size_t i = 0; i < n_entries; ++i) {
         uint64_t n, off;
         int es_s, es_d, conv;
@@ -326,9 +328,7 @@ extern "C" cfa_status cfa_unpack_noalloc(const cfa_tensor_entry *entries, size_t
         const uint64_t dst0 = (uint64_t)(uintptr_t)dsts[entries[i].dst_index].dev_ptr + off;
         const uint64_t items = nb < kTinyBytes ? tiny_items(dst0, nb)
                                                : (nb + kSlabBytes - 1) / kSlabBytes;
-        uint64_t total = items;
-        for (int k = 0; k < CFA_N_CLASSES; ++k)
-            for (int t = 0; t < kKinds; ++t) total += count[k][t];
+        total += items;
         if (total > CFA_NOALLOC_MAX_ITEMS) {
             say("cfa_unpack_noalloc: the manifest needs more than the %d work items of the "
                 "fixed scratch (one per 2 MiB of destination, one per 512 bytes of a tensor "
@@ -341,11 +341,11 @@ extern "C" cfa_status cfa_unpack_noalloc(const cfa_tensor_entry *entries, size_t
 
     /* lay the items out as [class 0 slabs][class 0 tiny][class 1 slabs] ... */
     uint32_t base[CFA_N_CLASSES][kKinds], cursor[CFA_N_CLASSES][kKinds];
-    uint32_t total = 0;
+    uint32_t at = 0;
     for (int k = 0; k < CFA_N_CLASSES; ++k)
         for (int t = 0; t < kKinds; ++t) {
-            base[k][t] = cursor[k][t] = total;
-            total += count[k][t];
+            base[k][t] = cursor[k][t] = at;
+            at += count[k][t];
         }
     for (size_t i = 0; i < n_entries; ++i) {
         uint64_t n, off;
@@ -398,7 +398,7 @@ extern "C" cfa_status cfa_unpack_noalloc(const cfa_tensor_entry *entries, size_t
      * waits for the upload, the others only end in order */
     int *status = status_dev ? status_dev : &scratch->status;
     unsigned long long *ck = reinterpret_cast<unsigned long long *>(cksum_dev);
-    e = put_items(scratch->items, g_host_items, total, status, ck, ck ? n_entries : 0, stream);
+    e = put_items(scratch->items, (uint32_t)total, status, ck, ck ? n_entries : 0, stream);
     const uint64_t src = (uint64_t)(uintptr_t)blob_dev;
     cfa_launch_ctl ctl{};
     ctl.flags = CFA_LAUNCH_EARLY | CFA_LAUNCH_WAIT_FIRST | CFA_LAUNCH_RELEASE;

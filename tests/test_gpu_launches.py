@@ -91,6 +91,31 @@ def test_noalloc_items_are_cut_into_parts():
     assert np.array_equal(ck.cpu().numpy().view(np.uint64), c.checksums())
 
 
+@pytest.mark.parametrize("n", [1, 112, 113, 1000, 1001, 1112, 2113, 16384])
+def test_noalloc_uploads_any_number_of_items(n):
+    """Item counts around what one launch of the upload carries, up to the most; twice, since a
+    call reads its descriptors where the one before left its own."""
+    per, es = 8192, 2
+    blob = torch.randint(0, 256, (n * per,), dtype=torch.uint8, device="cuda")
+    flip = torch.empty_like(blob)
+    ck = torch.full((n,), -1, dtype=torch.int64, device="cuda")
+    err = ctypes.create_string_buffer(256)
+    for order in (np.arange(n), np.arange(n)[::-1].copy()):
+        flip.fill_(0xA5)
+        ents = cfa.make_entries(dtype=["bf16"] * n, shape=[(per // es,)] * n,
+                                offset=np.arange(n) * per, dst=np.zeros(n, np.int64),
+                                row=order * (per // es))
+        dsts = cfa.make_dsts([(flip.data_ptr(), "bf16", (n * per // es,))])
+        st = _lib.load().cfa_unpack_noalloc(
+            ents.arr.ctypes.data, n, dsts.ctypes.data, 1, blob.data_ptr(), blob.numel(),
+            ck.data_ptr(), None, torch.cuda.current_stream().cuda_stream, err, len(err))
+        assert st == 0, err.value
+        to = torch.from_numpy(order).cuda()
+        assert torch.equal(flip.view(n, per)[to], blob.view(n, per))
+        sums = blob.view(torch.int16).view(n, -1).to(torch.int64).bitwise_and_(0xFFFF).sum(1)
+        assert torch.equal(ck, sums)
+
+
 def chunk_plan(c, chunk):
     return cfa.Plan(c.entries, c.dsts, c.blob_bytes, chunk_bytes=chunk, dev_slots=0, host_slots=0)
 
