@@ -231,12 +231,9 @@ template <bool ROWS> __device__ __forceinline__ BulkItem bulk_decode(const RawIt
     return w;
 }
 
-/* An early launch asks for the first stage of this many parts per CTA (45 MB in all, a third of
- * L2) before it may read them: consecutive 64 MiB chunks, 3.4 GB, 1233 us without, 1159 with two,
- * 1128 with three, 1181 with four; 16 MiB chunks, 1.4 GB, 764, 602, 620, 612. */
-constexpr uint32_t kAskParts = 3;
-
-/* Asks for the first stage of part v, a contiguous run, in L2. */
+/* Asks for the first stage of part v, a contiguous run, in L2.  An early launch does so for each
+ * CTA's first part before it may read it: consecutive 64 MiB chunks, 3.4 GB, 1245 us without, 1228
+ * so, 1264 with two parts, 1285 with three; 16 MiB chunks, 1.4 GB, 802, 790, 797, 789. */
 template <bool ROWS>
 __device__ __forceinline__ void bulk_ask(const BulkArgs &a, uint32_t v, const RawItem &raw)
 {
@@ -312,13 +309,8 @@ __global__ void __launch_bounds__(kThreads) cfa_bulk_kernel(const BulkArgs a)
     if (threadIdx.x == 0 && (a.ctl.flags & CFA_LAUNCH_WAIT_FIRST)) {
         /* The source is not to be read yet (the kernel before may still be writing it), but asking
          * for it in L2, where every write arrives, is harmless, and fills the time in which the
-         * kernel before runs out of work. */
+         * kernel before ends. */
         if (blockIdx.x < a.n_items) bulk_ask<ROWS>(a, blockIdx.x, cur);
-        if (blockIdx.x + gridDim.x < a.n_items) bulk_ask<ROWS>(a, blockIdx.x + gridDim.x, nxt);
-        for (uint32_t j = 2; j < kAskParts; ++j) {
-            const uint32_t v = blockIdx.x + j * gridDim.x;
-            if (v < a.n_items) bulk_ask<ROWS>(a, v, bulk_fetch<ROWS>(a, v));
-        }
     }
     launch_begin(a.ctl);
     __syncthreads();

@@ -212,7 +212,10 @@ static inline uint32_t cfa_parts_log2(const cfa_cut *cut, uint64_t n_items, uint
  *   WAIT_LAST   the kernel does not need the one before it (they write disjoint bytes and add
  *               checksums atomically) but ends only after it, so that whatever follows on the
  *               stream follows both
- *   RELEASE     the kernel releases its dependents as soon as its CTAs run
+ *   RELEASE     the kernel releases its dependents as soon as its CTAs run; never set on the last
+ *               kernel of a call, whose dependents are the caller's: a kernel of theirs with the
+ *               launch attribute starts when the CTAs of a call's last kernel have ended, as after
+ *               any kernel that does not release
  * clear: words set to zero by this launch (the checksum half of the next load), or NULL.
  */
 #define CFA_LAUNCH_EARLY 1u
@@ -225,6 +228,17 @@ typedef struct cfa_launch_ctl {
     uint32_t flags;
     uint32_t pad;
 } cfa_launch_ctl;
+
+/* Flags of kernel i of the n that a call launches one after the other on a stream, all independent
+ * of one another.  early: the first is launched with the attribute as well, and waits inside. */
+static inline uint32_t cfa_chain_flags(uint32_t i, uint32_t n, int early)
+{
+    uint32_t f = 0;
+    if (i > 0) f |= CFA_LAUNCH_EARLY | CFA_LAUNCH_WAIT_LAST;
+    else if (early) f |= CFA_LAUNCH_EARLY | CFA_LAUNCH_WAIT_FIRST;
+    if (i + 1 < n) f |= CFA_LAUNCH_RELEASE;
+    return f;
+}
 
 /* Sets the calling thread's detail string returned by cfa_last_error(NULL). */
 void cfa_internal_set_error(const char *msg);

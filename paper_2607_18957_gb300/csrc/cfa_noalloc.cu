@@ -114,17 +114,18 @@ template <int CAP> cudaError_t put(PutArgs &a, cfa_work *from, cudaStream_t stre
 
 /* Uploads the first n of g_host_items to `to` in stream order; the first launch clears the status
  * word and the checksums.  The launches write disjoint bytes: each starts once the one before it
- * runs and ends after it. */
+ * runs and ends after it; an unpack kernel follows if there are items. */
 cudaError_t put_items(cfa_work *to, uint32_t n, int *status, unsigned long long *clear,
                       uint64_t clear_words, cudaStream_t stream)
 {
+    const uint32_t launches = n ? (n + kPutLarge - 1) / kPutLarge + 1 : 1; /* the unpack counted */
     PutArgs a{};
     a.status = status;
     a.ctl.clear = clear;
     a.ctl.clear_words = clear_words;
-    a.ctl.flags = CFA_LAUNCH_RELEASE;
-    for (uint32_t at = 0;;) {
+    for (uint32_t at = 0, i = 0;; ++i) {
         const uint32_t left = n - at;
+        a.ctl.flags = cfa_chain_flags(i, launches, 0);
         a.to = to + at;
         a.n = left < (uint32_t)kPutLarge ? left : (uint32_t)kPutLarge;
         const cudaError_t e = a.n <= (uint32_t)kPutSmall
@@ -133,7 +134,6 @@ cudaError_t put_items(cfa_work *to, uint32_t n, int *status, unsigned long long 
         at += a.n;
         if (e != cudaSuccess || at == n) return e;
         a = PutArgs{};
-        a.ctl.flags = CFA_LAUNCH_EARLY | CFA_LAUNCH_WAIT_LAST | CFA_LAUNCH_RELEASE;
     }
 }
 
@@ -401,15 +401,16 @@ extern "C" cfa_status cfa_unpack_noalloc(const cfa_tensor_entry *entries, size_t
     e = put_items(scratch->items, (uint32_t)total, status, ck, ck ? n_entries : 0, stream);
     const uint64_t src = (uint64_t)(uintptr_t)blob_dev;
     cfa_launch_ctl ctl{};
-    ctl.flags = CFA_LAUNCH_EARLY | CFA_LAUNCH_WAIT_FIRST | CFA_LAUNCH_RELEASE;
+    uint32_t kernels = 0, i = 0;
+    for (int k = 0; k < CFA_N_CLASSES; ++k) kernels += count[k][SLAB] || count[k][TINY];
     for (int k = 0; e == cudaSuccess && k < CFA_N_CLASSES; ++k) {
         if (!count[k][SLAB] && !count[k][TINY]) continue;
+        ctl.flags = cfa_chain_flags(i++, kernels, 1);
         const cfa_cut cut = {kSlabBytes << (cfa_class_narrows(k) ? 1 : 0), slab_bytes[k],
                              kPartBytes};
         e = cfa_launch_unpack(k, scratch->items + base[k][SLAB], count[k][SLAB],
                               scratch->items + base[k][TINY], count[k][TINY], src, 0, 0,
                               blob_bytes, ck, status, g_grid_cap[dev][k], &cut, 1, &ctl, stream);
-        ctl.flags = CFA_LAUNCH_EARLY | CFA_LAUNCH_WAIT_LAST | CFA_LAUNCH_RELEASE;
     }
     if (e != cudaSuccess) {
         say("cfa_unpack_noalloc: CUDA error %s", cudaGetErrorString(e));

@@ -16,10 +16,12 @@ uint32_t parts_log2(uint64_t item_bytes, uint64_t bytes, uint32_t part_bytes, ui
     const cfa_cut cut = {item_bytes, bytes, part_bytes};
     return cfa_parts_log2(&cut, n_items, grid);
 }
+uint32_t chain_flags(uint32_t i, uint32_t n, int early) { return cfa_chain_flags(i, n, early); }
 """
 
 KIB, MIB = 1 << 10, 1 << 20
 GRID = 456
+EARLY, WAIT_FIRST, WAIT_LAST, RELEASE = 1, 2, 4, 8
 
 
 @pytest.fixture(scope="module")
@@ -58,3 +60,18 @@ def test_visits_stay_near_the_parts_that_hold_bytes(rules, item, part, n, mean):
 
 def test_no_cut_without_a_part_size(rules):
     assert rules.parts_log2(64 * MIB, 1 << 40, 0, 1 << 14, GRID) == 0
+
+
+@pytest.mark.parametrize("early", [0, 1])
+@pytest.mark.parametrize("n", [1, 2, 3, 9])
+def test_a_call_releases_its_own_kernels_only(rules, n, early):
+    """The last kernel of a call never releases its dependents, which are the caller's kernels; a
+    kernel that starts early without waiting first follows one that releases; and it waits at its
+    end, so that what follows on the stream follows every kernel of the call."""
+    flags = [rules.chain_flags(i, n, early) for i in range(n)]
+    assert not flags[-1] & RELEASE
+    assert flags[0] & (EARLY | WAIT_FIRST) == (EARLY | WAIT_FIRST if early else 0)
+    assert not flags[0] & WAIT_LAST
+    for before, f in zip(flags, flags[1:]):
+        assert before & RELEASE
+        assert f & EARLY and f & WAIT_LAST and not f & WAIT_FIRST
