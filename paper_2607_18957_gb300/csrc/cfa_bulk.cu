@@ -313,6 +313,9 @@ __global__ void __launch_bounds__(kThreads) cfa_bulk_kernel(const BulkArgs a)
         if (blockIdx.x < a.n_items) bulk_ask<ROWS>(a, blockIdx.x, cur);
     }
     launch_begin(a.ctl);
+    /* what the kernel before wrote is read by bulk copies (the async proxy) from here on */
+    if (threadIdx.x == 0 && (a.ctl.flags & CFA_LAUNCH_EARLY))
+        asm volatile("fence.proxy.async.global;" ::: "memory");
     __syncthreads();
     const uint32_t lane = threadIdx.x & 31u;
     const uint32_t limit = a.spin_limit & ~kLoseLoads;

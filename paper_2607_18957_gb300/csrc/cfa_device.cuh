@@ -34,20 +34,23 @@ template <> __device__ __forceinline__ uint64_t vsum<8>(uint4 v)
     return (((uint64_t)v.y << 32) | v.x) + (((uint64_t)v.w << 32) | v.z);
 }
 
-/* Before the first load of a kernel that may start while the one before it still runs, every
- * thread: nothing that an older kernel left in this SM's L1 is to be read, whether or not such a
- * start clears it.  (Staging slots and descriptor memory are written again between launches.) */
+/* Before a load that does not wait for the kernel before: nothing that an older kernel left in this
+ * SM's L1 is to be read, whether or not an early start clears it.  (Staging slots and descriptor
+ * memory are written again between launches.) */
 __device__ __forceinline__ void launch_early(const cfa_launch_ctl &c)
 {
     if (c.flags & CFA_LAUNCH_EARLY) __threadfence();
 }
 
-/* After launch_early, every thread: the launch's place in its stream (cfa_launch_ctl).
+/* Before a kernel's first load of its source, every thread: the launch's place in its stream
+ * (cfa_launch_ctl).  The fence comes after the wait, so that it also covers what came into L1
+ * before the wait was over.
  * Dependents are released only after the wait, so that a later kernel of the group, which does
  * not wait for the source itself, cannot start before the source is there. */
 __device__ __forceinline__ void launch_begin(const cfa_launch_ctl &c)
 {
     if (c.flags & CFA_LAUNCH_WAIT_FIRST) asm volatile("griddepcontrol.wait;" ::: "memory");
+    launch_early(c);
     if (c.flags & CFA_LAUNCH_RELEASE)
         asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     if (c.clear) {

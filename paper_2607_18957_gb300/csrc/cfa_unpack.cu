@@ -33,7 +33,6 @@ namespace {
 
 using cfa_dev::launch_begin;
 using cfa_dev::launch_ctl;
-using cfa_dev::launch_early;
 using cfa_dev::launch_end;
 using cfa_dev::vsum;
 using cfa_dev::warp_sum;
@@ -75,13 +74,17 @@ struct UnpackArgs {
     cfa_launch_ctl ctl;
 };
 
-/* ---- memory operations ------------------------------------------------------------------ */
+/* ---- memory operations ------------------------------------------------------------------
+ * Loads are coherent ones, not ld.global.nc: a kernel that is launched early is there while the
+ * kernel before it writes the source, or the descriptors of the no-alloc entry point, and the
+ * non-coherent form is for memory that nobody writes while the kernel runs (no difference in time
+ * on any load measured). */
 
 /* Streaming 16-byte load of staging data: read once, never by L1. */
 __device__ __forceinline__ uint4 ld_stream(const void *p)
 {
     uint4 v;
-    asm("ld.global.nc.L1::no_allocate.v4.u32 {%0, %1, %2, %3}, [%4];"
+    asm("ld.global.L1::no_allocate.v4.u32 {%0, %1, %2, %3}, [%4];"
         : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w)
         : "l"(p));
     return v;
@@ -91,9 +94,24 @@ __device__ __forceinline__ uint4 ld_stream(const void *p)
 __device__ __forceinline__ uint4 ld_shared_line(const void *p)
 {
     uint4 v;
-    asm("ld.global.nc.v4.u32 {%0, %1, %2, %3}, [%4];"
+    asm("ld.global.v4.u32 {%0, %1, %2, %3}, [%4];"
         : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w)
         : "l"(p));
+    return v;
+}
+
+/* The same for 8 and 4 bytes. */
+__device__ __forceinline__ uint2 ld_shared_line8(const void *p)
+{
+    uint2 v;
+    asm("ld.global.v2.u32 {%0, %1}, [%2];" : "=r"(v.x), "=r"(v.y) : "l"(p));
+    return v;
+}
+
+__device__ __forceinline__ uint32_t ld_shared_line4(const void *p)
+{
+    uint32_t v;
+    asm("ld.global.u32 %0, [%1];" : "=r"(v) : "l"(p));
     return v;
 }
 
@@ -489,7 +507,7 @@ __device__ uint64_t convert_run(const uint8_t *__restrict__ src, uint8_t *__rest
                     const uint2 *s2 = reinterpret_cast<const uint2 *>(src + 32ull * g);
 #pragma unroll
                     for (int q = 0; q < 4; ++q) {
-                        const uint2 v = __ldg(s2 + q);
+                        const uint2 v = ld_shared_line8(s2 + q);
                         x[u][2 * q] = v.x;
                         x[u][2 * q + 1] = v.y;
                     }
@@ -498,14 +516,14 @@ __device__ uint64_t convert_run(const uint8_t *__restrict__ src, uint8_t *__rest
                      * pairs */
                     const uint32_t *s1 = reinterpret_cast<const uint32_t *>(src + 32ull * g);
                     const uint2 *s2 = reinterpret_cast<const uint2 *>(s1 + 1);
-                    x[u][0] = __ldg(s1);
+                    x[u][0] = ld_shared_line4(s1);
 #pragma unroll
                     for (int q = 0; q < 3; ++q) {
-                        const uint2 v = __ldg(s2 + q);
+                        const uint2 v = ld_shared_line8(s2 + q);
                         x[u][1 + 2 * q] = v.x;
                         x[u][2 + 2 * q] = v.y;
                     }
-                    x[u][7] = __ldg(s1 + 7);
+                    x[u][7] = ld_shared_line4(s1 + 7);
                 }
             }
 #pragma unroll
@@ -666,7 +684,6 @@ __global__ void __launch_bounds__(kThreads, unpack_min_blocks(CLS))
     cfa_unpack_kernel(const UnpackArgs a)
 {
     __shared__ unsigned long long red[kWarps];
-    launch_early(a.ctl);
     launch_begin(a.ctl);
     const uint32_t n_groups = (a.n_tiny + kTinyPerGroup - 1) / kTinyPerGroup;
     const uint32_t n_slabs = a.n_slabs << a.parts_log2; /* parts of slabs */
@@ -901,10 +918,10 @@ __device__ __forceinline__ uint64_t copy_diff_phase(const uint8_t *src, uint8_t 
 __device__ __forceinline__ cfa_work ld_work_now(const cfa_work *p)
 {
     uint32_t a0, a1, a2, a3, b0, b1, b2, b3;
-    asm volatile("ld.global.nc.v4.u32 {%0, %1, %2, %3}, [%4];"
+    asm volatile("ld.global.v4.u32 {%0, %1, %2, %3}, [%4];"
                  : "=r"(a0), "=r"(a1), "=r"(a2), "=r"(a3)
                  : "l"(p));
-    asm volatile("ld.global.nc.v4.u32 {%0, %1, %2, %3}, [%4];"
+    asm volatile("ld.global.v4.u32 {%0, %1, %2, %3}, [%4];"
                  : "=r"(b0), "=r"(b1), "=r"(b2), "=r"(b3)
                  : "l"(reinterpret_cast<const uint8_t *>(p) + 16));
     cfa_work w;
@@ -1167,7 +1184,6 @@ template <int CLS>
 __global__ void __launch_bounds__(kThreads, (CLS == 0 ? kCopyMinBlocks : unpack_min_blocks(CLS)))
     cfa_tiny_kernel(const UnpackArgs a)
 {
-    launch_early(a.ctl);
     launch_begin(a.ctl);
     if constexpr (CLS < 4) {
         /* device-memory sources take the shared-memory pipeline; host memory read in place over
@@ -1294,7 +1310,6 @@ __global__ void __launch_bounds__(kThreads, (CLS == 0 || ClassOf<CLS>::ses == 2
     constexpr int DES = C::des;
     __shared__ unsigned long long red[kWarps];
     const uint32_t lane = threadIdx.x & 31u, warp = threadIdx.x >> 5;
-    launch_early(a.ctl);
     launch_begin(a.ctl);
     uint64_t acc = 0;
     uint32_t acc_ck = CFA_NO_CK;

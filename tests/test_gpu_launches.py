@@ -159,6 +159,33 @@ def test_chunks_through_one_slot_that_is_overwritten(chunk):
             assert torch.equal(c.out, c.want)
 
 
+@pytest.mark.parametrize("kind", ["aligned", "phases", "tiny"])
+def test_chunks_that_the_kernel_before_writes(kind):
+    """Chunks whose source is written by the kernel right before on the stream, an unpack of
+    another plan, with new contents each time: bytes and sums."""
+    chunk = 2 << 20
+    c = Copies({"aligned": tensors(SIZES, [(0, 0)]), "phases": tensors(SIZES, [(1, 0), (1, 3)]),
+                "tiny": tensors([96, 1000, 5000] * 60, [(0, 0), (1, 3)])}[kind])
+    n = c.blob_bytes
+    mid = torch.zeros(n, dtype=torch.uint8, device="cuda")
+    copy = cfa.make_entries(dtype=["u8"], shape=[(n,)], offset=[0], dst=[0])
+    with cfa.Plan(copy, [(mid.data_ptr(), "u8", (n,))], n, chunk_bytes=chunk, dev_slots=0,
+                  host_slots=0) as first, chunk_plan(c, chunk) as second:
+        second.load_async(cfa.Source.device(mid.data_ptr()))  # checksums are those of a load
+        for r in range(4):
+            c.blob.bitwise_xor_(0x5A + r)
+            c.out.fill_(0xA5)
+            second.reset_checksums()
+            for k in range(second.info()["n_chunks"]):
+                first.unpack_chunks_async(k, k + 1, c.blob.data_ptr() + k * chunk)
+                second.unpack_chunks_async(k, k + 1, mid.data_ptr() + k * chunk)
+            torch.cuda.synchronize()
+            for _, a, t, m in c.runs:
+                c.want[t:t + m] = c.blob[a:a + m]
+            assert torch.equal(c.out, c.want)
+            assert np.array_equal(second.checksums(), c.checksums())
+
+
 def test_consecutive_chunks_in_a_cuda_graph():
     chunk = 4 << 20
     c = Copies(tensors(SIZES + [96, 5000], [(0, 0), (1, 3)]))

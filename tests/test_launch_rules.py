@@ -2,6 +2,7 @@
 their own."""
 import ctypes
 import os
+import re
 import subprocess
 
 import pytest
@@ -75,3 +76,18 @@ def test_a_call_releases_its_own_kernels_only(rules, n, early):
     for before, f in zip(flags, flags[1:]):
         assert before & RELEASE
         assert f & EARLY and f & WAIT_LAST and not f & WAIT_FIRST
+
+
+def test_kernels_that_start_early_read_with_coherent_loads():
+    """A kernel launched early is resident while the one before it writes its source: non-coherent
+    loads, for memory that nobody writes while a kernel runs, are for a plan's own descriptors."""
+    csrc = os.path.join(ROOT, "paper_2607_18957_gb300", "csrc")
+    for name in sorted(os.listdir(csrc)):
+        if not name.endswith((".cu", ".cuh")):
+            continue
+        text = re.sub(r"/\*.*?\*/", "", open(os.path.join(csrc, name)).read(), flags=re.S)
+        assert "global.nc" not in text, name
+        if name == "cfa_bulk.cu":  # the descriptors, in bulk_fetch
+            fetch = text.index("bulk_fetch(")
+            text = text[:fetch] + text[text.index("return b;", fetch):]
+        assert "__ldg" not in text, name
