@@ -141,7 +141,12 @@ struct cfa_plan {
     int n_host_slots = 0;
     /* page-locked words for reading the status word, and a half of up to kReadWords words, back */
     unsigned long long *h_read = nullptr;
-    std::mutex read_mu;
+    /* Held while a load is enqueued and while the last load's half is read back: what is read is a
+     * load that has completed, and is read before the next load clears it.  Recursive for the
+     * gather callback, which runs inside cfa_load_async. */
+    std::recursive_mutex read_mu;
+    std::atomic<bool> enqueuing{false};   /* by a load, not by a reader */
+    std::atomic<uint64_t> n_recorded{0};  /* loads whose ev_all has been recorded */
     cudaStream_t fill_stream = nullptr, copy_stream = nullptr, aux_stream = nullptr;
     /* pinned sources: column slices read in place over the host link, beside the copy ring */
     cudaStream_t direct_stream = nullptr;
@@ -171,8 +176,8 @@ struct cfa_plan {
      * ev_all), so a load records one event per such point and not one per layer. */
     std::unique_ptr<std::atomic<cudaEvent_t>[]> layer_ready;
     std::unique_ptr<cfa::Pool> pool;
-    std::vector<std::unique_ptr<LoadCtx>> loads;
-    LoadCtx *last = nullptr;
+    std::vector<std::shared_ptr<LoadCtx>> loads;
+    std::shared_ptr<LoadCtx> last; /* read and replaced with std::atomic_load / atomic_store */
     std::mutex mu;
     char err[512] = {0};
     uint64_t n_loads = 0;
@@ -695,10 +700,9 @@ cfa_status check_status(cfa_plan *p, int h)
     return CFA_OK;
 }
 
-/* Reads the status word of the load that p->ev_all has completed. */
+/* Reads the status word of the completed last load (the caller holds read_mu). */
 cfa_status check_status_word(cfa_plan *p)
 {
-    std::lock_guard<std::mutex> lk(p->read_mu);
     CK(p, cudaMemcpyAsync(p->h_read, p->d_status, sizeof(int), cudaMemcpyDeviceToHost,
                           p->aux_stream));
     CK(p, cudaStreamSynchronize(p->aux_stream));
@@ -739,14 +743,55 @@ cfa_status wait_event_host(cfa_plan *p, cudaEvent_t ev, int64_t timeout_ns)
     }
 }
 
-/* The same, and the error of the load's source, if it had one. */
-cfa_status wait_on_host(cfa_plan *p, cudaEvent_t ev, int64_t timeout_ns)
+/* The error of the last load's source or gather callback, if it had one. */
+int load_error(cfa_plan *p)
 {
-    cfa_status st = wait_event_host(p, ev, timeout_ns);
-    if (st) return st;
-    const int e = p->last->error.load();
+    const std::shared_ptr<LoadCtx> last = std::atomic_load(&p->last);
+    return last->error.load();
+}
+
+bool has_load(const cfa_plan *p) { return std::atomic_load(&p->last) != nullptr; }
+
+/* The load error as the status of a host wait. */
+cfa_status load_status(cfa_plan *p)
+{
+    const int e = load_error(p);
     if (e && e != CFA_ERR_GATHER) set_err(p, "the source callback failed");
     return e;
+}
+
+/* Waits on the host for the end of the last load, and returns its load_status with `lk` locked on
+ * read_mu.  A load that another thread enqueues meanwhile becomes the last one: its ev_all is not
+ * recorded yet when the poll has seen the one before it complete, so the count of records tells
+ * whether that poll was of this load. */
+cfa_status wait_last_load(cfa_plan *p, int64_t timeout_ns,
+                          std::unique_lock<std::recursive_mutex> &lk)
+{
+    const auto t0 = std::chrono::steady_clock::now();
+    for (;;) {
+        int64_t left = timeout_ns;
+        if (timeout_ns > 0) {
+            left -= std::chrono::duration_cast<std::chrono::nanoseconds>(
+                        std::chrono::steady_clock::now() - t0)
+                        .count();
+            left = std::max<int64_t>(left, 0);
+        }
+        const uint64_t n = p->n_recorded.load();
+        cfa_status st = wait_event_host(p, p->ev_all, left);
+        if (st) return st;
+        /* another reader is done in microseconds; a load being enqueued may take longer */
+        if (!p->enqueuing.load()) lk.lock();
+        else if (!lk.try_lock()) {
+            if (left == 0) {
+                set_err(p, "wait timed out after %lld ns", (long long)timeout_ns);
+                return CFA_ERR_TIMEOUT;
+            }
+            std::this_thread::sleep_for(std::chrono::microseconds(2));
+            continue;
+        }
+        if (n == p->n_recorded.load()) return load_status(p);
+        lk.unlock();
+    }
 }
 
 } // namespace
@@ -907,8 +952,12 @@ cfa_status cfa_load_async(cfa_plan *p, const cfa_source *src, cfa_stream stream_
             return CFA_ERR_NOMEM;
         }
     }
-    std::unique_ptr<LoadCtx> ctx(new (std::nothrow) LoadCtx());
-    if (!ctx) return CFA_ERR_NOMEM;
+    std::shared_ptr<LoadCtx> ctx;
+    try {
+        ctx = std::make_shared<LoadCtx>();
+    } catch (const std::bad_alloc &) {
+        return CFA_ERR_NOMEM;
+    }
     ctx->plan = p;
     ctx->src = *src;
     if (staged) {
@@ -920,8 +969,21 @@ cfa_status cfa_load_async(cfa_plan *p, const cfa_source *src, cfa_stream stream_
                                    {}};
     }
     LoadCtx *cx = ctx.get();
-    p->loads.push_back(std::move(ctx));
-    p->last = cx;
+    p->loads.push_back(ctx);
+    struct Enqueuing {
+        cfa_plan *p;
+        explicit Enqueuing(cfa_plan *p_) : p(p_)
+        {
+            p->read_mu.lock();
+            p->enqueuing = true;
+        }
+        ~Enqueuing()
+        {
+            p->enqueuing = false;
+            p->read_mu.unlock();
+        }
+    } enqueuing(p);
+    std::atomic_store(&p->last, ctx);
     p->n_loads++;
     p->last_launches = 0;
     p->last_h2d = 0;
@@ -1170,6 +1232,7 @@ cfa_status cfa_load_async(cfa_plan *p, const cfa_source *src, cfa_stream stream_
         p->ck_clear_words = 0;
     }
     CK(p, cudaEventRecord(p->ev_all, cs));
+    p->n_recorded++;
     logf("load %llu enqueued: source kind %d, %llu kernel launches, %u staged chunks",
          (unsigned long long)p->n_loads, kind, (unsigned long long)p->last_launches, p->last_h2d);
     return cx->error.load() == CFA_ERR_GATHER ? CFA_ERR_GATHER : CFA_OK;
@@ -1178,7 +1241,7 @@ cfa_status cfa_load_async(cfa_plan *p, const cfa_source *src, cfa_stream stream_
 cfa_status cfa_wait_layer(cfa_plan *p, int32_t layer, cfa_stream consumer, int64_t timeout_ns)
 {
     if (!p || p->host_only) return CFA_ERR_INVAL;
-    if (!p->last) {
+    if (!has_load(p)) {
         set_err(p, "no load has been enqueued");
         return CFA_ERR_INVAL;
     }
@@ -1193,24 +1256,27 @@ cfa_status cfa_wait_layer(cfa_plan *p, int32_t layer, cfa_stream consumer, int64
     DeviceGuard g(p->device);
     if (consumer) {
         CK(p, cudaStreamWaitEvent(reinterpret_cast<cudaStream_t>(consumer), ev, 0));
-        const int e = p->last->error.load();
-        return e ? e : CFA_OK;
+        return load_error(p);
     }
-    cfa_status st = wait_on_host(p, ev, timeout_ns);
-    if (st) return st;
-    if (layer == CFA_ALL) return check_status_word(p);
-    return CFA_OK;
+    if (layer == CFA_ALL) {
+        std::unique_lock<std::recursive_mutex> lk(p->read_mu, std::defer_lock);
+        cfa_status st = wait_last_load(p, timeout_ns, lk);
+        return st ? st : check_status_word(p);
+    }
+    cfa_status st = wait_event_host(p, ev, timeout_ns);
+    return st ? st : load_status(p);
 }
 
 cfa_status cfa_get_checksums(cfa_plan *p, uint64_t *host_out, size_t n)
 {
     if (!p || p->host_only || (n && !host_out) || n > p->hp.n_entries) return CFA_ERR_INVAL;
-    if (!p->last) {
+    if (!has_load(p)) {
         set_err(p, "no load has been enqueued");
         return CFA_ERR_INVAL;
     }
     DeviceGuard g(p->device);
-    cfa_status st = wait_on_host(p, p->ev_all, -1);
+    std::unique_lock<std::recursive_mutex> lk(p->read_mu, std::defer_lock);
+    cfa_status st = wait_last_load(p, -1, lk);
     if (st) return st;
     if (p->ck_half_words > kReadWords) {
         if ((st = check_status_word(p)) || !n) return st;
@@ -1220,7 +1286,6 @@ cfa_status cfa_get_checksums(cfa_plan *p, uint64_t *host_out, size_t n)
         return CFA_OK;
     }
     /* the status word lies behind the checksums: one copy reads both */
-    std::lock_guard<std::mutex> lk(p->read_mu);
     CK(p, cudaMemcpyAsync(p->h_read, p->d_ck, p->ck_half_words * sizeof *p->h_read,
                           cudaMemcpyDeviceToHost, p->aux_stream));
     CK(p, cudaStreamSynchronize(p->aux_stream));
@@ -1254,7 +1319,7 @@ cfa_status cfa_get_stats(cfa_plan *p, cfa_stats *s)
     s->loads = p->n_loads;
     s->kernel_launches = p->last_launches;
     s->plan_ms = p->plan_ms;
-    if ((hp.opts.flags & CFA_OPT_TIMING) && p->last && !p->host_only) {
+    if ((hp.opts.flags & CFA_OPT_TIMING) && has_load(p) && !p->host_only) {
         DeviceGuard g(p->device);
         CK(p, cudaEventSynchronize(p->ev_all));
         float ms = 0;
@@ -1276,7 +1341,7 @@ cfa_status cfa_get_stats(cfa_plan *p, cfa_stats *s)
 cfa_status cfa_get_layer_times(cfa_plan *p, float *ms_out, size_t n)
 {
     if (!p || p->host_only || (n && !ms_out) || n > p->hp.n_layers) return CFA_ERR_INVAL;
-    if (!(p->hp.opts.flags & CFA_OPT_TIMING) || !p->last) {
+    if (!(p->hp.opts.flags & CFA_OPT_TIMING) || !has_load(p)) {
         set_err(p, "layer times need a CFA_OPT_TIMING plan and a load");
         return CFA_ERR_INVAL;
     }
@@ -1290,7 +1355,7 @@ cfa_status cfa_get_layer_times(cfa_plan *p, float *ms_out, size_t n)
 cfa_status cfa_get_timeline(cfa_plan *p, cfa_chunk_times *out, size_t n)
 {
     if (!p || p->host_only || (n && !out) || n > p->hp.n_chunks) return CFA_ERR_INVAL;
-    if (!(p->hp.opts.flags & CFA_OPT_TIMING) || !p->last) {
+    if (!(p->hp.opts.flags & CFA_OPT_TIMING) || !has_load(p)) {
         set_err(p, "the timeline needs a CFA_OPT_TIMING plan and a load");
         return CFA_ERR_INVAL;
     }

@@ -489,6 +489,53 @@ def test_tma_wait_that_runs_out_ends_the_kernel_cleanly():
     load_and_compare(CONFIGS["dense"](), "device", chunk=1 << 20)
 
 
+@pytest.mark.parametrize("n", [3, 9000])
+def test_checksums_read_while_another_thread_enqueues_loads(n):
+    """One thread loads two checkpoints in turn, often as soon as the load before has ended, while
+    another reads the checksums: every answer is one of the two checkpoints', whole.  Few and many
+    entries: read back in one copy, and in two."""
+    import threading
+    per = 32 << 20 if n == 3 else 4096
+    blobs = [torch.randint(0, 256, (n * per,), dtype=torch.uint8, device="cuda") for _ in range(2)]
+    want = [b.view(torch.int16).view(n, -1).to(torch.int64).bitwise_and_(0xFFFF).sum(1).cpu()
+            .numpy().view(np.uint64) for b in blobs]
+    out = torch.empty_like(blobs[0])
+    ents = cfa.make_entries(dtype=["bf16"] * n, shape=[(per // 2,)] * n,
+                            offset=np.arange(n) * per, dst=np.zeros(n, np.int64),
+                            row=np.arange(n) * (per // 2))
+    stop, failed, loads = threading.Event(), [], 0
+    with cfa.Plan(ents, [(out.data_ptr(), "bf16", (n * per // 2,))], out.numel(), dev_slots=0,
+                  host_slots=0) as plan:
+        sources = [cfa.Source.device(b.data_ptr()) for b in blobs]
+        plan.load_async(sources[0])
+        torch.cuda.synchronize()
+
+        def load():
+            nonlocal loads
+            stream = torch.cuda.Stream()
+            try:
+                while not stop.is_set():
+                    plan.load_async(sources[loads & 1], stream=stream)
+                    loads += 1
+                    stream.synchronize()
+            except Exception as e:
+                failed.append(e)
+
+        t = threading.Thread(target=load)
+        t.start()
+        try:
+            bad = 0
+            for k in range(2000):
+                if k % 4 == 0:
+                    plan.wait_layer()
+                ck = plan.checksums()
+                bad += not any(np.array_equal(ck, w) for w in want)
+        finally:
+            stop.set()
+            t.join()
+        assert not failed and bad == 0 and loads > 10, (failed, bad, loads)
+
+
 def test_two_plans_load_at_once_from_two_threads():
     """Two plans (different checkpoints, sources and destinations) loading at the same time on
     their own streams from their own host threads: each matches the oracle."""
