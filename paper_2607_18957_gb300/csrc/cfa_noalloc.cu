@@ -323,6 +323,8 @@ extern "C" cfa_status cfa_unpack_noalloc(const cfa_tensor_entry *entries, size_t
             place(entries[i], dsts, n_dsts, blob_bytes, i, &n, &es_s, &es_d, &off, &conv);
         if (st) return st;
         if (!n) continue;
+        if (((uintptr_t)cksum_dev & 7u) && (entries[i].flags & CFA_ENTRY_CKSUM))
+            return fail(CFA_ERR_ALIGN, "has a checksum, and cksum_dev is not 8-byte aligned", i);
         const int cls = conv ? CFA_CLASS_OF_CONV(conv) : log2_es(es_s);
         const uint64_t nb = n * (uint64_t)es_d;
         const uint64_t dst0 = (uint64_t)(uintptr_t)dsts[entries[i].dst_index].dev_ptr + off;
@@ -398,7 +400,12 @@ extern "C" cfa_status cfa_unpack_noalloc(const cfa_tensor_entry *entries, size_t
      * waits for the upload, the others only end in order */
     int *status = status_dev ? status_dev : &scratch->status;
     unsigned long long *ck = reinterpret_cast<unsigned long long *>(cksum_dev);
-    e = put_items(scratch->items, (uint32_t)total, status, ck, ck ? n_entries : 0, stream);
+    if ((uintptr_t)cksum_dev & 7u) { /* for entries without checksums: zeroed and nothing else */
+        e = cudaMemsetAsync(cksum_dev, 0, n_entries * sizeof *cksum_dev, stream);
+        ck = nullptr;
+    }
+    if (e == cudaSuccess)
+        e = put_items(scratch->items, (uint32_t)total, status, ck, ck ? n_entries : 0, stream);
     const uint64_t src = (uint64_t)(uintptr_t)blob_dev;
     cfa_launch_ctl ctl{};
     uint32_t kernels = 0, i = 0;

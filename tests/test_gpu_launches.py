@@ -116,6 +116,27 @@ def test_noalloc_uploads_any_number_of_items(n):
         assert torch.equal(ck, sums)
 
 
+def test_noalloc_checksum_array_off_the_8_byte_grid():
+    """It is zeroed for entries without a checksum, and refused on the host for one with."""
+    c = Copies(tensors([9000], [(0, 0)]))
+    n = len(c.runs)
+    room = torch.full((8 * n + 8,), 0xA5, dtype=torch.uint8, device="cuda")
+    dsts, err = cfa.make_dsts(c.dsts), ctypes.create_string_buffer(256)
+
+    def call(flag):
+        c.entries.arr["flags"] = flag
+        return _lib.load().cfa_unpack_noalloc(
+            c.entries.arr.ctypes.data, n, dsts.ctypes.data, n, c.blob.data_ptr(), c.blob_bytes,
+            room.data_ptr() + 4, None, torch.cuda.current_stream().cuda_stream, err, len(err))
+
+    assert call(_lib.ENTRY_CKSUM) == -11 and b"8-byte" in err.value
+    assert bool((room == 0xA5).all()) and bool((c.out == 0xA5).all())
+    assert call(0) == 0
+    assert torch.equal(c.out, c.want)
+    assert not room[4:4 + 8 * n].any() and bool((room[:4] == 0xA5).all())
+    assert bool((room[4 + 8 * n:] == 0xA5).all())
+
+
 def chunk_plan(c, chunk):
     return cfa.Plan(c.entries, c.dsts, c.blob_bytes, chunk_bytes=chunk, dev_slots=0, host_slots=0)
 
@@ -199,6 +220,53 @@ def test_consecutive_chunks_in_a_cuda_graph():
             unpack_through_one_slot(c, plan, chunk, slot)
             for k in range(plan.info()["n_chunks"]):  # and with nothing in between
                 plan.unpack_chunks_async(k, k + 1, c.blob.data_ptr() + k * chunk)
+        for _ in range(2):
+            c.out.fill_(0xA5)
+            graph.replay()
+            torch.cuda.synchronize()
+            assert torch.equal(c.out, c.want)
+        del graph
+
+
+@pytest.mark.parametrize("before", ["nothing", "memset", "copy_from_host", "other_stream", "kernel"])
+@pytest.mark.parametrize("kind", ["aligned", "phases"])
+def test_chunks_in_a_cuda_graph_behind_other_work(kind, before):
+    """A captured chunk call whose predecessor in the graph is no kernel, or not on its stream."""
+    chunk = 4 << 20
+    c = Copies(tensors(SIZES, [(0, 0)] if kind == "aligned" else [(1, 0), (1, 3)]))
+    host = c.blob.cpu().pin_memory()
+    slot = torch.zeros(chunk, dtype=torch.uint8, device="cuda")
+    other, joined = torch.cuda.Stream(), torch.cuda.Event()
+    with chunk_plan(c, chunk) as plan:
+        chunks = [(k, host[k * chunk:(k + 1) * chunk]) for k in range(plan.info()["n_chunks"])]
+
+        def load():
+            for k, part in chunks:
+                if before in ("nothing", "memset"):
+                    if before == "memset":
+                        plan.reset_checksums()
+                    plan.unpack_chunks_async(k, k + 1, c.blob.data_ptr() + k * chunk)
+                    continue
+                if before == "other_stream":
+                    other.wait_stream(torch.cuda.current_stream())
+                    with torch.cuda.stream(other):
+                        slot[:part.numel()].copy_(part, non_blocking=True)
+                        joined.record()
+                    torch.cuda.current_stream().wait_event(joined)
+                else:
+                    slot[:part.numel()].copy_(part, non_blocking=True)
+                    if before == "kernel":
+                        slot[:part.numel()].bitwise_xor_(0xFF).bitwise_xor_(0xFF)
+                plan.unpack_chunks_async(k, k + 1, slot.data_ptr())
+
+        side = torch.cuda.Stream()
+        with torch.cuda.stream(side):
+            load()
+        torch.cuda.synchronize()
+        assert torch.equal(c.out, c.want)
+        graph = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(graph):
+            load()
         for _ in range(2):
             c.out.fill_(0xA5)
             graph.replay()
