@@ -8,6 +8,7 @@ import numpy as np
 import pytest
 import torch
 
+import oracle
 import paper_2607_18957_gb300 as cfa
 from paper_2607_18957_gb300 import _lib
 
@@ -63,9 +64,11 @@ SIZES = [8192, PART - 16, PART, PART + 16, 2 * PART + 48, 7 * PART + 8, 300 * 10
 
 
 @pytest.mark.parametrize("phases", [[(0, 0)], [(0, 0), (1, 0), (0, 1), (1, 3)]])
-@pytest.mark.parametrize("slab_kib", [0, 256, 4096])
-def test_planned_items_are_cut_into_parts(phases, slab_kib):
-    c = Copies(tensors(SIZES, phases))
+@pytest.mark.parametrize("slab_kib,filler_mib", [(0, 0), (0, 600), (256, 0), (4096, 0)])
+def test_planned_items_are_cut_into_parts(phases, slab_kib, filler_mib):
+    """Whole loads.  The plan's own slabs are 32 KiB here, or 128 KiB with 600 MiB more in the load,
+    and those of aligned copies are then cut into four parts; the caller's slabs stay whole."""
+    c = Copies(tensors(SIZES, phases) + [("bf16", filler_mib << 20, 0, 0)] * (filler_mib > 0))
     with cfa.Plan(c.entries, c.dsts, c.blob_bytes, dev_slots=0, host_slots=0,
                   slab_bytes=slab_kib << 10) as plan:
         plan.load_async(cfa.Source.device(c.blob.data_ptr()))
@@ -137,8 +140,9 @@ def test_noalloc_checksum_array_off_the_8_byte_grid():
     assert bool((room[4 + 8 * n:] == 0xA5).all())
 
 
-def chunk_plan(c, chunk):
-    return cfa.Plan(c.entries, c.dsts, c.blob_bytes, chunk_bytes=chunk, dev_slots=0, host_slots=0)
+def chunk_plan(c, chunk, slab_kib=0):
+    return cfa.Plan(c.entries, c.dsts, c.blob_bytes, chunk_bytes=chunk, slab_bytes=slab_kib << 10,
+                    dev_slots=0, host_slots=0)
 
 
 def test_a_chunk_of_very_many_small_items_under_large_slabs():
@@ -168,16 +172,76 @@ def unpack_through_one_slot(c, plan, chunk, slot):
         plan.unpack_chunks_async(k, k + 1, slot.data_ptr())
 
 
-@pytest.mark.parametrize("chunk", [1 << 20, 8 << 20])
-def test_chunks_through_one_slot_that_is_overwritten(chunk):
+@pytest.mark.parametrize("chunk,slab_kib", [(1 << 20, 0), (8 << 20, 0), (8 << 20, 256),
+                                            (8 << 20, 4096)])
+def test_chunks_through_one_slot_that_is_overwritten(chunk, slab_kib):
+    """The plan's own slabs hold one part here; slabs of 256 KiB and 4 MiB are cut into several."""
     c = Copies(tensors(SIZES + [96, 5000], [(0, 0), (1, 3)]))
     slot = torch.empty(chunk, dtype=torch.uint8, device="cuda")
-    with chunk_plan(c, chunk) as plan:
+    with chunk_plan(c, chunk, slab_kib) as plan:
+        plan.load_async(cfa.Source.device(c.blob.data_ptr()))  # checksums are those of a load
         for _ in range(3):
             c.out.fill_(0xA5)
             plan.reset_checksums()
             unpack_through_one_slot(c, plan, chunk, slot)
+            torch.cuda.synchronize()
             assert torch.equal(c.out, c.want)
+            assert np.array_equal(plan.checksums(), c.checksums())
+
+
+PAIRS = [("f32", "bf16"), ("f32", "f16"), ("f16", "bf16"), ("bf16", "f32"), ("f16", "f32")]
+UINT = {1: np.uint8, 2: np.uint16, 4: np.uint32, 8: np.uint64}
+
+
+@pytest.mark.parametrize("chunk,slab_kib", [(1 << 20, 0), (8 << 20, 256), (8 << 20, 4096)])
+def test_converted_chunks_and_column_slices_through_one_slot(chunk, slab_kib):
+    """Every conversion, and column slices on both of their kernels and with a conversion, by
+    chunks from a slot that is overwritten in between; the larger slabs are cut into parts, row
+    blocks in the middle of rows."""
+    rng = np.random.default_rng(11)
+    es = {**ES, "f16": 2}
+    jobs = [(s, d, None, n) for s, d in PAIRS for n in (5000, 33_000, 400_003)]
+    jobs += [(s, d, 70, n // es[s]) for n in (1000, 4112, 7168, 32_784, 100_000)
+             for s, d in (("u8", "u8"), ("f32", "f32"), ("f32", "bf16"), ("bf16", "f32"))]
+    rows, at, to = [], 0, 0
+    for i, (s, d, r, n) in enumerate(jobs):
+        off = es[s] * (i % 3) if r is None else 64 + 16 * (i % 2)
+        at, to = (at + 255) // 256 * 256, (to + 255) // 256 * 256 + 16 * (i % 5)
+        pitch = 0 if r is None else -(-n * es[s] // 16) * 16 + 128  # source bytes between rows
+        rows.append((at + off, to, pitch))
+        at += off + (n * es[s] if r is None else pitch * r)
+        to += n * (r or 1) * es[d]
+    blob = rng.integers(0, 256, -(-at // 256) * 256, dtype=np.uint8)
+    dev = torch.from_numpy(blob).cuda()
+    out = torch.full((to + 256,), 0xA5, dtype=torch.uint8, device="cuda")
+    want, sums = np.full(to + 256, 0xA5, np.uint8), []
+    for (s, d, r, n), (a, t, pitch) in zip(jobs, rows):
+        cut = blob[a:a + n * es[s]] if r is None else np.stack(
+            [blob[a + k * pitch:a + k * pitch + n * es[s]] for k in range(r)])
+        bits = np.ascontiguousarray(cut).reshape(-1).view(UINT[es[s]])
+        y = bits if s == d else oracle.convert(s, d, bits)
+        want[t:t + y.nbytes] = y.view(np.uint8)
+        sums.append(y.astype(np.uint64).sum(dtype=np.uint64))
+    shapes = [(n,) if r is None else (r, n) for _, _, r, n in jobs]
+    ents = cfa.make_entries(dtype=[j[0] for j in jobs], shape=shapes, offset=[x[0] for x in rows],
+                            dst=list(range(len(jobs))), cast=[j[0] != j[1] for j in jobs],
+                            src_row_stride=[x[2] // es[j[0]] for x, j in zip(rows, jobs)])
+    dsts = [(out.data_ptr() + x[1], j[1], s) for x, j, s in zip(rows, jobs, shapes)]
+    slot = torch.empty(chunk, dtype=torch.uint8, device="cuda")
+    with cfa.Plan(ents, dsts, blob.nbytes, chunk_bytes=chunk, slab_bytes=slab_kib << 10,
+                  dev_slots=0, host_slots=0) as plan:
+        plan.load_async(cfa.Source.device(dev.data_ptr()))
+        for _ in range(2):
+            out.fill_(0xA5)
+            plan.reset_checksums()
+            for k in range(plan.info()["n_chunks"]):
+                part = dev[k * chunk:(k + 1) * chunk]
+                slot[:part.numel()].copy_(part).bitwise_xor_(0xFF).bitwise_xor_(0xFF)
+                plan.unpack_chunks_async(k, k + 1, slot.data_ptr())
+            torch.cuda.synchronize()
+            bad = np.nonzero(out.cpu().numpy() != want)[0]
+            assert bad.size == 0, [j for j, x in zip(jobs, rows) if x[1] <= bad[0]][-1]
+            assert np.array_equal(plan.checksums(), np.array(sums))
 
 
 @pytest.mark.parametrize("kind", ["aligned", "phases", "tiny"])
@@ -275,26 +339,30 @@ def test_chunks_in_a_cuda_graph_behind_other_work(kind, before):
         del graph
 
 
-@pytest.mark.parametrize("row_bytes", [16, 1008, 1024, 1040, 7168, 32768, 32784, 300_000])
+@pytest.mark.parametrize("row_bytes", [16, 1008, 1024, 1040, 4080, 4096, 4112, 7168, 8176, 8192,
+                                       8208, 32768, 32784, 300_000])
 def test_column_slices_by_row_length(row_bytes):
-    """Rows below, at and above the shortest that go to the TMA kernel, the stage and a slab, at
-    column offsets on and off the 16-byte grid, from device memory and (in place) pinned memory."""
+    """Rows below, at and above the shortest that go to the TMA kernel (4096), the shortest that
+    are cut into segments off it (8192), the stage and a slab, at column offsets on and off the
+    16-byte grid and destinations at several offsets within 128 bytes, from device memory and (in
+    place) pinned memory."""
     rows, lead = 37, 6
-    cases = [(d, off) for d in ES for off in (0, 16, 16 + ES[d])]
+    cases = [(d, off, to) for d in ES for off, to in ((0, 0), (16, 16), (16 + ES[d], 0),
+                                                      (16, 112), (0, 48 + ES[d]), (ES[d], 120))]
     entries, outs, want = [], [], []
     g = torch.Generator(device="cuda").manual_seed(9)
     pitch = row_bytes + 64
     blob = torch.randint(0, 256, (rows * pitch + 256,), dtype=torch.uint8, device="cuda",
                          generator=g)
     grid = blob[:rows * pitch].view(rows, pitch)
-    for d, off in cases:
+    for d, off, _ in cases:
         entries.append((d, (rows, row_bytes // ES[d]), off, pitch // ES[d]))
         outs.append(torch.zeros(rows * row_bytes + 256 * lead, dtype=torch.uint8, device="cuda"))
         want.append(grid[:, off:off + row_bytes].contiguous().view(-1))
     ents = cfa.make_entries(dtype=[e[0] for e in entries], shape=[e[1] for e in entries],
                             offset=[e[2] for e in entries], dst=list(range(len(entries))),
                             src_row_stride=[e[3] for e in entries])
-    dsts = [(o.data_ptr(), e[0], e[1]) for o, e in zip(outs, entries)]
+    dsts = [(o.data_ptr() + q[2], e[0], e[1]) for o, e, q in zip(outs, entries, cases)]
     host = blob.cpu().pin_memory()
     with cfa.Plan(ents, dsts, blob.numel(), dev_slots=2, host_slots=0,
                   chunk_bytes=1 << 20) as plan:
@@ -306,9 +374,10 @@ def test_column_slices_by_row_length(row_bytes):
             plan.wait_layer()
             ck = plan.checksums()
             for i, (o, w) in enumerate(zip(outs, want)):
-                assert torch.equal(o[:w.numel()], w), (i, cases[i])
-                assert not o[w.numel():].any()
-                u = {1: np.uint8, 2: np.uint16, 4: np.uint32, 8: np.uint64}[ES[cases[i][0]]]
+                to = cases[i][2]
+                assert torch.equal(o[to:to + w.numel()], w), (i, cases[i])
+                assert not o[:to].any() and not o[to + w.numel():].any()
+                u = UINT[ES[cases[i][0]]]
                 total = w.cpu().numpy().view(u).astype(np.uint64).sum(dtype=np.uint64)
                 assert int(ck[i]) == int(total)
 
