@@ -160,7 +160,8 @@ def recorded_traffic(workload):
 def kernel_names(st, types=""):
     """The unpack kernels one load of a plan with these stats and element types (path_types)
     launches: a whole load of up to 32 GiB of aligned copies of one type with few tiny pieces takes
-    the vector kernel alone."""
+    the vector kernel alone (plain_class in cfa_runtime.cu).  n_strided counts the column slices of
+    both kernels that take them."""
     out = []
     if (st["n_bulk"] and not st["n_slabs"] and not st["n_strided"] and
             st["n_tiny"] <= st["n_bulk"] // 8 and types in ("u16", "u32", "u64") and
@@ -175,7 +176,8 @@ def kernel_names(st, types=""):
     elif st["n_tiny"]:
         out.append("cfa_tiny_kernel (tiny pieces)")
     if st["n_strided"]:
-        out.append("cfa_strided_kernel (column slices)")
+        out.append("column slices: cfa_bulk_kernel for rows of 4 KiB and more on the 16-byte grid, "
+                   "else cfa_strided_kernel")
     return " + ".join(out)
 
 

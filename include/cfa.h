@@ -161,8 +161,10 @@ typedef struct cfa_dst {
 #define CFA_OPT_BULK            0x8u  /* copy cast-free slabs whose source, destination and
                                          length are multiples of 16 bytes with the TMA bulk-copy
                                          kernel; without it every slab takes the 16-byte vector
-                                         kernel.  Set by cfa_plan_opts_default: the bulk kernel
-                                         is 1-4 % faster on GB300 */
+                                         kernel.  Set by cfa_plan_opts_default.  A whole load from
+                                         device memory that is aligned copies of one 2-, 4- or
+                                         8-byte type with few tiny pieces, up to 32 GiB, takes the
+                                         vector kernel all the same */
 #define CFA_OPT_NO_MERGE        0x10u /* DEVICE sources: one launch per chunk instead of one
                                          launch per contiguous run of chunks */
 #define CFA_OPT_STAGE_SLICES    0x20u /* PINNED sources: copy column slices through the device
@@ -202,8 +204,10 @@ typedef struct cfa_plan_opts {
     uint32_t slab_bytes;      /* destination bytes per block-level work item, a multiple of 4096
                                  in [4096, 64 MiB], or 0 (the default): chosen by the plan for
                                  about 4096 items per load, a power of two in [32 KiB, 256 KiB]
-                                 (256 KiB from 1 GiB of destinations up), which launches may
-                                 cut further */
+                                 (256 KiB from 1 GiB of destinations up).  Launches cut items
+                                 further, down to 32 KiB: those of the plan's choice always,
+                                 those of the caller's size where a launch covers only some of
+                                 the chunks */
     uint32_t tiny_bytes;      /* pieces with fewer destination bytes become warp-level items of
                                  at most 512 destination bytes, each copied by four or eight
                                  lanes of a warp; default 8192 */
@@ -421,7 +425,9 @@ cfa_status cfa_plan_get_pieces(const cfa_plan *plan, cfa_piece *out, size_t cap,
 /*
  * Unpacks chunks [chunk_begin, chunk_end) that the caller has already placed in device memory:
  * blob byte o of those chunks is at chunk_src + (o - chunk_begin * chunk_bytes).  chunk_src is a
- * device pointer, 256-byte aligned.  One kernel launch on `stream`; checksums accumulate into
+ * device pointer, 256-byte aligned.  One launch or a few on `stream`, after all work enqueued on
+ * it before; what is enqueued on it afterwards follows them (a kernel with the programmatic
+ * serialization attribute starts when their blocks have ended).  Checksums accumulate into
  * the plan's checksum buffer (cleared by cfa_load_async, or by cfa_reset_checksums).  This is the
  * bare "InGPU -> Loaded" transition of section 4.2 for callers that manage their own staging.
  */
@@ -457,7 +463,8 @@ cfa_status cfa_unpack_chunks_async(cfa_plan *plan, uint32_t chunk_begin, uint32_
  *   blob_dev, blob_bytes   the blob in device memory (256-byte aligned); must stay valid and
  *                          unchanged until the unpack has run on `stream`
  *   cksum_dev              device array of n_entries uint64 receiving the checksums
- *                          (cleared by the call), or NULL for none
+ *                          (cleared by the call; 8-byte aligned if any entry has a checksum),
+ *                          or NULL for none
  *   status_dev             optional device int (4-byte aligned) receiving the kernels' own
  *                          status word: the call sets it to 0 on `stream`, and a kernel that
  *                          rejects a work item (its source outside the blob, a misaligned

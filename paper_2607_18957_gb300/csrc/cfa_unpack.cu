@@ -4,7 +4,7 @@
  * carries).  One launch handles every work item of one chunk, or of a run of chunks that sit
  * contiguously in device memory.
  *
- * The work is pure data movement plus integer arithmetic, so it is bound by HBM bandwidth:
+ * The work is data movement with little arithmetic, so it is bound by HBM bandwidth:
  * every source byte is read once from the staging buffer and every destination byte written
  * once.  Design points:
  *   - block-per-slab: a slab (tens of KiB of one piece) is copied by a whole CTA with 16-byte
@@ -16,7 +16,9 @@
  *   - source and destination offsets that differ modulo 16 are realigned in registers (two
  *     aligned loads and a funnel shift per 16-byte store), so stores stay 16 bytes wide;
  *   - dtype conversions (fp32 -> bf16 / fp16, fp16 -> bf16 with round-to-nearest-even;
- *     bf16 / fp16 -> fp32 exactly) work on bit patterns with integer operations;
+ *     bf16 / fp16 -> fp32 exactly) take eight elements at a time: fp32 -> bf16 and bf16 -> fp32 as
+ *     integer operations on the bit patterns, the others with the hardware's conversion
+ *     instructions and NaN results put right; a run's ends as integer operations throughout;
  *   - checksums are sums modulo 2^64 of the destination element bit patterns, reduced inside the
  *     CTA or warp and added with one 64-bit atomic per (CTA, run of same-tensor slabs) or per
  *     tiny piece; integer addition is associative, so the result does not depend on the order.
@@ -974,6 +976,9 @@ __device__ __forceinline__ TinyItem tiny_fetch(const UnpackArgs &a, uint32_t gro
 
 /* A lane's share of an item's checksum: 8- and 16-bit elements add up to less than 2^32 over an
  * item (CFA_TINY_SEG_BYTES), so one dot-product instruction with ones per word and 32 bits do. */
+static_assert(CFA_TINY_SEG_BYTES * 0xFFull < (1ull << 32) &&
+                  CFA_TINY_SEG_BYTES / 2 * 0xFFFFull < (1ull << 32),
+              "an item's 8- or 16-bit elements add up in 32 bits");
 template <int ES> struct TinySum {
     typedef uint64_t T;
     static __device__ __forceinline__ void add(T &acc, const uint4 &v) { acc += vsum<ES>(v); }

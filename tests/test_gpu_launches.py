@@ -1,7 +1,8 @@
-"""How launches are cut and chained: block-level items cut into parts where a launch has few of
-them (sizes around the parts, sources and destinations at odd phases), one TMA launch over several
-element sizes, and chunks unpacked one after the other from a staging slot that the caller
-overwrites in between, on a stream and in a CUDA graph.  Checked against slices of the blob."""
+"""How launches are cut and chained: block-level items cut into parts (sizes around the parts,
+sources and destinations at odd phases), one TMA launch over several element sizes, the no-alloc
+entry point's upload, and chunks unpacked one after the other from a staging slot that the caller,
+or the kernel before, overwrites in between, on a stream and in a CUDA graph.  Checked against
+slices of the blob, and against the oracle where elements are converted."""
 import ctypes
 
 import numpy as np
