@@ -304,13 +304,13 @@ __global__ void __launch_bounds__(kThreads) cfa_bulk_kernel(const BulkArgs a)
     RawItem cur{}, nxt{};
     if (threadIdx.x == 0) {
         if (blockIdx.x < a.n_items) cur = bulk_fetch<ROWS>(a, blockIdx.x);
-        if (blockIdx.x + gridDim.x < a.n_items) nxt = bulk_fetch<ROWS>(a, blockIdx.x + gridDim.x);
-    }
-    if (threadIdx.x == 0 && (a.ctl.flags & CFA_LAUNCH_WAIT_FIRST)) {
         /* The source is not to be read yet (the kernel before may still be writing it), but asking
          * for it in L2, where every write arrives, is harmless, and fills the time in which the
-         * kernel before ends. */
-        if (blockIdx.x < a.n_items) bulk_ask<ROWS>(a, blockIdx.x, cur);
+         * kernel before ends; first of all, so that it gets the most of that time (3.4 GB in 64 MiB
+         * chunks 1231 us, 1242 behind the second descriptor's fetch). */
+        if ((a.ctl.flags & CFA_LAUNCH_WAIT_FIRST) && blockIdx.x < a.n_items)
+            bulk_ask<ROWS>(a, blockIdx.x, cur);
+        if (blockIdx.x + gridDim.x < a.n_items) nxt = bulk_fetch<ROWS>(a, blockIdx.x + gridDim.x);
     }
     launch_begin(a.ctl);
     /* what the kernel before wrote is read by bulk copies (the async proxy) from here on */
